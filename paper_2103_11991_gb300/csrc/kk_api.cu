@@ -2205,7 +2205,7 @@ kk_status batched_packed_symbolic(kk_spgemm_handle h, int32_t count, const kk_cs
                                cudaMemcpyHostToDevice, s), "upload");
   }
   // pageable sources above: staged before return, so base may go out of scope
-  KK_CUDA(h, launch_b_pack(s, h->num_sms, count, dd, h->d_pbase.as<long long>(), false,
+  KK_CUDA(h, launch_b_pack(s, count, dd, h->d_pbase.as<long long>(), false,
                            h->d_pa_rp.as<int32_t>(), h->d_pa_ci.as<int32_t>(), h->d_pa_v.as<double>(),
                            h->d_pb_rp.as<int32_t>(), h->d_pb_ci.as<int32_t>(), h->d_pb_v.as<double>(),
                            RA, NA, RB, NB), "pack");
@@ -2246,7 +2246,7 @@ kk_status batched_packed_numeric(kk_spgemm_handle h, int32_t count, bool moved, 
   PairDesc* hd2 = static_cast<PairDesc*>(h->h_bdesc2);
   if (count > 0)
     KK_CUDA(h, cudaMemcpyAsync(dd, hd2, sizeof(PairDesc) * count, cudaMemcpyHostToDevice, s), "upload");
-  KK_CUDA(h, launch_b_pack(s, h->num_sms, count, dd, h->d_pbase.as<long long>(), !moved,
+  KK_CUDA(h, launch_b_pack(s, count, dd, h->d_pbase.as<long long>(), !moved,
                            h->d_pa_rp.as<int32_t>(), h->d_pa_ci.as<int32_t>(), h->d_pa_v.as<double>(),
                            h->d_pb_rp.as<int32_t>(), h->d_pb_ci.as<int32_t>(), h->d_pb_v.as<double>(),
                            h->p_RA, h->p_NA, h->p_RB, h->p_NB), "pack");

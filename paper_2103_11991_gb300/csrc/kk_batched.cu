@@ -562,43 +562,74 @@ cudaError_t launch_b_offsets(cudaStream_t s, int32_t count, const PairDesc* d, l
 namespace kk {
 namespace {
 
-// One CTA per pair: A_k's rows go to packed rows [R_k, R_k + A_k.m) with
-// columns shifted to B_k's packed rows; B_k's rows go to [RB_k, RB_k + B_k.m)
-// with their columns unchanged (C_k's columns stay local to the pair).
-// vals_only: copy values only (numeric calls on the same structure).
-__global__ void k_b_pack(int32_t count, const PairDesc* __restrict__ d,
-                         const long long* __restrict__ base, int32_t vals_only, int32_t* pa_rp,
-                         int32_t* pa_ci, double* pa_v, int32_t* pb_rp, int32_t* pb_ci, double* pb_v,
-                         long long RA, long long NA, long long RB, long long NB) {
-  for (int k = blockIdx.x; k < count; k += gridDim.x) {
-    const CsrView A = d[k].A, B = d[k].B;
-    // base[4k ..]: A rows, A entries, B rows, B entries before pair k
-    const long long ra = base[4 * k], na = base[4 * k + 1], rb = base[4 * k + 2], nb = base[4 * k + 3];
-    if (!vals_only) {
-      for (int r = threadIdx.x; r < A.m; r += blockDim.x) pa_rp[ra + r] = (int32_t)(na + A.rowptr[r]);
-      for (int q = threadIdx.x; q < A.nnz; q += blockDim.x) pa_ci[na + q] = (int32_t)(rb + A.colind[q]);
-      for (int r = threadIdx.x; r < B.m; r += blockDim.x) pb_rp[rb + r] = (int32_t)(nb + B.rowptr[r]);
-      for (int q = threadIdx.x; q < B.nnz; q += blockDim.x) pb_ci[nb + q] = B.colind[q];
-    }
-    for (int q = threadIdx.x; q < A.nnz; q += blockDim.x) pa_v[na + q] = A.vals ? A.vals[q] : 0.0;
-    for (int q = threadIdx.x; q < B.nnz; q += blockDim.x) pb_v[nb + q] = B.vals ? B.vals[q] : 0.0;
-  }
-  if (!vals_only && blockIdx.x == 0 && threadIdx.x == 0) {
+// A_k's rows go to packed rows [R_k, R_k + A_k.m) with columns shifted to B_k's
+// packed rows; B_k's rows go to [RB_k, RB_k + B_k.m) with their columns
+// unchanged (C_k's columns stay local to the pair).  vals_only: copy values
+// only (numeric calls on the same structure).
+// A copy, bound by HBM.  blockIdx.y picks A's rows, A's entries, B's rows or B's
+// entries of the whole batch; a CTA copies kPackChunk consecutive packed
+// elements, whichever pairs they belong to, so the uneven sizes of the pairs
+// do not matter (with a CTA per pair the largest pairs ran alone at the end: 6.4
+// ms symbolic and 3.2 ms numeric for 256 pairs of 100 to 50,000 rows).
+constexpr int kPackThreads = 256;
+constexpr int kPackChunk = 4096;
+__global__ void __launch_bounds__(kPackThreads)
+k_b_pack(int32_t count, const PairDesc* __restrict__ d, const long long* __restrict__ base, int32_t vals_only,
+         int32_t* __restrict__ pa_rp, int32_t* __restrict__ pa_ci, double* __restrict__ pa_v,
+         int32_t* __restrict__ pb_rp, int32_t* __restrict__ pb_ci, double* __restrict__ pb_v, long long RA,
+         long long NA, long long RB, long long NB) {
+  const int part = blockIdx.y;
+  const long long n = part == 0 ? RA : part == 1 ? NA : part == 2 ? RB : NB;
+  long long pos = (long long)blockIdx.x * kPackChunk;
+  if (!vals_only && part == 0 && blockIdx.x == 0 && threadIdx.x == 0) {
     pa_rp[RA] = (int32_t)NA;
     pb_rp[RB] = (int32_t)NB;
+  }
+  if (pos >= n || (vals_only && !(part & 1))) return;
+  const long long end = min(n, pos + kPackChunk);
+  // pair of the chunk's first element: the last k with base[4k + part] <= pos
+  int lo = 0, hi = count;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (base[4 * mid + part] <= pos) lo = mid;
+    else hi = mid;
+  }
+  for (int k = lo; pos < end; ++k) {
+    // base[4k ..]: A rows, A entries, B rows, B entries before pair k
+    const long long first = base[4 * k + part];
+    const long long stop = min(end, k + 1 < count ? base[4 * (k + 1) + part] : n);
+    if (stop <= pos) continue;
+    const CsrView M = part < 2 ? d[k].A : d[k].B;
+    if (part & 1) {
+      const int shift = part == 1 ? (int)base[4 * k + 2] : 0;  // A's columns are B_k's rows
+      int32_t* ci = part == 1 ? pa_ci : pb_ci;
+      double* v = part == 1 ? pa_v : pb_v;
+#pragma unroll 4
+      for (long long e = pos + threadIdx.x; e < stop; e += kPackThreads) {
+        if (!vals_only) ci[e] = M.colind[e - first] + shift;
+        v[e] = M.vals ? M.vals[e - first] : 0.0;
+      }
+    } else {
+      const int shift = (int)base[4 * k + part + 1];
+      int32_t* rp = part == 0 ? pa_rp : pb_rp;
+#pragma unroll 4
+      for (long long e = pos + threadIdx.x; e < stop; e += kPackThreads) rp[e] = M.rowptr[e - first] + shift;
+    }
+    pos = stop;
   }
 }
 
 }  // namespace
 
-cudaError_t launch_b_pack(cudaStream_t s, int num_sms, int32_t count, const PairDesc* d,
+cudaError_t launch_b_pack(cudaStream_t s, int32_t count, const PairDesc* d,
                           const long long* base, bool vals_only, int32_t* pa_rp, int32_t* pa_ci,
                           double* pa_v, int32_t* pb_rp, int32_t* pb_ci, double* pb_v, long long RA,
                           long long NA, long long RB, long long NB) {
   if (count <= 0) return cudaSuccess;
-  const int grid = count < num_sms * 8 ? count : num_sms * 8;
-  k_b_pack<<<grid, 256, 0, s>>>(count, d, base, vals_only ? 1 : 0, pa_rp, pa_ci, pa_v, pb_rp, pb_ci,
-                                pb_v, RA, NA, RB, NB);
+  const long long most = max(max(RA, NA), max(RB, NB));
+  const dim3 grid((unsigned)((most + kPackChunk - 1) / kPackChunk > 0 ? (most + kPackChunk - 1) / kPackChunk : 1), 4);
+  k_b_pack<<<grid, kPackThreads, 0, s>>>(count, d, base, vals_only ? 1 : 0, pa_rp, pa_ci, pa_v, pb_rp, pb_ci, pb_v,
+                                         RA, NA, RB, NB);
   return cudaGetLastError();
 }
 
