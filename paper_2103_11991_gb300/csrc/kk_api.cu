@@ -126,41 +126,44 @@ struct DevBuf {
   }
 };
 
-constexpr int kMaxBins = 32;
+constexpr int kMaxBins = 48;
 constexpr uint8_t kSkipBin = 0xFF;
 
 // Device-side classifier: first bin whose hi bound covers q and whose mode
 // (0 = vector only, 1 = flattened only, 2 = either) admits the row's mode.
-// Window bins (window tier) are tried first: a row qualifies for window class
-// w when B's rows are sorted, its span fits kWindowBits[w], the window is not
-// too wide for its flop count, and (numeric) its nnz fits the dense value slots.
+// The thread bin (first) comes before everything, then the window bins: a row
+// qualifies for one when its span fits win_bits, the window is not too wide for
+// its flop count and q lies in the bin's range.  Kept bins (numeric) also need
+// the structure kept by the symbolic phase; the others take unsorted B too
+// (any_order), over all of its columns.
 struct BinTable {
   int32_t nb;
   long long hi[kMaxBins];
   int32_t mode[kMaxBins];  // 0 vector, 1 flattened, 2 either, 3 thread tier (flop capped too)
   long long thread_flop;
+  int32_t cols;  // columns of B
   int32_t nwin;
   int32_t win_bits[kMaxWindowBins];
   int32_t win_bin[kMaxWindowBins];
+  int32_t win_kept[kMaxWindowBins];     // 1: rows with kept structure only
+  int32_t win_any_order[kMaxWindowBins];
   long long win_q[kMaxWindowBins];      // largest binning quantity of each window bin
-  long long win_qlo[kMaxWindowBins];    // binning quantity must exceed this
   long long win_ratio[kMaxWindowBins];  // window W only when W <= ratio * flop
 };
 
 __device__ __forceinline__ uint8_t classify(const BinTable& t, long long q, int flat, int span,
-                                            long long flop, int sorted) {
+                                            long long flop, int sorted, bool kept) {
   if (q <= 0) return kSkipBin;
-  if (sorted && span > 0) {
+  if (t.mode[0] == 3 && q <= t.hi[0] && flop <= t.thread_flop) return 0;
+  const int sp = sorted ? span : t.cols;
+  if (sp > 0) {
     for (int w = 0; w < t.nwin; ++w)
-      if (q > t.win_qlo[w] && q <= t.win_q[w] && span <= t.win_bits[w] &&
-          (long long)t.win_bits[w] <= t.win_ratio[w] * flop)
+      if (q <= t.win_q[w] && sp <= t.win_bits[w] && (sorted || t.win_any_order[w]) &&
+          (!t.win_kept[w] || kept) && (long long)t.win_bits[w] <= t.win_ratio[w] * flop)
         return (uint8_t)t.win_bin[w];
   }
   for (int b = 0; b < t.nb; ++b) {
-    if (t.mode[b] == 3) {
-      if (q <= t.hi[b] && flop <= t.thread_flop) return (uint8_t)b;
-      continue;
-    }
+    if (t.mode[b] == 3) continue;
     if (q <= t.hi[b] && (t.mode[b] == 2 || t.mode[b] == flat)) return (uint8_t)b;
   }
   return (uint8_t)(t.nb - 1);
@@ -264,7 +267,7 @@ k_analyze_a(CsrView A, const int32_t* __restrict__ brp,
       row_lo[r] = hi >= lo ? lo : 0;
       row_span[r] = sp;
       const int flat = (f < (long long)vec_min_len * (pe - pa)) ? 1 : 0;
-      bin[r] = classify(tab, f, flat, sp, f, sorted);
+      bin[r] = classify(tab, f, flat, sp, f, sorted, false);
       if (STATS) stat[r] = make_int2(mx, pe > pa ? mn : 0);
       acc += (unsigned long long)f;
     }
@@ -455,8 +458,8 @@ __global__ void __launch_bounds__(kScanBlock)
 k_scan_final(int32_t m, const int32_t* __restrict__ cnt, const long long* __restrict__ blk_off,
              const long long* __restrict__ flop, const int32_t* __restrict__ arp,
              const int32_t* __restrict__ row_span, const int32_t* __restrict__ b_sorted,
-             int32_t vec_min_len, BinTable ntab, int64_t* __restrict__ rowptr,
-             uint8_t* __restrict__ nbin) {
+             int32_t vec_min_len, BinTable ntab, const int32_t* __restrict__ kept_n,
+             int64_t* __restrict__ rowptr, uint8_t* __restrict__ nbin) {
   const int sorted = *b_sorted;
   __shared__ long long scratch[33];
   const long long base = (long long)blockIdx.x * kScanRows + (long long)threadIdx.x * kScanPer;
@@ -475,7 +478,7 @@ k_scan_final(int32_t m, const int32_t* __restrict__ cnt, const long long* __rest
       if (nbin) {
         const int nza = arp[r + 1] - arp[r];
         const int flat = (flop[r] < (long long)vec_min_len * nza) ? 1 : 0;
-        nbin[r] = classify(ntab, v[t], flat, row_span[r], flop[r], sorted);
+        nbin[r] = classify(ntab, v[t], flat, row_span[r], flop[r], sorted, kept_n != nullptr && kept_n[r] >= 0);
       }
       if (r == m - 1) rowptr[m] = run + v[t];
     }
@@ -825,7 +828,6 @@ struct kk_spgemm_handle_s {
   DevBuf d_cw;         // uint16[m * kCacheWords]
   DevBuf d_cm;         // uint32[m * kCacheWords]
   DevBuf d_cn;         // int32[m]
-  DevBuf d_left;       // int32[1 + m]: count, then rows left to the window kernel
   bool cache_valid = false;
   // wide-tier bit vectors kept by the symbolic phase
   DevBuf d_wbits, d_wslot, d_wnext;
@@ -977,36 +979,33 @@ void build_bins(const kk_spgemm_options& o, bool numeric, std::vector<BinSpec>& 
     for (int w = 0; w < kNumWindowClasses; ++w)
       out.push_back(BinSpec{kTierWindow, 128, kWindowBits[w], 0, 0,
                             numeric ? kWindowMaxNnz : (long long)9e18});
-    // numeric rows of up to kWindowMaxNnzWide columns: large value arrays
+    // numeric rows without kept structure: by slots, then by window
     if (numeric)
-      for (const int32_t vmax : {kWindowMidNnz, kWindowMaxNnzWide})
-        for (int w = 0; w < kNumWideWindowClasses; ++w)
-          out.push_back(BinSpec{kTierWindow, 128, kWideWindowBits[w], 0, 0, vmax});
+      for (const int32_t vmax : kRankNnz)
+        for (const int32_t bits : kRankBits) out.push_back(BinSpec{kTierRank, 64, bits, 0, 0, vmax});
   }
 }
 
-BinTable to_table(const std::vector<BinSpec>& bins) {
+BinTable to_table(const std::vector<BinSpec>& bins, bool numeric, int32_t cols) {
   BinTable t{};
   t.nb = 0;
   t.nwin = 0;
+  t.cols = cols;
   for (size_t b = 0; b < bins.size(); ++b) {
-    if (bins[b].tier == kTierWindow) {
+    const bool rank = bins[b].tier == kTierRank;
+    if (rank || bins[b].tier == kTierWindow) {
       t.win_bits[t.nwin] = bins[b].slots;
       t.win_bin[t.nwin] = (int32_t)b;
       t.win_q[t.nwin] = bins[b].hi;
-      // large-value numeric bins take only rows of more than kWindowMaxNnz
-      // columns (sparser rows than the ratio of the others admits: their cost
-      // follows the touched words rather than W); rows of fewer columns that
-      // miss the other window bins go to the hash tiers
-      const bool large = bins[b].hi > kWindowMaxNnz && bins[b].hi <= kWindowMaxNnzWide;
-      t.win_ratio[t.nwin] = large ? kWindowFlopRatioNum : kWindowFlopRatio;
-      t.win_qlo[t.nwin] = large ? kWindowMaxNnz : 0;
+      t.win_kept[t.nwin] = numeric && !rank ? 1 : 0;
+      t.win_any_order[t.nwin] = rank ? 1 : 0;
+      t.win_ratio[t.nwin] = rank ? kRankFlopRatio : kWindowFlopRatio;
       ++t.nwin;
     } else {
       t.nb = (int32_t)b + 1;
     }
   }
-  t.thread_flop = kThreadNumMaxFlop;
+  t.thread_flop = numeric ? kThreadNumMaxFlop : kThreadSymMax;
   for (int b = 0; b < t.nb; ++b) {
     t.hi[b] = bins[b].hi;
     t.mode[b] = bins[b].tier == kTierThread ? 3 : bins[b].tier == kTierTeam ? bins[b].flat : 2;
@@ -1170,20 +1169,19 @@ void keep_for_numeric(kk_spgemm_handle h, const CsrView& av, const CsrView& bv) 
   }
 }
 
-// The kept structure, if it belongs to these index arrays, and the scratch
-// its numeric launches need.  Unless options.debug_checks asks for a check of
+// Kept word counts of the rows of this symbolic call (-1: no kept structure),
+// null when it keeps none.
+const int32_t* kept_counts(kk_spgemm_handle h) { return h->cache_valid ? h->d_cn.as<int32_t>() : nullptr; }
+
+// The kept structure, if it belongs to these index arrays.  Unless options.debug_checks asks for a check of
 // every product, the arrays' fingerprint is taken again and ctx->fingerprint
 // points the numeric kernels at both fingerprints.
-kk_status cache_view(kk_spgemm_handle h, const CsrView& av, const CsrView& bv, WinCacheView* view,
-                     WinScratch* scratch, LaunchCtx* ctx) {
+kk_status cache_view(kk_spgemm_handle h, const CsrView& av, const CsrView& bv, WinCacheView* view, LaunchCtx* ctx) {
   *view = WinCacheView{nullptr, nullptr, nullptr};
-  *scratch = WinScratch{nullptr, nullptr};
   if (!h->cache_valid || h->cache_key[0] != av.rowptr || h->cache_key[1] != av.colind ||
       h->cache_key[2] != bv.rowptr || h->cache_key[3] != bv.colind)
     return KK_OK;
-  KK_CUDA(h, h->d_left.ensure(sizeof(int32_t) * ((size_t)av.m + 1)), "alloc window scratch");
   *view = WinCacheView{h->d_cw.as<uint16_t>(), h->d_cm.as<uint32_t>(), h->d_cn.as<int32_t>()};
-  *scratch = WinScratch{h->d_left.as<int32_t>() + 1, h->d_left.as<int32_t>()};
   if (!h->opt.debug_checks) {
     Misc* dm = h->d_misc.as<Misc>();
     kk_status st = fingerprint(h, av, bv, &dm->fp[1]);
@@ -1191,6 +1189,27 @@ kk_status cache_view(kk_spgemm_handle h, const CsrView& av, const CsrView& bv, W
     ctx->fingerprint = dm->fp;
   }
   return KK_OK;
+}
+
+// One numeric bin.  Rows binned for their kept structure go to the rank kernel
+// when it is not the one of these arrays.
+cudaError_t launch_numeric_rows(kk_spgemm_handle h, const LaunchCtx& ctx, const BinSpec& bin, const CsrView& av,
+                                const CsrView& bv, const BComp& bcomp, const WinCacheView& kept,
+                                const float2* bsplit, int32_t arith, const int64_t* c_rowptr, const int32_t* rows,
+                                int32_t cnt, int32_t* c_colind, double* c_vals) {
+  const int32_t* range_bad = &h->d_misc.as<Misc>()->range_bad;
+  if (bin.tier == kTierWindow && kept.n) {
+    timer_begin(ctx.timer, ctx.stream, "num_kept");
+    const cudaError_t e = launch_num_kept(ctx, av, bv, kept, bsplit, range_bad, ctx.kept_f64 ? kArithF64 : arith,
+                                          c_rowptr, rows, cnt, c_colind, c_vals);
+    timer_end(ctx.timer, ctx.stream);
+    return e;
+  }
+  if (bin.tier == kTierWindow || bin.tier == kTierRank)
+    return launch_num_rank(ctx, bin, av, bv, h->b_sorted, bcomp, bsplit, range_bad, arith, c_rowptr, rows, cnt,
+                           c_colind, c_vals);
+  return launch_numeric_bin(ctx, bin, av, bv, h->b_sorted, bsplit, range_bad, arith, c_rowptr, rows, cnt, c_colind,
+                            c_vals, h->opt.debug_checks);
 }
 
 int grid_for(long long work, int per_block, int cap) {
@@ -1282,7 +1301,7 @@ static void launch_analyze_a(kk_spgemm_handle h, const CsrView& av, const CsrVie
   }
   const int64_t m = av.m;
   k_analyze_a<T, U, STATS><<<grid_for(m * T, 256, h->num_sms * (per_sm > 0 ? per_sm : 1)), 256, 0, s>>>(
-      av, bv.rowptr, bv.colind, bv.m, &dm->sorted, to_table(h->sym_bins), h->opt.team_vec_min_len,
+      av, bv.rowptr, bv.colind, bv.m, &dm->sorted, to_table(h->sym_bins, false, bv.n), h->opt.team_vec_min_len,
       h->d_flop.as<long long>(), bin, h->d_rowlo.as<int32_t>(), h->d_span.as<int32_t>(), stat,
       &dm->total_flop, &dm->status);
 }
@@ -1538,8 +1557,8 @@ kk_status kk_spgemm_symbolic(kk_spgemm_handle h, const kk_csr* A, const kk_csr* 
     k_scan_top<<<1, 1024, 0, s>>>(nblk_scan, h->d_scan.as<long long>(), &dm->grand);
     k_scan_final<<<nblk_scan, kScanBlock, 0, s>>>(
         m, h->d_cnt.as<int32_t>(), h->d_scan.as<long long>(), h->d_flop.as<long long>(), av.rowptr,
-        h->d_span.as<int32_t>(), &dm->sorted, h->opt.team_vec_min_len, to_table(h->num_bins),
-        c_rowptr, h->d_nbin.as<uint8_t>());
+        h->d_span.as<int32_t>(), &dm->sorted, h->opt.team_vec_min_len,
+        to_table(h->num_bins, true, bv.n), kept_counts(h), c_rowptr, h->d_nbin.as<uint8_t>());
     timer_end(h->timer, s);
     KK_CUDA(h, cudaGetLastError(), "scan launch");
     if ((st = run_binning(h, m, h->d_nbin.as<uint8_t>(), nbn, h->d_nrows.as<int32_t>(), num_start)) != KK_OK)
@@ -1641,7 +1660,7 @@ static kk_status numeric_impl(kk_spgemm_handle h, const kk_csr* A, const kk_csr*
   h->stats[9] = (arith == kArithDF32 && bv.nnz > 0) ? 1 : 0;
   bool any_win = false;
   for (int b = 0; b < nbn; ++b)
-    if (h->num_bins[b].tier == kTierWindow && h->num_start[b + 1] > h->num_start[b]) any_win = true;
+    if (stat_tier(h->num_bins[b].tier) == kTierWindow && h->num_start[b + 1] > h->num_start[b]) any_win = true;
   BComp bcomp{nullptr, nullptr};
   if (any_win) {
     int built = 0;
@@ -1649,8 +1668,7 @@ static kk_status numeric_impl(kk_spgemm_handle h, const kk_csr* A, const kk_csr*
     h->stats[9] += built;
   }
   WinCacheView wview;
-  WinScratch wscratch;
-  if ((st = cache_view(h, av, bv, &wview, &wscratch, &ctx)) != KK_OK) return st;
+  if ((st = cache_view(h, av, bv, &wview, &ctx)) != KK_OK) return st;
   for (int b = 0; b < nbn; ++b) {
     const int cnt = h->num_start[b + 1] - h->num_start[b];
     if (cnt <= 0) continue;
@@ -1662,13 +1680,8 @@ static kk_status numeric_impl(kk_spgemm_handle h, const kk_csr* A, const kk_csr*
       if (e != cudaSuccess) return cuda_fail(h, e, "Jacobi launch");
       h->stats[9] += 1;
     }
-    cudaError_t e = h->num_bins[b].tier == kTierWindow
-                        ? launch_numeric_window(ctx, h->num_bins[b], av, bv, bcomp, wview, wscratch, bsplit,
-                                                &dm->range_bad, arith, c_rowptr, rows, cnt, c_colind,
-                                                c_vals)
-                        : launch_numeric_bin(ctx, h->num_bins[b], av, bv, h->b_sorted, bsplit,
-                                             &dm->range_bad, arith, c_rowptr, rows, cnt, c_colind,
-                                             c_vals, h->opt.debug_checks);
+    cudaError_t e = launch_numeric_rows(h, ctx, h->num_bins[b], av, bv, bcomp, wview, bsplit, arith, c_rowptr, rows,
+                                        cnt, c_colind, c_vals);
     if (e != cudaSuccess) return cuda_fail(h, e, "numeric launch");
   }
   return KK_OK;
@@ -1705,7 +1718,7 @@ namespace {
 // Exclusive scan of int32 counts into int64 offsets out[0..m] (out[m] = total,
 // also written to *grand); nbin (nullable) receives numeric bin ids.
 kk_status run_scan(kk_spgemm_handle h, int32_t m, const int32_t* cnt, int64_t* out, long long* grand,
-                   const CsrView& av, uint8_t* nbin) {
+                   const CsrView& av, int32_t cols, uint8_t* nbin) {
   cudaStream_t s = h->stream;
   const int nblk = (int)((m + kScanRows - 1) / kScanRows);
   if (m == 0) return KK_OK;
@@ -1715,7 +1728,8 @@ kk_status run_scan(kk_spgemm_handle h, int32_t m, const int32_t* cnt, int64_t* o
   k_scan_top<<<1, 1024, 0, s>>>(nblk, h->d_scan.as<long long>(), grand);
   k_scan_final<<<nblk, kScanBlock, 0, s>>>(m, cnt, h->d_scan.as<long long>(), h->d_flop.as<long long>(),
                                            av.rowptr, h->d_span.as<int32_t>(), &dm->sorted,
-                                           h->opt.team_vec_min_len, to_table(h->num_bins), out, nbin);
+                                           h->opt.team_vec_min_len, to_table(h->num_bins, true, cols),
+                                           nbin ? kept_counts(h) : nullptr, out, nbin);
   KK_CUDA(h, cudaGetLastError(), "scan launch");
   return KK_OK;
 }
@@ -1758,7 +1772,7 @@ kk_status kk_spadd_symbolic(kk_spgemm_handle h, const kk_csr* A, const kk_csr* B
     timer_end(h->timer, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "SpAdd symbolic launch");
     timer_begin(h->timer, s, "scan");
-    if ((st = run_scan(h, m, h->d_acnt.as<int32_t>(), c_rowptr, &dm->grand, view(A), nullptr)) != KK_OK)
+    if ((st = run_scan(h, m, h->d_acnt.as<int32_t>(), c_rowptr, &dm->grand, view(A), 0, nullptr)) != KK_OK)
       return st;
     timer_end(h->timer, s);
   } else {
@@ -1902,7 +1916,7 @@ kk_status kk_spgemm_learned_symbolic(kk_spgemm_handle h, const kk_csr* A, const 
     timer_end(h->timer, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "learned analyze");
     timer_begin(h->timer, s, "learned_plan");
-    if ((st = run_scan(h, m, h->d_cap.as<int32_t>(), h->d_soff.as<int64_t>(), &dm->grand2, av, nullptr)) != KK_OK)
+    if ((st = run_scan(h, m, h->d_cap.as<int32_t>(), h->d_soff.as<int64_t>(), &dm->grand2, av, 0, nullptr)) != KK_OK)
       return st;
     timer_end(h->timer, s);
     if ((st = run_binning(h, m, h->d_lbin.as<uint8_t>(), nbl, h->d_lrows.as<int32_t>(), l_start)) != KK_OK)
@@ -1999,7 +2013,7 @@ kk_status kk_spgemm_learned_symbolic(kk_spgemm_handle h, const kk_csr* A, const 
     h->stats[14] = heavy;
     h->stats[15] = staging;
     timer_begin(h->timer, s, "scan");
-    if ((st = run_scan(h, m, h->d_cnt.as<int32_t>(), c_rowptr, &dm->grand, av, h->d_nbin.as<uint8_t>())) != KK_OK)
+    if ((st = run_scan(h, m, h->d_cnt.as<int32_t>(), c_rowptr, &dm->grand, av, bv.n, h->d_nbin.as<uint8_t>())) != KK_OK)
       return st;
     timer_end(h->timer, s);
     if ((st = run_binning(h, m, h->d_nbin.as<uint8_t>(), nbn, h->d_nrows.as<int32_t>(), num_start)) != KK_OK)
@@ -2059,24 +2073,20 @@ kk_status kk_spgemm_learned_numeric(kk_spgemm_handle h, const kk_csr* A, const k
   const int nbn = (int)h->num_bins.size();
   bool any_win = false;
   for (int b = 0; b < nbn; ++b)
-    if (h->num_bins[b].tier == kTierWindow && h->lnum_start[b + 1] > h->lnum_start[b]) any_win = true;
+    if (stat_tier(h->num_bins[b].tier) == kTierWindow && h->lnum_start[b + 1] > h->lnum_start[b]) any_win = true;
   BComp bcomp{nullptr, nullptr};
   if (any_win) {
     int built = 0;
     if ((st = ensure_bcomp(h, bv, &bcomp, &built)) != KK_OK) return st;
   }
   WinCacheView wview;
-  WinScratch wscratch;
-  if ((st = cache_view(h, av, bv, &wview, &wscratch, &ctx)) != KK_OK) return st;
+  if ((st = cache_view(h, av, bv, &wview, &ctx)) != KK_OK) return st;
   for (int b = 0; b < nbn; ++b) {
     const int cnt = h->lnum_start[b + 1] - h->lnum_start[b];
     if (cnt <= 0) continue;
     const int32_t* rows = h->d_lrows2.as<int32_t>() + h->lnum_start[b];
-    e = h->num_bins[b].tier == kTierWindow
-            ? launch_numeric_window(ctx, h->num_bins[b], av, bv, bcomp, wview, wscratch, bsplit, &dm->range_bad,
-                                    arith, c_rowptr, rows, cnt, c_colind, c_vals)
-            : launch_numeric_bin(ctx, h->num_bins[b], av, bv, h->b_sorted, bsplit, &dm->range_bad, arith,
-                                 c_rowptr, rows, cnt, c_colind, c_vals, h->opt.debug_checks);
+    e = launch_numeric_rows(h, ctx, h->num_bins[b], av, bv, bcomp, wview, bsplit, arith, c_rowptr, rows, cnt,
+                            c_colind, c_vals);
     if (e != cudaSuccess) return cuda_fail(h, e, "numeric launch");
   }
   return KK_OK;
@@ -2350,7 +2360,7 @@ kk_status kk_spgemm_batched_symbolic(kk_spgemm_handle h, int32_t count, const kk
       KK_CUDA(h, launch_b_symbolic(ctx, dd, h->d_rowpair.as<int32_t>(), h->d_bsrows.as<int32_t>(), sym_start,
                                    h->d_btiles.as<int32_t>(), h->b_sym, h->d_bqueue.as<int>(),
                                    h->d_bcnt.as<int32_t>()), "batched symbolic");
-      if ((st2 = run_scan(h, (int32_t)R, h->d_bcnt.as<int32_t>(), c_rowptr, &dm->grand, none, nullptr)) != KK_OK)
+      if ((st2 = run_scan(h, (int32_t)R, h->d_bcnt.as<int32_t>(), c_rowptr, &dm->grand, none, 0, nullptr)) != KK_OK)
         return st2;
       KK_CUDA(h, launch_b_nclassify(s, h->num_sms, R, dd, h->d_rowpair.as<int32_t>(), c_rowptr,
                                     h->d_bflop.as<long long>(), h->b_num, h->opt.team_vec_min_len,
@@ -2526,7 +2536,7 @@ kk_status kk_spgemm_destroy(kk_spgemm_handle h) {
                     &h->d_sval, &h->d_sball, &h->d_nbin2, &h->d_lrows, &h->d_lrows2, &h->d_mm,
                     &h->d_bdesc, &h->d_rowpair, &h->d_bflop, &h->d_bsbin, &h->d_bnbin, &h->d_bsrows,
                     &h->d_bnrows, &h->d_bcnt, &h->d_btiles, &h->d_bstart, &h->d_bqueue, &h->d_bsplit2,
-                    &h->d_boff, &h->d_bc, &h->d_bclen, &h->d_cw, &h->d_cm, &h->d_cn, &h->d_left, &h->d_wbits,
+                    &h->d_boff, &h->d_bc, &h->d_bclen, &h->d_cw, &h->d_cm, &h->d_cn, &h->d_wbits,
                     &h->d_wslot, &h->d_wnext, &h->d_pa_rp, &h->d_pa_ci, &h->d_pa_v, &h->d_pb_rp, &h->d_pb_ci,
                     &h->d_pb_v, &h->d_pbase})
     b->release();

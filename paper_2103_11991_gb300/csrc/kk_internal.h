@@ -38,10 +38,9 @@ struct LaunchCtx {
   // structure fingerprints of the index arrays at the symbolic call ([0]) and
   // at this numeric call ([1]); null when the kept structure is not in use
   const unsigned long long* fingerprint;
-  // 1: the window tier's rows of at most kWindowMaxNnz columns (the
-  // kept-structure value pass and its rebuild) run in float64 whatever the
-  // call's arithmetic (options.arith = AUTO: on GB300 native float64 measured
-  // faster there, 1.91 ms against 2.42 for the 27-point value pass)
+  // 1: the window and rank tiers' rows run in float64 whatever the call's
+  // arithmetic (options.arith = AUTO: on GB300 native float64 measured faster
+  // there, 1.91 ms against 2.42 for the 27-point value pass)
   int kept_f64;
 };
 
@@ -86,9 +85,12 @@ __device__ __forceinline__ double a_value(const CsrView& A, int i, int p) {
 }
 #endif
 
-// Accumulator tiers.  The thread tier counts as the team tier in statistics.
-enum Tier : int32_t { kTierTeam = 0, kTierCta = 1, kTierDense = 2, kTierWindow = 3, kTierThread = 4 };
-__host__ __device__ constexpr int32_t stat_tier(int32_t t) { return t == kTierThread ? kTierTeam : t; }
+// Accumulator tiers.  In statistics the thread tier counts as the team tier, the
+// rank tier as the window tier.
+enum Tier : int32_t { kTierTeam = 0, kTierCta = 1, kTierDense = 2, kTierWindow = 3, kTierThread = 4, kTierRank = 5 };
+__host__ __device__ constexpr int32_t stat_tier(int32_t t) {
+  return t == kTierThread ? kTierTeam : t == kTierRank ? kTierWindow : t;
+}
 
 // Thread tier (kk_thread.cu): one thread per row, accumulator in registers.
 constexpr int kThreadSymMax = 16;     // symbolic rows: flop bound <= this
@@ -112,16 +114,15 @@ __host__ __device__ constexpr int32_t window_bits(int w) {
   return w == 0 ? 4096 : w == 1 ? 12288 : w == 2 ? 24576 : w == 3 ? 40960 : 65536;
 }
 constexpr int32_t kWindowMaxNnz = 256;   // numeric window rows: nnz(C(i,:)) <= this
-constexpr int32_t kWindowMaxNnzWide = 1024;  // ... or this, in the large-value window bins
-constexpr int32_t kWindowFlopRatio = 128;  // symbolic window used only when W <= ratio * flop
-constexpr int32_t kWindowFlopRatioNum = 512;  // large-value numeric window bins
-// Large-value numeric window bins (nnz(C(i,:)) in (kWindowMaxNnz, kWindowMaxNnzWide]),
-// with value arrays of kWindowMidNnz or kWindowMaxNnzWide slots (the smaller
-// array leaves room for more warps per SM).
-constexpr int32_t kWindowMidNnz = 512;
-constexpr int kNumWideWindowClasses = 3;
-constexpr int32_t kWideWindowBits[kNumWideWindowClasses] = {24576, 40960, 65536};
-constexpr int kMaxWindowBins = kNumWindowClasses + 2 * kNumWideWindowClasses;
+constexpr int32_t kWindowFlopRatio = 128;  // window used only when W <= ratio * flop
+
+// Rank tier (kk_rank.cu): numeric rows without kept structure, nnz(C(i,:)) at
+// most kRankNnz[2], span at most kRankBits of the bin.
+constexpr int kNumRankBits = 5, kNumRankNnz = 3;
+constexpr int32_t kRankBits[kNumRankBits] = {4096, 8192, 16384, 32768, 65536};
+constexpr int32_t kRankNnz[kNumRankNnz] = {256, 512, 1024};
+constexpr int32_t kRankFlopRatio = 512;  // rank tier used only when W <= ratio * flop
+constexpr int kMaxWindowBins = kNumWindowClasses + kNumRankBits * kNumRankNnz;
 
 // Compressed B (the paper's B_C): row j of B as (column >> 5, 32-bit column
 // mask) pairs in column order, stored at B's own row offsets
@@ -147,12 +148,15 @@ struct WinCacheView {
   const uint32_t* m;
   const int32_t* n;
 };
-// Scratch of the numeric window launch: rows left to the window kernel by the
-// kept-structure kernel (count first, then the rows).
-struct WinScratch {
-  int32_t* rows;
-  int32_t* count;
+// One bin of rows: its tier and the accumulator geometry.
+struct BinSpec {
+  int32_t tier;
+  int32_t team;   // lanes per row (team tier); threads per CTA otherwise
+  int32_t slots;  // hash slots (team / CTA tiers); chunk width in columns (dense)
+  int32_t flat;   // 1: lanes walk the flattened (A entry, B entry) products
+  int64_t lo, hi; // bin range of the binning quantity (flop or nnz), inclusive
 };
+
 // Analysis of B (kk_window.cu): clears *sorted_flag unless every row is
 // strictly ascending, sets KK_ERR_BAD_INDEX on out-of-range structure, and,
 // when bc is non-null, writes the compressed rows (pairs counted into *pairs).
@@ -167,24 +171,21 @@ cudaError_t launch_spadd_numeric(const LaunchCtx& ctx, const CsrView& A, const C
                                  double beta, const int64_t* c_rowptr, const int32_t* apos,
                                  const int32_t* bpos, int32_t* c_colind, double* c_vals);
 
-// Numeric phase of window rows with kept structure (kk_kept.cu); rows without
-// it are appended to left_rows / *left_count for the rebuild kernel.
+// Numeric phase of window rows with kept structure (kk_kept.cu).
 cudaError_t launch_num_kept(const LaunchCtx& ctx, const CsrView& A, const CsrView& B,
                             const WinCacheView& cache, const float2* b_split, const int32_t* b_range_bad,
                             int32_t arith, const int64_t* c_rowptr, const int32_t* rows, int32_t nrows,
-                            int32_t* c_colind, double* c_vals, int32_t* left_rows, int32_t* left_count);
+                            int32_t* c_colind, double* c_vals);
+
+// Numeric phase of the rank tier's rows (kk_rank.cu): window of bin.slots
+// columns, at most bin.hi columns of C per row.
+cudaError_t launch_num_rank(const LaunchCtx& ctx, const BinSpec& bin, const CsrView& A, const CsrView& B,
+                            int32_t b_sorted, const BComp& bcomp, const float2* b_split,
+                            const int32_t* b_range_bad, int32_t arith, const int64_t* c_rowptr,
+                            const int32_t* rows, int32_t nrows, int32_t* c_colind, double* c_vals);
 
 cudaError_t launch_analyze_b(const LaunchCtx& ctx, const CsrView& B, int32_t* sorted_flag,
                              int2* bc, int32_t* len, unsigned long long* pairs);
-
-// One bin of rows: its tier and the accumulator geometry.
-struct BinSpec {
-  int32_t tier;
-  int32_t team;   // lanes per row (team tier); threads per CTA otherwise
-  int32_t slots;  // hash slots (team / CTA tiers); chunk width in columns (dense)
-  int32_t flat;   // 1: lanes walk the flattened (A entry, B entry) products
-  int64_t lo, hi; // bin range of the binning quantity (flop or nnz), inclusive
-};
 
 // Arithmetic mode for the numeric kernels.
 enum ArithMode : int32_t { kArithF64 = 1, kArithDF32 = 2 };
@@ -229,13 +230,6 @@ cudaError_t launch_numeric_thread(const LaunchCtx& ctx, const CsrView& A, const 
 cudaError_t launch_symbolic_window(const LaunchCtx& ctx, const BinSpec& bin, const CsrView& A,
                                    const CsrView& B, const BComp& bcomp, const int32_t* rows,
                                    int32_t nrows, int32_t* cnt, const WinCache& cache);
-cudaError_t launch_numeric_window(const LaunchCtx& ctx, const BinSpec& bin, const CsrView& A,
-                                  const CsrView& B, const BComp& bcomp, const WinCacheView& cache,
-                                  const WinScratch& scratch, const float2* b_split,
-                                  const int32_t* b_range_bad, int32_t arith,
-                                  const int64_t* c_rowptr, const int32_t* rows, int32_t nrows,
-                                  int32_t* c_colind, double* c_vals);
-
 // Speculative one-pass (learned form) over rows whose predicted table is
 // 2^log2s slots (log2s in 5..9); see k_num_warp_vec<LOG2S, true>.
 cudaError_t launch_onepass(const LaunchCtx& ctx, int32_t log2s, const CsrView& A, const CsrView& B,
@@ -250,11 +244,6 @@ constexpr int kOnepassClasses = 5;
 // [kOnepassClasses, kLearnedHeavy) window one-pass by window class,
 // kLearnedHeavy = plain path.
 constexpr int kLearnedHeavy = kOnepassClasses + kNumWindowClasses;
-cudaError_t launch_onepass_window(const LaunchCtx& ctx, int32_t wclass, const CsrView& A,
-                                  const CsrView& B, const BComp& bcomp, const float2* b_split,
-                                  const int32_t* b_range_bad, int32_t arith, const int64_t* soff,
-                                  const int32_t* cap, const int32_t* rows, int32_t nrows,
-                                  int32_t* scol, double* sval, int32_t* cnt_out);
 // Speculative one-pass for window rows through a word table (kk_onepass.cu).
 cudaError_t launch_onepass_table(const LaunchCtx& ctx, const CsrView& A, const CsrView& B,
                                  const BComp& bcomp, const float2* b_split,

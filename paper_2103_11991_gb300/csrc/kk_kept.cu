@@ -18,8 +18,7 @@ constexpr size_t al16(size_t x) { return (x + 15) / 16 * 16; }
 // span and more rows are in flight per SM.  Words less than 256 apart never
 // share a slot; a row whose words did collide takes the probing variant of the
 // value pass.  An entry packs the word's bits (low 32), its prefix count (bits
-// 32..47) and the word index (48..63).  Rows without kept structure are
-// appended to `left` for k_num_window.
+// 32..47) and the word index (48..63).
 constexpr int kKeptWarps = 8;
 struct KeptGeom {
   // table u64[kKeptSlots] | vacc u64[kWindowMaxNnz + 2] | ainfo int4[32]
@@ -37,7 +36,6 @@ k_num_kept(CsrView A, CsrView B, WinCacheView cache, const int32_t* __restrict__
            const float2* __restrict__ bspl, const int32_t* __restrict__ b_range_bad, int32_t arith,
            const int64_t* __restrict__ c_rowptr, const int32_t* __restrict__ rows, int32_t nrows,
            int32_t* __restrict__ c_colind, double* __restrict__ c_vals, int* status,
-           int32_t* __restrict__ left_rows, int32_t* __restrict__ left_count,
            const unsigned long long* __restrict__ fp) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -54,8 +52,8 @@ k_num_kept(CsrView A, CsrView B, WinCacheView cache, const int32_t* __restrict__
   for (int r = blockIdx.x * kKeptWarps + warp; r < nrows; r += nw) {
     const int i = rows[r];
     const int L = cache.n[i];
-    if (L < 0 || L > kCacheWords) {
-      if (lane == 0) left_rows[atomicAdd(left_count, 1)] = i;
+    if (L < 0 || L > kCacheWords) {  // only rows with kept structure are binned here
+      if (lane == 0) set_status(status, KK_ERR_STRUCTURE_MISMATCH);
       continue;
     }
     const int lo_c = (row_lo[i] >> 5) * 32;
@@ -128,7 +126,7 @@ k_num_kept(CsrView A, CsrView B, WinCacheView cache, const int32_t* __restrict__
 cudaError_t launch_num_kept(const LaunchCtx& ctx, const CsrView& A, const CsrView& B,
                             const WinCacheView& cache, const float2* b_split, const int32_t* b_range_bad,
                             int32_t arith, const int64_t* c_rowptr, const int32_t* rows, int32_t nrows,
-                            int32_t* c_colind, double* c_vals, int32_t* left_rows, int32_t* left_count) {
+                            int32_t* c_colind, double* c_vals) {
   const size_t smem = (size_t)kKeptWarps * KeptGeom::kWarpBytes;
   const bool check = ctx.fingerprint == nullptr;
   const bool jac = A.jac_s != nullptr;
@@ -150,7 +148,7 @@ cudaError_t launch_num_kept(const LaunchCtx& ctx, const CsrView& A, const CsrVie
   if (blocks < 1) blocks = 1;
   kern<<<(int)blocks, kKeptWarps * 32, smem, ctx.stream>>>(
       A, B, cache, ctx.row_lo, b_split, b_range_bad, arith, c_rowptr, rows, nrows, c_colind, c_vals,
-      ctx.status, left_rows, left_count, ctx.fingerprint);
+      ctx.status, ctx.fingerprint);
   return cudaGetLastError();
 }
 
