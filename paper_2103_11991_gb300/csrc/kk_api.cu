@@ -830,12 +830,13 @@ struct kk_spgemm_handle_s {
   DevBuf d_cn;         // int32[m]
   bool cache_valid = false;
   // wide-tier bit vectors kept by the symbolic phase
-  DevBuf d_wbits, d_wslot, d_wnext;
+  DevBuf d_wbits, d_wslot, d_wnext, d_wtasks, d_widx, d_wtab;
+  int32_t wide_kept = 0;  // rows kept with tasks by the last symbolic call
   bool b_overflow = false;             // the persistent batched form handed a batch to the packed form
   unsigned long long b_overflow_key = 0;  // ... the batch's key (pairs, output pointer, count)
   bool keep_valid = false;
   const void* keep_key[4] = {nullptr, nullptr, nullptr, nullptr};
-  WideKeep keep{nullptr, nullptr, nullptr, 0, 0};  // what the next launches use
+  WideKeep keep{};  // what the next launches use
   size_t dev_total = 0;
   // packed batch: block-diagonal A and B of the last batched symbolic call
   DevBuf d_pa_rp, d_pa_ci, d_pa_v, d_pb_rp, d_pb_ci, d_pb_v, d_pbase;
@@ -862,7 +863,10 @@ struct Misc {
   unsigned long long bc_pairs;   // pairs of the compressed B
   unsigned long long fp[2];      // structure fingerprints: symbolic call, numeric call
   int32_t small_flags[4];        // small-product path: row beyond it, bad index, CTA ticket
+  int32_t wide_kept;             // rows kept with chunk tasks
+  int32_t pad2;
 };
+static_assert(sizeof(Misc) <= 256, "the staging buffer's bin starts follow at byte 256");
 
 kk_status fail(kk_spgemm_handle h, kk_status s, const std::string& msg) {
   if (h) h->last_error = msg;
@@ -996,7 +1000,9 @@ BinTable to_table(const std::vector<BinSpec>& bins, bool numeric, int32_t cols) 
     if (rank || bins[b].tier == kTierWindow) {
       t.win_bits[t.nwin] = bins[b].slots;
       t.win_bin[t.nwin] = (int32_t)b;
-      t.win_q[t.nwin] = bins[b].hi;
+      // a heavy row's products are too many for the window's one warp where the
+      // wide tier's bit vector is no larger than a window
+      t.win_q[t.nwin] = !numeric && cols <= kWindowBits[kNumWindowClasses - 1] ? kWindowMaxFlop : bins[b].hi;
       t.win_kept[t.nwin] = numeric && !rank ? 1 : 0;
       t.win_any_order[t.nwin] = rank ? 1 : 0;
       t.win_ratio[t.nwin] = rank ? kRankFlopRatio : kWindowFlopRatio;
@@ -1133,24 +1139,52 @@ kk_status cache_for_symbolic(kk_spgemm_handle h, int32_t m, bool any_window, con
 // the option is off, no row takes the wide tier or the budget is zero).
 kk_status keep_for_symbolic(kk_spgemm_handle h, int32_t m, int64_t wide_rows, const CsrView& av,
                             const CsrView& bv) {
-  h->keep = WideKeep{nullptr, nullptr, nullptr, 0, 0};
+  h->keep = WideKeep{};
   h->keep_valid = false;
   if (!h->opt.structure_cache || h->opt.wide_cache_mb < 0 || wide_rows <= 0 || m <= 0) return KK_OK;
   const LaunchCtx probe = ctx_of(h);
   if (!wide_symbolic_fits(probe, bv.n) || !wide_numeric_fits(probe, bv.n)) return KK_OK;
   const size_t words = (size_t)wide_word_count(bv.n);
+  // sorted B: rows of more columns than the rank tier takes, computed in chunks;
+  // unsorted B: rows whose values do not fit the wide kernel's shared memory
+  const bool tasks = h->b_sorted != 0;
+  const int32_t chunks = tasks ? wide_max_chunks(bv.n) : 0;
+  const size_t stride = words + ((size_t)chunks * 2 + 3) / 4 * 4;
   const size_t budget = h->opt.wide_cache_mb > 0 ? ((size_t)h->opt.wide_cache_mb << 20) : h->dev_total / 8;
-  long long slots = (long long)(budget / (words * 4));
+  long long slots = (long long)(budget / (stride * 4));
   if (slots > wide_rows) slots = wide_rows;
   if (slots > 0x7fffffff) slots = 0x7fffffff;
   if (slots <= 0) return KK_OK;
-  KK_CUDA(h, h->d_wbits.ensure(words * 4 * (size_t)slots), "alloc wide cache");
+  long long ntasks = tasks ? wide_max_tasks(bv.n, h->stats[6], slots) : 0;
+  if (ntasks > (1 << 28)) ntasks = 1 << 28;
+  KK_CUDA(h, h->d_wbits.ensure(stride * 4 * (size_t)slots), "alloc wide cache");
   KK_CUDA(h, h->d_wslot.ensure(sizeof(int32_t) * (size_t)m), "alloc wide cache");
-  KK_CUDA(h, h->d_wnext.ensure(sizeof(int32_t)), "alloc wide cache");
+  KK_CUDA(h, h->d_wnext.ensure(sizeof(int32_t) * 4), "alloc wide cache");
+  if (tasks) KK_CUDA(h, h->d_wtasks.ensure(sizeof(int2) * (size_t)ntasks), "alloc wide cache");
   KK_CUDA(h, cudaMemsetAsync(h->d_wslot.p, 0xFF, sizeof(int32_t) * (size_t)m, h->stream), "memset");
-  KK_CUDA(h, cudaMemsetAsync(h->d_wnext.p, 0, sizeof(int32_t), h->stream), "memset");
-  h->keep = WideKeep{h->d_wbits.as<uint32_t>(), h->d_wslot.as<int32_t>(), h->d_wnext.as<int32_t>(),
-                     (int32_t)slots, wide_keep_min_cnt(probe, bv.n)};
+  KK_CUDA(h, cudaMemsetAsync(h->d_wnext.p, 0, sizeof(int32_t) * 4, h->stream), "memset");
+  h->keep.bits = h->d_wbits.as<uint32_t>();
+  h->keep.slot = h->d_wslot.as<int32_t>();
+  h->keep.next = h->d_wnext.as<int32_t>();
+  h->keep.tasks = tasks ? h->d_wtasks.as<int2>() : nullptr;
+  h->keep.kept = &h->d_misc.as<Misc>()->wide_kept;
+  h->keep.max_slots = (int32_t)slots;
+  h->keep.min_cnt = tasks ? kRankNnz[kNumRankNnz - 1] : wide_keep_min_cnt(probe, bv.n);
+  h->keep.stride = (int32_t)stride;
+  h->keep.max_chunks = chunks;
+  h->keep.max_tasks = (int32_t)ntasks;
+  if (tasks) {
+    const size_t rows = (size_t)wide_index_slots(bv), tab = (size_t)wide_index_stride(bv.n);
+    KK_CUDA(h, h->d_widx.ensure(sizeof(int32_t) * ((size_t)bv.m + rows)), "alloc wide cache");
+    KK_CUDA(h, h->d_wtab.ensure(sizeof(int32_t) * rows * tab), "alloc wide cache");
+    h->keep.bidx = h->d_widx.as<int32_t>();
+    h->keep.btab = h->d_wtab.as<int32_t>();
+    h->keep.tab_stride = (int32_t)tab;
+    h->keep.shift = wide_chunk_shift(bv.n);
+    KK_CUDA(h, launch_chunk_index(ctx_of(h), bv, h->d_widx.as<int32_t>(), h->d_widx.as<int32_t>() + bv.m,
+                                  h->d_wtab.as<int32_t>()),
+            "index launch");
+  }
   h->keep_valid = true;
   h->keep_key[0] = av.rowptr;
   h->keep_key[1] = av.colind;
@@ -1162,11 +1196,9 @@ kk_status keep_for_symbolic(kk_spgemm_handle h, int32_t m, int64_t wide_rows, co
 // The kept wide bit vectors for a numeric call, if they belong to its arrays.
 void keep_for_numeric(kk_spgemm_handle h, const CsrView& av, const CsrView& bv) {
   if (h->keep_valid && h->keep_key[0] == av.rowptr && h->keep_key[1] == av.colind &&
-      h->keep_key[2] == bv.rowptr && h->keep_key[3] == bv.colind) {
-    h->keep.next = nullptr;  // the numeric phase only reads
-  } else {
-    h->keep = WideKeep{nullptr, nullptr, nullptr, 0, 0};
-  }
+      h->keep_key[2] == bv.rowptr && h->keep_key[3] == bv.colind)
+    return;
+  h->keep = WideKeep{};
 }
 
 // Kept word counts of the rows of this symbolic call (-1: no kept structure),
@@ -1188,6 +1220,22 @@ kk_status cache_view(kk_spgemm_handle h, const CsrView& av, const CsrView& bv, W
     if (st != KK_OK) return st;
     ctx->fingerprint = dm->fp;
   }
+  return KK_OK;
+}
+
+// The rows kept with chunk tasks; *skip_wide = true when no row of the wide
+// tier is left (start: the bins' row starts).
+kk_status launch_kept_chunks(kk_spgemm_handle h, const LaunchCtx& ctx, const CsrView& av, const CsrView& bv,
+                             const std::vector<int32_t>& start, const int64_t* c_rowptr, int32_t* c_colind,
+                             double* c_vals, bool* skip_wide) {
+  *skip_wide = false;
+  if (!ctx.keep.tasks || h->wide_kept <= 0) return KK_OK;
+  KK_CUDA(h, launch_num_chunk(ctx, av, bv, c_rowptr, c_colind, c_vals), "chunk launch");
+  h->stats[9] += 1;
+  int64_t wide = 0;
+  for (size_t b = 0; b < h->num_bins.size(); ++b)
+    if (h->num_bins[b].tier == kTierCta || h->num_bins[b].tier == kTierDense) wide += start[b + 1] - start[b];
+  *skip_wide = wide == h->wide_kept;
   return KK_OK;
 }
 
@@ -1471,7 +1519,7 @@ kk_status kk_spgemm_symbolic(kk_spgemm_handle h, const kk_csr* A, const kk_csr* 
       h->stats[30] = m;
       h->small = true;
       h->cache_valid = false;
-      h->keep = WideKeep{nullptr, nullptr, nullptr, 0, 0};
+      h->keep = WideKeep{};
       h->keep_valid = false;
       h->learned_valid = false;
       h->nnz_c = hm->grand;
@@ -1533,7 +1581,8 @@ kk_status kk_spgemm_symbolic(kk_spgemm_handle h, const kk_csr* A, const kk_csr* 
     WinCache wcache;
     if ((st = cache_for_symbolic(h, m, any_win, av, bv, &wcache)) != KK_OK) return st;
     int64_t tier_rows[4] = {0, 0, 0, 0};
-    for (int b = 0; b < nbs; ++b) {
+    ctx.bcomp = bcomp;
+    for (int b = nbs - 1; b >= 0; --b) {  // heaviest rows first: they get the kept-bits slots
       const int cnt = h_start[b + 1] - h_start[b];
       if (cnt <= 0) continue;
       tier_rows[stat_tier(h->sym_bins[b].tier)] += cnt;
@@ -1588,6 +1637,7 @@ kk_status kk_spgemm_symbolic(kk_spgemm_handle h, const kk_csr* A, const kk_csr* 
     h->stats[20 + t] = (int64_t)hm->tier_a[t];
     h->stats[26 + t] = (int64_t)hm->tier_f[t];
   }
+  h->wide_kept = hm->wide_kept;
   h->stats[24] = (int64_t)hm->kept;
   h->stats[25] = (int64_t)hm->bc_pairs;
   h->am = m;
@@ -1669,9 +1719,21 @@ static kk_status numeric_impl(kk_spgemm_handle h, const kk_csr* A, const kk_csr*
   }
   WinCacheView wview;
   if ((st = cache_view(h, av, bv, &wview, &ctx)) != KK_OK) return st;
+  bool skip_wide = false;
+  if (jac && ctx.keep.tasks && h->wide_kept > 0) {
+    // the kept rows' scales come before their chunks
+    for (int b = 0; b < nbn; ++b) {
+      const int cnt = h->num_start[b + 1] - h->num_start[b];
+      if (cnt <= 0 || (h->num_bins[b].tier != kTierCta && h->num_bins[b].tier != kTierDense)) continue;
+      cudaError_t e = launch_jacobi_rows(h, av, h->d_nrows.as<int32_t>() + h->num_start[b], cnt);
+      if (e != cudaSuccess) return cuda_fail(h, e, "Jacobi launch");
+    }
+  }
+  if ((st = launch_kept_chunks(h, ctx, av, bv, h->num_start, c_rowptr, c_colind, c_vals, &skip_wide)) != KK_OK) return st;
   for (int b = 0; b < nbn; ++b) {
     const int cnt = h->num_start[b + 1] - h->num_start[b];
     if (cnt <= 0) continue;
+    if (skip_wide && (h->num_bins[b].tier == kTierCta || h->num_bins[b].tier == kTierDense)) continue;
     h->stats[9] += 1;
     const int32_t* rows = h->d_nrows.as<int32_t>() + h->num_start[b];
     if (jac && h->num_bins[b].tier != kTierThread) {
@@ -1863,7 +1925,7 @@ kk_status kk_spgemm_learned_symbolic(kk_spgemm_handle h, const kk_csr* A, const 
   h->have_symbolic = false;
   h->small = false;
   h->learned_valid = false;
-  h->keep = WideKeep{nullptr, nullptr, nullptr, 0, 0};
+  h->keep = WideKeep{};
   h->keep_valid = false;
   const int32_t m = A->m;
   const size_t mm1 = (size_t)(m > 0 ? m : 1);
@@ -1995,8 +2057,9 @@ kk_status kk_spgemm_learned_symbolic(kk_spgemm_handle h, const kk_csr* A, const 
     if ((st = cache_for_symbolic(h, m, any_win, av, bv, &wcache)) != KK_OK) return st;
     if ((st = keep_for_symbolic(h, m, wide_rows, av, bv)) != KK_OK) return st;
     ctx = ctx_of(h);
+    ctx.bcomp = bcomp;
     int64_t plain_rows = 0;
-    for (int b = 0; b < nbs; ++b) {
+    for (int b = nbs - 1; b >= 0; --b) {
       const int cnt = h_start[b + 1] - h_start[b];
       if (cnt <= 0) continue;
       plain_rows += cnt;
@@ -2035,6 +2098,7 @@ kk_status kk_spgemm_learned_symbolic(kk_spgemm_handle h, const kk_csr* A, const 
   h->nnz_c = m > 0 ? hm->grand : 0;
   h->num_start.assign(h_start, h_start + nbn + 1);
   h->lnum_start.assign(h_start2, h_start2 + nbn + 1);
+  h->wide_kept = hm->wide_kept;
   h->stats[24] = (int64_t)hm->kept;
   h->stats[25] = (int64_t)hm->bc_pairs;
   h->am = m;
@@ -2081,9 +2145,13 @@ kk_status kk_spgemm_learned_numeric(kk_spgemm_handle h, const kk_csr* A, const k
   }
   WinCacheView wview;
   if ((st = cache_view(h, av, bv, &wview, &ctx)) != KK_OK) return st;
+  bool skip_wide = false;
+  if ((st = launch_kept_chunks(h, ctx, av, bv, h->lnum_start, c_rowptr, c_colind, c_vals, &skip_wide)) != KK_OK)
+    return st;
   for (int b = 0; b < nbn; ++b) {
     const int cnt = h->lnum_start[b + 1] - h->lnum_start[b];
     if (cnt <= 0) continue;
+    if (skip_wide && (h->num_bins[b].tier == kTierCta || h->num_bins[b].tier == kTierDense)) continue;
     const int32_t* rows = h->d_lrows2.as<int32_t>() + h->lnum_start[b];
     e = launch_numeric_rows(h, ctx, h->num_bins[b], av, bv, bcomp, wview, bsplit, arith, c_rowptr, rows, cnt,
                             c_colind, c_vals);
@@ -2537,7 +2605,7 @@ kk_status kk_spgemm_destroy(kk_spgemm_handle h) {
                     &h->d_bdesc, &h->d_rowpair, &h->d_bflop, &h->d_bsbin, &h->d_bnbin, &h->d_bsrows,
                     &h->d_bnrows, &h->d_bcnt, &h->d_btiles, &h->d_bstart, &h->d_bqueue, &h->d_bsplit2,
                     &h->d_boff, &h->d_bc, &h->d_bclen, &h->d_cw, &h->d_cm, &h->d_cn, &h->d_wbits,
-                    &h->d_wslot, &h->d_wnext, &h->d_pa_rp, &h->d_pa_ci, &h->d_pa_v, &h->d_pb_rp, &h->d_pb_ci,
+                    &h->d_wslot, &h->d_wnext, &h->d_wtasks, &h->d_widx, &h->d_wtab, &h->d_pa_rp, &h->d_pa_ci, &h->d_pa_v, &h->d_pb_rp, &h->d_pb_ci,
                     &h->d_pb_v, &h->d_pbase})
     b->release();
   for (void* p : {h->h_bdesc, h->h_bdesc2, h->h_boff})

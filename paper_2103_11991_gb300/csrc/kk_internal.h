@@ -14,14 +14,33 @@ void timer_begin(KernelTimer* t, cudaStream_t s, const char* name);
 void timer_end(KernelTimer* t, cudaStream_t s);
 
 // Bit vectors of wide-tier rows kept by the symbolic phase for the numeric
-// phase of the same arrays: rows whose nnz(C(i,:)) exceeds min_cnt (their
-// values go to C with atomics) get a slot of `words` u32 when one is left.
+// phase of the same arrays: rows whose nnz(C(i,:)) exceeds min_cnt get a slot
+// of `stride` u32 (the bits, then the chunk table) when one is left.  With
+// tasks (sorted B) the numeric phase computes them chunk by chunk
+// (k_num_chunk); without, the wide kernel loads their bits.
 struct WideKeep {
-  uint32_t* bits;     // max_slots slots of `words` words
+  uint32_t* bits;     // max_slots slots
   int32_t* slot;      // per row: slot or -1
-  int32_t* next;      // slot counter
+  int32_t* next;      // [0] slots, [1] tasks, [2] tasks claimed by the numeric phase, [3] indexed rows of B
+  int2* tasks;        // (row, chunk), max_tasks of them; null: no tasks
+  int* kept;          // += rows kept with tasks
+  const int32_t* bidx;  // index slot of every row of B (-1: none)
+  const int32_t* btab;  // tab_stride positions per slot
+  int32_t tab_stride;
+  int32_t shift;        // chunks end at multiples of 2^shift columns
   int32_t max_slots;  // 0: nothing kept / nothing to use
   int32_t min_cnt;
+  int32_t stride;
+  int32_t max_chunks;  // chunk table entries of a slot
+  int32_t max_tasks;
+};
+
+// Compressed B (the paper's B_C): row j of B as (column >> 5, 32-bit column
+// mask) pairs in column order, stored at B's own row offsets
+// bc[B.rowptr[j] .. B.rowptr[j] + len[j]).  Built only for sorted B.
+struct BComp {
+  const int2* bc;
+  const int32_t* len;
 };
 
 struct LaunchCtx {
@@ -42,6 +61,7 @@ struct LaunchCtx {
   // arithmetic (options.arith = AUTO: on GB300 native float64 measured faster
   // there, 1.91 ms against 2.42 for the 27-point value pass)
   int kept_f64;
+  BComp bcomp;  // compressed B, when the call has it (wide symbolic)
 };
 
 struct CsrView {
@@ -115,6 +135,7 @@ __host__ __device__ constexpr int32_t window_bits(int w) {
 }
 constexpr int32_t kWindowMaxNnz = 256;   // numeric window rows: nnz(C(i,:)) <= this
 constexpr int32_t kWindowFlopRatio = 128;  // window used only when W <= ratio * flop
+constexpr long long kWindowMaxFlop = 4096;  // symbolic rows of a narrow B (k <= 65,536): flop bound <= this
 
 // Rank tier (kk_rank.cu): numeric rows without kept structure, nnz(C(i,:)) at
 // most kRankNnz[2], span at most kRankBits of the bin.
@@ -123,14 +144,6 @@ constexpr int32_t kRankBits[kNumRankBits] = {4096, 8192, 16384, 32768, 65536};
 constexpr int32_t kRankNnz[kNumRankNnz] = {256, 512, 1024};
 constexpr int32_t kRankFlopRatio = 512;  // rank tier used only when W <= ratio * flop
 constexpr int kMaxWindowBins = kNumWindowClasses + kNumRankBits * kNumRankNnz;
-
-// Compressed B (the paper's B_C): row j of B as (column >> 5, 32-bit column
-// mask) pairs in column order, stored at B's own row offsets
-// bc[B.rowptr[j] .. B.rowptr[j] + len[j]).  Built only for sorted B.
-struct BComp {
-  const int2* bc;
-  const int32_t* len;
-};
 
 // Per-row structure kept by the symbolic window kernel for the numeric phase
 // of the same A and B: the row's non-empty window words (index relative to
@@ -211,10 +224,20 @@ int32_t wide_keep_min_cnt(const LaunchCtx& ctx, int32_t k);  // rows above this 
 bool wide_numeric_fits(const LaunchCtx& ctx, int32_t k);
 cudaError_t launch_symbolic_wide(const LaunchCtx& ctx, const CsrView& A, const CsrView& B,
                                  const long long* flop, const int32_t* rows, int32_t nrows,
-                                 int32_t* cnt);
+                                 int32_t* cnt, bool light);
 cudaError_t launch_numeric_wide(const LaunchCtx& ctx, const CsrView& A, const CsrView& B,
                                 const int64_t* c_rowptr, const int32_t* rows, int32_t nrows,
-                                int32_t* c_colind, double* c_vals);
+                                int32_t* c_colind, double* c_vals, long long max_nnz);
+// The rows kept with tasks by the symbolic phase (ctx.keep), and the index of B's
+// longer rows that their numeric phase uses.
+int32_t wide_chunk_shift(int32_t k);
+int32_t wide_max_chunks(int32_t k);                                       // of a row of k columns
+long long wide_max_tasks(int32_t k, long long flops, long long slots);  // of `slots` rows with `flops` products
+int32_t wide_index_stride(int32_t k);
+int32_t wide_index_slots(const CsrView& B);
+cudaError_t launch_chunk_index(const LaunchCtx& ctx, const CsrView& B, int32_t* slot, int32_t* row, int32_t* tab);
+cudaError_t launch_num_chunk(const LaunchCtx& ctx, const CsrView& A, const CsrView& B, const int64_t* c_rowptr,
+                             int32_t* c_colind, double* c_vals);
 
 cudaError_t launch_symbolic_thread(const LaunchCtx& ctx, const CsrView& A, const CsrView& B,
                                    const int32_t* rows, int32_t nrows, int32_t* cnt);

@@ -729,7 +729,7 @@ cudaError_t launch_numeric_bin(const LaunchCtx& ctx, const BinSpec& bin, const C
   }
   if ((bin.tier == kTierCta || bin.tier == kTierDense) && wide_numeric_fits(ctx, B.n)) {
     timer_begin(ctx.timer, ctx.stream, "num_wide");
-    e = launch_numeric_wide(ctx, A, B, c_rowptr, rows, nrows, c_colind, c_vals);
+    e = launch_numeric_wide(ctx, A, B, c_rowptr, rows, nrows, c_colind, c_vals, bin.hi);
     timer_end(ctx.timer, ctx.stream);
     return e;
   }

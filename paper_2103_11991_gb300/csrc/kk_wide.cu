@@ -30,7 +30,14 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kWideU = 4;      // warp steps whose loads are issued together
-constexpr int kWideBlock = 1024;
+constexpr int kWideBlock = 1024;  // threads of a CTA on the heaviest rows
+// Chunks of a kept row (k_num_chunk): they end at multiples of 2^shift columns,
+// with at most kChunkSlots columns of C and kChunkWords words of the bit vector.
+constexpr int kChunkSlots = 3584;
+constexpr int kChunkWords = 2048;
+constexpr int kIndexMinLen = 128;  // B rows with an index (positions of the multiples of 2^shift)
+__host__ __device__ constexpr int chunk_shift(int k) { return k <= (1 << 18) ? 9 : 10; }
+__host__ __device__ constexpr int chunk_cols(int k) { return kChunkSlots - (1 << chunk_shift(k)); }
 constexpr int kKeepU = 4;      // 16-byte loads in flight per thread when a kept bit vector is loaded
 
 // Words of the column bit vector: ceil(k / 32) rounded up to a multiple of
@@ -92,30 +99,33 @@ __device__ __forceinline__ T block_exscan(T v, T* tmp, T* total) {
 
 // Shared scratch of the product walk: the segment's product prefix and B row
 // starts, the work-item counter and the scan buffer.
-constexpr int kSeg = kWideBlock;       // A entries per segment (one per thread)
+// SEG: A entries per segment, one per thread of the CTA.
 constexpr int kItem = 32 * kWideU * 2;  // products per work item
+template <int SEG>
 struct WalkSmem {
-  long long pre[kSeg + 1];
-  int bst[kSeg];
+  long long pre[SEG + 1];
+  int bst[SEG];
   long long tmp[33];
   int next;
 };
 
 // Visit every product A(i,j)*B(j,c) of the A entries [pa, pe) of a row with
 // the whole CTA, balanced to kItem products: the row's A entries are taken
-// kSeg at a time; their products, flattened in storage order, are cut into
+// SEG at a time; their products, flattened in storage order, are cut into
 // items of kItem that warps claim from a shared counter; a warp walks its item
 // with lanes over consecutive products, 32 A entries' bounds held in lanes,
-// and issues kWideU steps of loads before using them.  use(c, ab, ok) gets
-// the column (and with VALS the product a*b in float64).  Ends with a barrier.
-template <bool VALS, class Use>
-__device__ __forceinline__ void wide_walk(const CsrView& A, const CsrView& B, int pa, int pe,
-                                          WalkSmem& ws, int& bad, Use use, int row = 0) {
+// and issues kWideU steps of loads before using them.  use(c, ab) gets the
+// column (-1 on idle lanes) and with VALS the product a*b in float64; with
+// PAIRS the walk is over the compressed rows of B and use(word, mask) gets a
+// pair (mask 0 on idle lanes).  Ends with a barrier.
+template <int SEG, bool VALS, bool PAIRS, class Use>
+__device__ __forceinline__ void wide_walk(const CsrView& A, const CsrView& B, const BComp& bc, int pa, int pe,
+                                          WalkSmem<SEG>& ws, int& bad, Use use, int row = 0) {
   const int lane = threadIdx.x & 31;
   const int32_t* __restrict__ bcol = B.colind;
   const double* __restrict__ bval = B.vals;
-  for (int s0 = pa; s0 < pe; s0 += kSeg) {
-    const int ns = min(kSeg, pe - s0);
+  for (int s0 = pa; s0 < pe; s0 += SEG) {
+    const int ns = min(SEG, pe - s0);
     {
       const int t = threadIdx.x;
       int bs = 0;
@@ -124,7 +134,7 @@ __device__ __forceinline__ void wide_walk(const CsrView& A, const CsrView& B, in
         const int j = A.colind[s0 + t];
         if ((unsigned)j < (unsigned)B.m) {
           bs = B.rowptr[j];
-          len = B.rowptr[j + 1] - bs;
+          len = PAIRS ? bc.len[j] : B.rowptr[j + 1] - bs;
         } else {
           bad = 1;
         }
@@ -173,6 +183,7 @@ __device__ __forceinline__ void wide_walk(const CsrView& A, const CsrView& B, in
         for (int g = done; g < lim; g += 32 * kWideU) {
           int col[kWideU];
           double ab[kWideU];
+          uint32_t mask[kWideU];
 #pragma unroll
           for (int u = 0; u < kWideU; ++u) {
             const int f = g + u * 32 + lane;
@@ -186,13 +197,23 @@ __device__ __forceinline__ void wide_walk(const CsrView& A, const CsrView& B, in
             const double a = VALS ? __shfl_sync(kFull, al, own) : 0.0;
             col[u] = -1;
             ab[u] = 0.0;
+            mask[u] = 0u;
             if (f < lim) {
-              col[u] = bcol[q];
+              if (PAIRS) {
+                const int2 v = bc.bc[q];
+                col[u] = v.x;
+                mask[u] = (uint32_t)v.y;
+              } else {
+                col[u] = bcol[q];
+              }
               if (VALS) ab[u] = a * bval[q];
             }
           }
 #pragma unroll
-          for (int u = 0; u < kWideU; ++u) use(col[u], ab[u]);
+          for (int u = 0; u < kWideU; ++u) {
+            if constexpr (PAIRS) use(col[u], mask[u]);
+            else use(col[u], ab[u]);
+          }
         }
         done = lim;
         t0 += 32;
@@ -287,23 +308,24 @@ __device__ __forceinline__ void stage_walk(const CsrView& B, StageState& st, int
 // piece's B entries, kWideU loads in flight.  Same contract as wide_walk.
 constexpr int kPieceMin = 256, kPieceMax = 2048;
 constexpr long long kLongMean = 64;
+template <int SEG>
 struct LongSmem {
-  int ipre[kSeg + 1];
-  int bst[kSeg];
-  int blen[kSeg];
+  int ipre[SEG + 1];
+  int bst[SEG];
+  int blen[SEG];
   int tmp[33];
   int next;
 };
 
-template <bool VALS, class Use>
-__device__ __forceinline__ void wide_walk_long(const CsrView& A, const CsrView& B, int pa, int pe,
-                                               LongSmem& ls, int psz, int& bad, Use use, StageState* st = nullptr,
-                                               int* status = nullptr, int row = 0) {
+template <int SEG, bool VALS, bool PAIRS, class Use>
+__device__ __forceinline__ void wide_walk_long(const CsrView& A, const CsrView& B, const BComp& bc, int pa, int pe,
+                                               LongSmem<SEG>& ls, int psz, int& bad, Use use,
+                                               StageState* st = nullptr, int* status = nullptr, int row = 0) {
   const int lane = threadIdx.x & 31;
   const int32_t* __restrict__ bcol = B.colind;
   const double* __restrict__ bval = B.vals;
-  for (int s0 = pa; s0 < pe; s0 += kSeg) {
-    const int ns = min(kSeg, pe - s0);
+  for (int s0 = pa; s0 < pe; s0 += SEG) {
+    const int ns = min(SEG, pe - s0);
     {
       const int t = threadIdx.x;
       int bs = 0, len = 0;
@@ -311,7 +333,7 @@ __device__ __forceinline__ void wide_walk_long(const CsrView& A, const CsrView& 
         const int j = A.colind[s0 + t];
         if ((unsigned)j < (unsigned)B.m) {
           bs = B.rowptr[j];
-          len = B.rowptr[j + 1] - bs;
+          len = PAIRS ? bc.len[j] : B.rowptr[j + 1] - bs;
         } else {
           bad = 1;
         }
@@ -348,26 +370,39 @@ __device__ __forceinline__ void wide_walk_long(const CsrView& A, const CsrView& 
       const int piece = it - ls.ipre[t];
       const int q0 = ls.bst[t] + piece * psz;
       const int n = min(psz, ls.blen[t] - piece * psz);
-      if (!VALS && st != nullptr && st->ok && n >= 2 * kStageCols) {
-        stage_walk(B, *st, q0, n, status, [&](int c) { use(c, 0.0); });
-        continue;
+      if constexpr (!VALS && !PAIRS) {
+        if (st != nullptr && st->ok && n >= 2 * kStageCols) {
+          stage_walk(B, *st, q0, n, status, [&](int c) { use(c, 0.0); });
+          continue;
+        }
       }
       const double a = VALS ? a_value(A, row, s0 + t) : 0.0;
       for (int g = 0; g < n; g += 32 * kWideU) {
         int col[kWideU];
         double ab[kWideU];
+        uint32_t mask[kWideU];
 #pragma unroll
         for (int u = 0; u < kWideU; ++u) {
           const int f = g + u * 32 + lane;
           col[u] = -1;
           ab[u] = 0.0;
+          mask[u] = 0u;
           if (f < n) {
-            col[u] = bcol[q0 + f];
+            if (PAIRS) {
+              const int2 v = bc.bc[q0 + f];
+              col[u] = v.x;
+              mask[u] = (uint32_t)v.y;
+            } else {
+              col[u] = bcol[q0 + f];
+            }
             if (VALS) ab[u] = a * bval[q0 + f];
           }
         }
 #pragma unroll
-        for (int u = 0; u < kWideU; ++u) use(col[u], ab[u]);
+        for (int u = 0; u < kWideU; ++u) {
+          if constexpr (PAIRS) use(col[u], mask[u]);
+          else use(col[u], ab[u]);
+        }
       }
     }
     __syncthreads();
@@ -375,9 +410,10 @@ __device__ __forceinline__ void wide_walk_long(const CsrView& A, const CsrView& 
 }
 
 // The two walks' shared state (never used at the same time).
+template <int SEG>
 union WideWalkSmem {
-  WalkSmem ws;
-  LongSmem ls;
+  WalkSmem<SEG> ws;
+  LongSmem<SEG> ls;
 };
 
 // Walk of row i: 0 for the flattened walk, else the piece size of the
@@ -386,19 +422,31 @@ union WideWalkSmem {
 // of the CTA, kPieceMin .. kPieceMax products each.
 __device__ __forceinline__ int wide_piece(const long long* flop, int i, int pa, int pe) {
   if (flop == nullptr || pe <= pa || flop[i] < kLongMean * (long long)(pe - pa)) return 0;
-  const long long per = flop[i] / (kWideBlock / 32 * 8);
+  const long long per = flop[i] / ((int)blockDim.x / 32 * 8);
   return per <= kPieceMin ? kPieceMin : per >= kPieceMax ? kPieceMax : (int)per;
 }
 
 // OR the column bits of the products of A entries [pa, pe) into bits (and,
-// with SUM, the summary bits of their words).  Ends with a barrier.
-template <bool SUM>
-__device__ __forceinline__ void wide_set_bits(const CsrView& A, const CsrView& B, int pa, int pe,
-                                              int psz, WideWalkSmem& wsm, uint32_t* bits,
+// with SUM, the summary bits of their words).  PAIRS: from the compressed B,
+// whose pairs of one row touch different words (a long row's neighbouring
+// columns share words, and its lanes' atomics on one word take turns).  Ends
+// with a barrier.
+template <int SEG, bool SUM, bool PAIRS>
+__device__ __forceinline__ void wide_set_bits(const CsrView& A, const CsrView& B, const BComp& bc, int pa, int pe,
+                                              int psz, WideWalkSmem<SEG>& wsm, uint32_t* bits,
                                               uint32_t* sum, int words, int& bad, StageState* st = nullptr,
                                               int* status = nullptr) {
-  auto set = [&](int c, double) {
-    if (c >= 0) {
+  auto set = [&](int c, auto v) {
+    if constexpr (PAIRS) {
+      if (v != 0u) {
+        if ((unsigned)c < (unsigned)words) {
+          atomicOr(&bits[c], v);
+          if (SUM) atomicOr(&sum[c >> 5], 1u << (c & 31));
+        } else {
+          bad = 1;
+        }
+      }
+    } else if (c >= 0) {
       if ((unsigned)c < (unsigned)(words * 32)) {
         atomicOr(&bits[c >> 5], 1u << (c & 31));
         if (SUM) atomicOr(&sum[c >> 10], 1u << ((c >> 5) & 31));
@@ -407,21 +455,62 @@ __device__ __forceinline__ void wide_set_bits(const CsrView& A, const CsrView& B
       }
     }
   };
-  if (psz > 0) wide_walk_long<false>(A, B, pa, pe, wsm.ls, psz, bad, set, st, status);
-  else wide_walk<false>(A, B, pa, pe, wsm.ws, bad, set);
+  if (psz > 0) wide_walk_long<SEG, false, PAIRS>(A, B, bc, pa, pe, wsm.ls, psz, bad, set, st, status);
+  else wide_walk<SEG, false, PAIRS>(A, B, bc, pa, pe, wsm.ws, bad, set);
 }
 
-__global__ void __launch_bounds__(kWideBlock, 1)
-k_sym_wide(CsrView A, CsrView B, int32_t words, uint32_t sum_off, uint32_t stage_off,
+// The chunk table of a kept row (see k_num_chunk) and its tasks: the bit vector
+// in groups of 2^shift columns; a group ends a chunk when the count of columns
+// passes a multiple of chunk_cols in it or when it is the last of kChunkWords
+// words.  end[c] = (first word, first rank) past chunk c.  Returns false when
+// the tasks do not fit (the row is then not kept).
+template <int BLOCK>
+__device__ __forceinline__ bool wide_chunks(const uint32_t* bits, int words, int row, const WideKeep& keep,
+                                            int2* __restrict__ end, int* tmp, int* s_base) {
+  const uint4* b4 = reinterpret_cast<const uint4*>(bits);
+  const int gw = 1 << (keep.shift - 5), np = gw >> 2;  // words and 16-byte pieces of a group
+  const int ngroups = words / gw;
+  const int most = kChunkSlots - (1 << keep.shift);
+  int run = 0, nch = 0;
+  for (int g0 = 0; g0 < ngroups; g0 += BLOCK) {
+    const int g = g0 + threadIdx.x;
+    int c = 0;
+    if (g < ngroups) {
+      for (int k = 0; k < np; ++k) {  // rotated: the lanes' pieces spread over the banks
+        const uint4 v = b4[g * np + ((k + threadIdx.x) & (np - 1))];
+        c += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+      }
+    }
+    int tot, nc;
+    const int p = run + block_exscan<int>(c, tmp, &tot) + c;
+    const bool last = g < ngroups && ((g + 1) * gw % kChunkWords == 0 || g + 1 == ngroups ||
+                                      p / most != (p - c) / most);
+    const int at = nch + block_exscan<int>(last ? 1 : 0, tmp, &nc);
+    if (last && at < keep.max_chunks) end[at] = make_int2((g + 1) * gw, p);
+    run += tot;
+    nch += nc;
+  }
+  if (threadIdx.x == 0) *s_base = atomicAdd(keep.next + 1, nch);
+  __syncthreads();
+  const int base = *s_base;
+  const bool ok = nch <= keep.max_chunks && base + nch <= keep.max_tasks;
+  for (int c = threadIdx.x; c < nch && base + c < keep.max_tasks; c += BLOCK)
+    keep.tasks[base + c] = ok ? make_int2(row, c) : make_int2(-1, 0);
+  return ok;
+}
+
+template <int BLOCK, bool PAIRS>
+__global__ void __launch_bounds__(BLOCK)
+k_sym_wide(CsrView A, CsrView B, BComp bc, int32_t words, uint32_t sum_off, uint32_t stage_off,
            const long long* __restrict__ flop, const int32_t* __restrict__ rows, int32_t nrows,
            int32_t* __restrict__ cnt, WideKeep keep, int* status) {
   extern __shared__ __align__(16) unsigned char wsm[];
   uint32_t* bits = reinterpret_cast<uint32_t*>(wsm);
   uint32_t* sum = reinterpret_cast<uint32_t*>(wsm + sum_off);
-  __shared__ WideWalkSmem walk;
+  __shared__ WideWalkSmem<BLOCK> walk;
   __shared__ int tmp[33];
-  __shared__ int s_slot;
-  __shared__ unsigned long long sbar[kWideBlock / 32 * 2];
+  __shared__ int s_slot, s_base;
+  __shared__ unsigned long long sbar[BLOCK / 32 * 2];
   const int nsum = words >> 5;
   // staging of long B-row pieces through bulk copies (stage_off = 0: off)
   StageState stage{nullptr, nullptr, 0u, stage_off != 0};
@@ -442,15 +531,15 @@ k_sym_wide(CsrView A, CsrView B, int32_t words, uint32_t sum_off, uint32_t stage
   int bad = 0;
   for (int r = blockIdx.x; r < nrows; r += gridDim.x) {
     const int i = rows[r];
-    const bool sparse = flop[i] < (long long)words;  // few words touched: walk the summary
+    // few words touched: walk the summary instead of all words.  Such a row
+    // keeps nothing; with chunk tasks the line lies lower, because a kept row's
+    // numeric phase is much the faster one.
+    const bool sparse = flop[i] < (long long)(keep.tasks ? words / 4 : words);
     const int lng = wide_piece(flop, i, A.rowptr[i], A.rowptr[i + 1]);
     int c = 0;
     if (sparse) {
-      // few words touched: count and clear them through the summary (such rows
-      // keep nothing: walking their products again costs less than storing
-      // and reloading a k-bit vector)
-      wide_set_bits<true>(A, B, A.rowptr[i], A.rowptr[i + 1], lng, walk, bits, sum, words, bad,
-                          stage_off ? &stage : nullptr, status);
+      wide_set_bits<BLOCK, true, PAIRS>(A, B, bc, A.rowptr[i], A.rowptr[i + 1], lng, walk, bits, sum, words, bad,
+                                        stage_off ? &stage : nullptr, status);
       for (int s = threadIdx.x; s < nsum; s += blockDim.x) {
         uint32_t m = sum[s];
         sum[s] = 0u;
@@ -466,31 +555,36 @@ k_sym_wide(CsrView A, CsrView B, int32_t words, uint32_t sum_off, uint32_t stage
       block_exscan<int>(c, tmp, &tot);
       if (threadIdx.x == 0) cnt[i] = tot;
     } else {
-      wide_set_bits<false>(A, B, A.rowptr[i], A.rowptr[i + 1], lng, walk, bits, sum, words, bad,
-                           stage_off ? &stage : nullptr, status);
+      wide_set_bits<BLOCK, false, PAIRS>(A, B, bc, A.rowptr[i], A.rowptr[i + 1], lng, walk, bits, sum, words, bad,
+                                         stage_off ? &stage : nullptr, status);
       for (int w = threadIdx.x * 4; w < words; w += blockDim.x * 4) {
         const uint4 v = *reinterpret_cast<const uint4*>(&bits[w]);
         c += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
       }
       int tot;
       block_exscan<int>(c, tmp, &tot);
-      // rows whose values will go to C by atomics keep their bits for the
-      // numeric phase, while slots last
+      // kept rows store their bits for the numeric phase, while slots last
       if (threadIdx.x == 0) {
         int sl = -1;
         if (keep.max_slots > 0 && tot > keep.min_cnt) {
           sl = atomicAdd(keep.next, 1);
           if (sl >= keep.max_slots) sl = -1;
-          if (sl >= 0) keep.slot[i] = sl;
         }
         s_slot = sl;
       }
       __syncthreads();
-      const int sl = s_slot;
-      uint32_t* dst = sl >= 0 ? keep.bits + (size_t)sl * words : nullptr;
+      int sl = s_slot;
+      uint32_t* dst = sl >= 0 ? keep.bits + (size_t)sl * keep.stride : nullptr;
+      if (sl >= 0 && keep.tasks &&
+          !wide_chunks<BLOCK>(bits, words, i, keep, reinterpret_cast<int2*>(dst + words), tmp, &s_base))
+        sl = -1;
+      if (sl >= 0 && threadIdx.x == 0) {
+        keep.slot[i] = sl;
+        if (keep.tasks) atomicAdd(keep.kept, 1);
+      }
       for (int w = threadIdx.x * 4; w < words; w += blockDim.x * 4) {
         uint4* q = reinterpret_cast<uint4*>(&bits[w]);
-        if (dst) *reinterpret_cast<uint4*>(&dst[w]) = *q;
+        if (sl >= 0) *reinterpret_cast<uint4*>(&dst[w]) = *q;
         *q = make_uint4(0u, 0u, 0u, 0u);
       }
       if (threadIdx.x == 0) cnt[i] = tot;
@@ -584,12 +678,15 @@ __device__ __forceinline__ void wide_write_columns(const uint32_t* bits, const u
   }
 }
 
-__global__ void __launch_bounds__(kWideBlock, 1)
+// Rows without chunk tasks.  BLOCK threads per row; vcap value slots.
+template <int BLOCK>
+__global__ void __launch_bounds__(BLOCK)
 k_num_wide(CsrView A, CsrView B, int32_t words, int32_t vcap, uint32_t sum_off, uint32_t reg_off,
            uint32_t val_off, const int64_t* __restrict__ c_rowptr, const long long* __restrict__ flop,
            const int32_t* __restrict__ rows, int32_t nrows, int32_t* __restrict__ c_colind,
            double* __restrict__ c_vals, WideKeep keep, int* status) {
   extern __shared__ __align__(16) unsigned char wsm[];
+  const BComp none{nullptr, nullptr};
   uint32_t* bits = reinterpret_cast<uint32_t*>(wsm);
   uint32_t* sum = reinterpret_cast<uint32_t*>(wsm + sum_off);
   uint16_t* wpre16 = reinterpret_cast<uint16_t*>(wsm + reg_off);  // rows with values here
@@ -597,7 +694,7 @@ k_num_wide(CsrView A, CsrView B, int32_t words, int32_t vcap, uint32_t sum_off, 
   uint8_t* wpre8 = wsm + reg_off + (size_t)(words / 8) * 4;       // rows with values in C
   double* vals = reinterpret_cast<double*>(wsm + val_off);
   uint16_t* list = reinterpret_cast<uint16_t*>(wsm + val_off);
-  __shared__ WideWalkSmem walk;
+  __shared__ WideWalkSmem<BLOCK> walk;
   __shared__ int tmp[33];
   __shared__ int col_next;
   const int nsum = words >> 5;
@@ -610,6 +707,7 @@ k_num_wide(CsrView A, CsrView B, int32_t words, int32_t vcap, uint32_t sum_off, 
   int bad = 0, mismatch = 0;
   for (int r = blockIdx.x; r < nrows; r += gridDim.x) {
     const int i = rows[r];
+    if (keep.tasks && keep.slot[i] >= 0) continue;  // k_num_chunk's
     const int pa = A.rowptr[i], pe = A.rowptr[i + 1];
     const int64_t off = c_rowptr[i];
     const int cnt = (int)(c_rowptr[i + 1] - off);
@@ -619,7 +717,7 @@ k_num_wide(CsrView A, CsrView B, int32_t words, int32_t vcap, uint32_t sum_off, 
     bool row_bad = false;
     int total;
     if (sparse) {
-      wide_set_bits<true>(A, B, pa, pe, lng, walk, bits, sum, words, bad);
+      wide_set_bits<BLOCK, true, false>(A, B, none, pa, pe, lng, walk, bits, sum, words, bad);
       // ordered list of touched words: summary words in order, bits in order,
       // in rounds of blockDim summary words
       int L = 0;
@@ -671,7 +769,7 @@ k_num_wide(CsrView A, CsrView B, int32_t words, int32_t vcap, uint32_t sum_off, 
       if (sl >= 0) {  // the symbolic phase kept this row's bits
         // kKeepU 16-byte pieces per thread in flight at once; read once, so
         // streamed past L2
-        const uint4* src = reinterpret_cast<const uint4*>(keep.bits + (size_t)sl * words);
+        const uint4* src = reinterpret_cast<const uint4*>(keep.bits + (size_t)sl * keep.stride);
         uint4* dst4 = reinterpret_cast<uint4*>(bits);
         const int n4 = words >> 2;
         for (int v0 = threadIdx.x; v0 < n4; v0 += blockDim.x * kKeepU) {
@@ -689,7 +787,7 @@ k_num_wide(CsrView A, CsrView B, int32_t words, int32_t vcap, uint32_t sum_off, 
         }
         __syncthreads();
       } else {
-        wide_set_bits<false>(A, B, pa, pe, lng, walk, bits, sum, words, bad);
+        wide_set_bits<BLOCK, false, false>(A, B, none, pa, pe, lng, walk, bits, sum, words, bad);
       }
       const int wpw = words / nwarps_blk;  // words per warp (words is a multiple of 32 * 32)
       const int w0 = warp * wpw;
@@ -764,11 +862,11 @@ k_num_wide(CsrView A, CsrView B, int32_t words, int32_t vcap, uint32_t sum_off, 
       }
     };
     if (sparse) {
-      if (lng) wide_walk_long<true>(A, B, pa, pe, walk.ls, lng, bad, add_smem, nullptr, nullptr, i);
-      else wide_walk<true>(A, B, pa, pe, walk.ws, bad, add_smem, i);
+      if (lng) wide_walk_long<BLOCK, true, false>(A, B, none, pa, pe, walk.ls, lng, bad, add_smem, nullptr, nullptr, i);
+      else wide_walk<BLOCK, true, false>(A, B, none, pa, pe, walk.ws, bad, add_smem, i);
     } else {
-      if (lng) wide_walk_long<true>(A, B, pa, pe, walk.ls, lng, bad, add_glob, nullptr, nullptr, i);
-      else wide_walk<true>(A, B, pa, pe, walk.ws, bad, add_glob, i);
+      if (lng) wide_walk_long<BLOCK, true, false>(A, B, none, pa, pe, walk.ls, lng, bad, add_glob, nullptr, nullptr, i);
+      else wide_walk<BLOCK, true, false>(A, B, none, pa, pe, walk.ws, bad, add_glob, i);
     }
     if (sparse) {
       for (int e = threadIdx.x; e < cnt; e += blockDim.x) c_vals[off + e] = vals[e];
@@ -786,20 +884,280 @@ k_num_wide(CsrView A, CsrView B, int32_t words, int32_t vcap, uint32_t sum_off, 
   if (mismatch) set_status(status, KK_ERR_STRUCTURE_MISMATCH);
 }
 
-// Dynamic shared memory available to the wide kernels (their static arrays
-// take the rest of the opt-in limit).
-size_t wide_budget(const LaunchCtx& ctx) {
-  const size_t stat = sizeof(WideWalkSmem) + 33 * sizeof(int) + 512;
-  return (size_t)ctx.max_smem_optin > stat ? (size_t)ctx.max_smem_optin - stat : 0;
+// ---------------------------------------------------------------------------
+// Chunk tasks: the numeric phase of rows whose bits the symbolic phase kept.
+//
+// A row is cut into chunks of consecutive columns with at most kChunkSlots
+// columns of C each (and at most kChunkWords words of the bit vector, so that a
+// column's offset fits 16 bits); a CTA of 256 threads computes one chunk.  The
+// chunk's bits, ranks, values and columns fit 55 KB of shared memory whatever
+// the row, so four CTAs share an SM and cover each other's barriers and loads.
+// Every A entry's part of the chunk is a consecutive piece of its B row; chunks
+// end at multiples of 2^shift columns, where an index of B's longer rows gives
+// the piece's bounds without a search (k_index_fill).  The pieces' products are
+// walked flattened, a run of consecutive ones per warp, and added with a
+// compare-and-swap loop around one fma (in no fixed order).
+// What bounds it: the shared-memory data path (78% busy, 35 wavefronts per 32
+// products) and the float64 pipe, on which an instruction costs a warp the same
+// with one lane as with 32.  atomicAdd(double) needs a product and an addition
+// per try where this loop needs one fma: 22.6 -> 21.0 ms for the 2.85e9 products
+// of the scale-18 R-MAT square.  The kernel that this one replaces there (a CTA
+// of 1,024 threads per row and SM, atomics in shared memory or in C, the bits
+// walked again) took 26.3 ms, on scale 15 2.8 ms where this takes 0.7.  Without
+// atomics it was slower: one piece at a time (distinct columns) with a barrier
+// each 48 ms, or in a warp's own smaller chunk 46 ms (pieces of 35 products on
+// the heaviest rows, and a full instruction for each); rounds of 512 products
+// with tags against clashes 30 to 39 ms (the pieces of a chunk share columns, so
+// half of the products clash).  128 threads per chunk 25.7 ms, 512 threads 26.
+// ---------------------------------------------------------------------------
+constexpr int kChunkThreads = 256;
+constexpr int kChunkU = 2;  // steps of 32 products whose loads are issued together
+struct ChunkSmem {
+  double vals[kChunkSlots + 2];
+  uint4 bits[kChunkWords / 4];
+  uint4 pre[kChunkWords / 8];  // u16 per word: columns before it
+  int4 piece[kChunkThreads];   // first B entry, length, A value
+  int start[kChunkThreads + 32];
+  uint16_t cols[kChunkSlots + 2];
+  long long tmp[33];
+  int task;
+};
+
+// *v = fma(x, y, *v) in shared memory, bounded retries (false: they ran out).
+__device__ __forceinline__ bool f64_atomic_fma(double* v, double x, double y) {
+  unsigned long long* p = reinterpret_cast<unsigned long long*>(v);
+  unsigned long long old = *reinterpret_cast<volatile unsigned long long*>(p);
+  for (int it = 0; it < kCasRetryLimit; ++it) {
+    const unsigned long long seen =
+        atomicCAS(p, old, (unsigned long long)__double_as_longlong(fma(x, y, __longlong_as_double((long long)old))));
+    if (seen == old) return true;
+    old = seen;
+  }
+  return false;
 }
 
-int wide_grid(const LaunchCtx& ctx, size_t smem, int nrows) {
+// First entry of the sorted B row [lo, hi) whose column is >= key.
+__device__ __forceinline__ int chunk_bound(const int32_t* __restrict__ col, int lo, int hi, int key) {
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (col[mid] < key) lo = mid + 1;
+    else hi = mid;
+  }
+  return lo;
+}
+
+// Index of B's rows of at least kIndexMinLen entries: their numbers (slot of
+// row j, -1 for a short one; row of a slot), then the position of every
+// multiple of 2^shift columns in each of them.
+__global__ void __launch_bounds__(256)
+k_index_rows(int32_t m, const int32_t* __restrict__ rowptr, int32_t max_slots, int32_t* __restrict__ slot,
+             int32_t* __restrict__ row, int32_t* __restrict__ count) {
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < m; j += gridDim.x * blockDim.x) {
+    int s = -1;
+    if (rowptr[j + 1] - rowptr[j] >= kIndexMinLen) {
+      s = atomicAdd(count, 1);
+      if (s < max_slots) row[s] = j;
+      else s = -1;
+    }
+    slot[j] = s;
+  }
+}
+
+__global__ void __launch_bounds__(256)
+k_index_fill(CsrView B, int32_t shift, int32_t stride, int32_t max_slots, const int32_t* __restrict__ row,
+             const int32_t* __restrict__ count, int32_t* __restrict__ tab) {
+  const long long n = (long long)min(*count, max_slots) * stride;
+  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n;
+       e += (long long)gridDim.x * blockDim.x) {
+    const int s = (int)(e / stride), g = (int)(e - (long long)s * stride);
+    const int j = row[s];
+    const long long key = (long long)g << shift;
+    const int lo = B.rowptr[j], hi = B.rowptr[j + 1];
+    tab[e] = key > 0x7fffffff ? hi : chunk_bound(B.colind, lo, hi, (int)key);
+  }
+}
+
+__global__ void __launch_bounds__(kChunkThreads, 1024 / kChunkThreads)
+k_num_chunk(CsrView A, CsrView B, int32_t words, const int64_t* __restrict__ c_rowptr,
+            int32_t* __restrict__ c_colind, double* __restrict__ c_vals, WideKeep keep, int* status) {
+  extern __shared__ __align__(16) unsigned char wsm[];
+  ChunkSmem& sm = *reinterpret_cast<ChunkSmem*>(wsm);
+  const uint32_t* bits = reinterpret_cast<const uint32_t*>(sm.bits);
+  const uint16_t* pre = reinterpret_cast<const uint16_t*>(sm.pre);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int32_t* __restrict__ bcol = B.colind;
+  const double* __restrict__ bval = B.vals;
+  const int ntasks = min(keep.next[1], keep.max_tasks);
+  int mismatch = 0;
+  bool ok = true;
+  for (;;) {
+    __syncthreads();  // the last task's shared memory is free
+    if (tid == 0) sm.task = atomicAdd(keep.next + 2, 1);
+    __syncthreads();
+    const int t = sm.task;
+    if (t >= ntasks) break;
+    const int2 task = keep.tasks[t];
+    const int i = task.x;
+    if (i < 0) continue;
+    const uint32_t* row_bits = keep.bits + (size_t)keep.slot[i] * keep.stride;
+    const int2* end = reinterpret_cast<const int2*>(row_bits + words);
+    const int2 beg = task.y > 0 ? end[task.y - 1] : make_int2(0, 0), fin = end[task.y];
+    const int nw4 = (fin.x - beg.x) >> 2, n = fin.y - beg.y;
+    const int64_t off = c_rowptr[i] + beg.y;
+    const bool last = fin.x >= words;
+    if (n <= 0 || n > kChunkSlots || off + n > c_rowptr[i + 1] || (last && off + n != c_rowptr[i + 1])) {
+      if (n != 0) mismatch = 1;
+      continue;
+    }
+    const int c0 = beg.x * 32, c1 = fin.x * 32;
+    const uint4* src = reinterpret_cast<const uint4*>(row_bits + beg.x);
+    for (int q = tid; q < nw4; q += kChunkThreads) sm.bits[q] = __ldcs(&src[q]);
+    for (int e = tid; e < n; e += kChunkThreads) sm.vals[e] = 0.0;
+    __syncthreads();
+    for (int q0 = 0, run = 0; q0 < nw4; q0 += 2 * kChunkThreads) {  // columns before every word: 8 words a thread
+      const int q = q0 + 2 * tid;
+      const uint4 v = q < nw4 ? sm.bits[q] : make_uint4(0u, 0u, 0u, 0u);
+      const uint4 w = q + 1 < nw4 ? sm.bits[q + 1] : make_uint4(0u, 0u, 0u, 0u);
+      const int p1 = __popc(v.x), p2 = p1 + __popc(v.y), p3 = p2 + __popc(v.z), p4 = p3 + __popc(v.w);
+      const int p5 = p4 + __popc(w.x), p6 = p5 + __popc(w.y), p7 = p6 + __popc(w.z), p8 = p7 + __popc(w.w);
+      long long tot;
+      const unsigned b = (unsigned)(run + (int)block_exscan<long long>(p8, sm.tmp, &tot));
+      if (q < nw4)
+        sm.pre[q >> 1] = make_uint4(b | ((b + p1) << 16), (b + p2) | ((b + p3) << 16), (b + p4) | ((b + p5) << 16),
+                                    (b + p6) | ((b + p7) << 16));
+      run += (int)tot;
+      if (q0 + 2 * kChunkThreads >= nw4 && run != n) mismatch = 1;
+    }
+    const uint32_t wmax = (uint32_t)(nw4 * 4 - 1);
+    // slot of column c (a spare one for a column outside the kept bits)
+    auto slot_of = [&](int c) -> int {
+      const uint32_t o = (uint32_t)(c - c0), w = min(o >> 5, wmax);
+      const uint32_t m = bits[w], bit = 1u << (o & 31);
+      const bool member = (o >> 5) == w && (m & bit) != 0u;
+      if (!member) mismatch = 1;
+      const int s = member ? min((int)pre[w] + __popc(m & (bit - 1u)), kChunkSlots) : kChunkSlots;
+      sm.cols[s] = (uint16_t)o;
+      return s;
+    };
+    const int pa = A.rowptr[i], pe = A.rowptr[i + 1];
+    for (int p0 = pa; p0 < pe; p0 += kChunkThreads) {
+      const int p = p0 + tid;
+      int s = 0, len = 0;
+      double a = 0.0;
+      if (p < pe) {
+        const int j = A.colind[p];
+        const int bs = B.rowptr[j], be = B.rowptr[j + 1], x = keep.bidx[j];
+        const int32_t* tab = keep.btab + (size_t)(x < 0 ? 0 : x) * keep.tab_stride;
+        s = beg.x == 0 ? bs : x >= 0 ? tab[c0 >> keep.shift] : chunk_bound(bcol, bs, be, c0);
+        len = (last ? be : x >= 0 ? tab[c1 >> keep.shift] : chunk_bound(bcol, s, be, c1)) - s;
+        a = a_value(A, i, p);
+      }
+      long long tot;
+      const long long ex = block_exscan<long long>(len > 0 ? (1ll << 40) + len : 0ll, sm.tmp, &tot);
+      const int total = (int)(tot & ((1ll << 40) - 1)), np = (int)(tot >> 40);
+      if (len > 0) {
+        const int k = (int)(ex >> 40), f = (int)(ex & ((1ll << 40) - 1));
+        sm.start[k] = f;
+        sm.piece[k] = make_int4(s - f, 0, __double2loint(a), __double2hiint(a));
+      }
+      if (tid == 0) sm.start[np] = 0x7fffffff;
+      __syncthreads();
+      if (total == 0) continue;
+      // every warp takes a run of consecutive products
+      const int per = (total + kChunkThreads - 1) / kChunkThreads * 32;
+      const int f_lo = min(warp * per, total), f_hi = min(f_lo + per, total);
+      int seen = 0;  // pieces that start before the next step's first product
+      for (int k = 0; k < np; k += 32) {
+        const unsigned m = __ballot_sync(kFull, sm.start[min(k + lane, np)] < f_lo);
+        seen += __popc(m);
+        if (m != kFull) break;
+      }
+      for (int f = f_lo; f < f_hi; f += 32 * kChunkU) {
+        int c[kChunkU];
+        double x[kChunkU], y[kChunkU];
+#pragma unroll
+        for (int u = 0; u < kChunkU; ++u) {
+          const int fb = f + u * 32;
+          const unsigned at = (unsigned)(sm.start[min(seen + lane, np)] - fb);
+          const unsigned m = __reduce_or_sync(kFull, at < 32u ? 1u << at : 0u);
+          const int own = min(seen + __popc(m & (0xffffffffu >> (31 - lane))) - 1, np - 1);
+          seen += __popc(m);
+          const int4 in = sm.piece[own];
+          const int q = in.x + min(fb + lane, f_hi - 1);
+          c[u] = bcol[q];
+          y[u] = bval[q];
+          x[u] = __hiloint2double(in.w, in.z);
+        }
+#pragma unroll
+        for (int u = 0; u < kChunkU; ++u)
+          if (f + u * 32 + lane < f_hi) ok &= f64_atomic_fma(&sm.vals[slot_of(c[u])], x[u], y[u]);
+      }
+      __syncthreads();
+    }
+    __syncthreads();
+    // written once and larger than L2 as a whole: streamed past it
+    for (int e = tid; e < n; e += kChunkThreads) {
+      __stcs(&c_colind[off + e], c0 + (int)sm.cols[e]);
+      __stcs(&c_vals[off + e], sm.vals[e]);
+    }
+  }
+  if (mismatch) set_status(status, KK_ERR_STRUCTURE_MISMATCH);
+  if (!ok) set_status(status, KK_ERR_TIMEOUT);
+}
+
+// Dynamic shared memory available to the wide kernels of BLOCK threads (their
+// static arrays take the rest of the opt-in limit).
+template <int BLOCK>
+size_t wide_static() {
+  return sizeof(WideWalkSmem<BLOCK>) + 33 * sizeof(int) + 512;
+}
+size_t wide_budget(const LaunchCtx& ctx) {
+  return (size_t)ctx.max_smem_optin > wide_static<kWideBlock>() ? (size_t)ctx.max_smem_optin - wide_static<kWideBlock>()
+                                                                : 0;
+}
+
+int wide_per_sm(const LaunchCtx& ctx, size_t smem, int block) {
   int per_sm = (int)(((size_t)ctx.max_smem_optin + 1024) / (smem + 1024));
   if (per_sm < 1) per_sm = 1;
-  if (per_sm > 2048 / kWideBlock) per_sm = 2048 / kWideBlock;
-  long long g = (long long)ctx.num_sms * per_sm;
-  if (g > nrows) g = nrows;
-  return (int)(g < 1 ? 1 : g);
+  return per_sm > 2048 / block ? 2048 / block : per_sm;
+}
+
+// CTA size of a wide kernel: rows of a few thousand products do not feed 1,024
+// threads (two thirds of their time went to barriers), so they take the
+// smallest CTAs of which an SM still holds 1,024 threads.
+int wide_block(const LaunchCtx& ctx, size_t dyn, bool light) {
+  if (light && wide_per_sm(ctx, dyn + wide_static<256>(), 256) >= 4) return 256;
+  if (light && wide_per_sm(ctx, dyn + wide_static<512>(), 512) >= 2) return 512;
+  return kWideBlock;
+}
+
+template <int BLOCK, bool PAIRS>
+cudaError_t sym_wide(const LaunchCtx& ctx, const CsrView& A, const CsrView& B, const BComp& bc, int words,
+                     const WideGeom& g, uint32_t stage_off, size_t bytes, const long long* flop,
+                     const int32_t* rows, int32_t nrows, int32_t* cnt) {
+  auto kern = k_sym_wide<BLOCK, PAIRS>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e != cudaSuccess) return e;
+  long long grid = (long long)ctx.num_sms * wide_per_sm(ctx, bytes + wide_static<BLOCK>(), BLOCK);
+  if (grid > nrows) grid = nrows;
+  kern<<<(int)grid, BLOCK, bytes, ctx.stream>>>(A, B, bc, words, (uint32_t)g.sum_off, stage_off, flop, rows, nrows,
+                                                cnt, ctx.keep, ctx.status);
+  return cudaGetLastError();
+}
+
+template <int BLOCK>
+cudaError_t num_wide(const LaunchCtx& ctx, const CsrView& A, const CsrView& B, int words, const WideGeom& g,
+                     const int64_t* c_rowptr, const int32_t* rows, int32_t nrows, int32_t* c_colind,
+                     double* c_vals) {
+  auto kern = k_num_wide<BLOCK>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.bytes);
+  if (e != cudaSuccess) return e;
+  long long grid = (long long)ctx.num_sms * wide_per_sm(ctx, g.bytes + wide_static<BLOCK>(), BLOCK);
+  if (grid > nrows) grid = nrows;
+  kern<<<(int)grid, BLOCK, g.bytes, ctx.stream>>>(A, B, words, g.vcap, (uint32_t)g.sum_off, (uint32_t)g.reg_off,
+                                                  (uint32_t)g.val_off, c_rowptr, ctx.flop, rows, nrows, c_colind,
+                                                  c_vals, ctx.keep, ctx.status);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -822,9 +1180,30 @@ bool wide_numeric_fits(const LaunchCtx& ctx, int32_t k) {
   return g.val_off <= wide_budget(ctx) && g.vcap >= 64;
 }
 
+int32_t wide_chunk_shift(int32_t k) { return chunk_shift(k); }
+int32_t wide_max_chunks(int32_t k) { return k / chunk_cols(k) + wide_words(k) / kChunkWords + 2; }
+long long wide_max_tasks(int32_t k, long long flops, long long slots) {
+  // a chunk ends with every chunk_cols columns (a column has a product) and at
+  // fixed words
+  return flops / chunk_cols(k) + slots * (wide_words(k) / kChunkWords + 2);
+}
+int32_t wide_index_stride(int32_t k) { return (wide_words(k) * 32 >> chunk_shift(k)) + 1; }
+int32_t wide_index_slots(const CsrView& B) { return B.nnz / kIndexMinLen + 1; }
+
+cudaError_t launch_chunk_index(const LaunchCtx& ctx, const CsrView& B, int32_t* slot, int32_t* row, int32_t* tab) {
+  const int slots = wide_index_slots(B), stride = wide_index_stride(B.n);
+  timer_begin(ctx.timer, ctx.stream, "chunk_index");
+  k_index_rows<<<min(ctx.num_sms * 8, (B.m + 255) / 256), 256, 0, ctx.stream>>>(B.m, B.rowptr, slots, slot, row,
+                                                                            ctx.keep.next + 3);
+  k_index_fill<<<ctx.num_sms * 8, 256, 0, ctx.stream>>>(B, chunk_shift(B.n), stride, slots, row, ctx.keep.next + 3,
+                                                       tab);
+  timer_end(ctx.timer, ctx.stream);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_symbolic_wide(const LaunchCtx& ctx, const CsrView& A, const CsrView& B,
                                  const long long* flop, const int32_t* rows, int32_t nrows,
-                                 int32_t* cnt) {
+                                 int32_t* cnt, bool light) {
   if (nrows <= 0) return cudaSuccess;
   const int words = wide_words(B.n);
   const WideGeom g = wide_geom(words, wide_budget(ctx), false);
@@ -837,25 +1216,49 @@ cudaError_t launch_symbolic_wide(const LaunchCtx& ctx, const CsrView& A, const C
   if (ctx.stage_long_rows && ((uintptr_t)B.colind & 15) == 0 && st_off + stage_bytes <= wide_budget(ctx) - 1024) {
     stage_off = (uint32_t)st_off;
     bytes = st_off + stage_bytes;
+    return sym_wide<kWideBlock, false>(ctx, A, B, ctx.bcomp, words, g, stage_off, bytes, flop, rows, nrows, cnt);
   }
-  cudaError_t e = cudaFuncSetAttribute(k_sym_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e != cudaSuccess) return e;
-  k_sym_wide<<<wide_grid(ctx, bytes, nrows), kWideBlock, bytes, ctx.stream>>>(
-      A, B, words, (uint32_t)g.sum_off, stage_off, flop, rows, nrows, cnt, ctx.keep, ctx.status);
-  return cudaGetLastError();
+  const int block = wide_block(ctx, bytes, light);
+#define KK_SYM_WIDE(BL)                                                                                      \
+  return ctx.bcomp.bc ? sym_wide<BL, true>(ctx, A, B, ctx.bcomp, words, g, 0, bytes, flop, rows, nrows, cnt) \
+                      : sym_wide<BL, false>(ctx, A, B, ctx.bcomp, words, g, 0, bytes, flop, rows, nrows, cnt)
+  if (block == 256) KK_SYM_WIDE(256);
+  if (block == 512) KK_SYM_WIDE(512);
+  KK_SYM_WIDE(kWideBlock);
+#undef KK_SYM_WIDE
 }
 
 cudaError_t launch_numeric_wide(const LaunchCtx& ctx, const CsrView& A, const CsrView& B,
                                 const int64_t* c_rowptr, const int32_t* rows, int32_t nrows,
-                                int32_t* c_colind, double* c_vals) {
+                                int32_t* c_colind, double* c_vals, long long max_nnz) {
   if (nrows <= 0) return cudaSuccess;
   const int words = wide_words(B.n);
-  const WideGeom g = wide_geom(words, wide_budget(ctx), true);
-  cudaError_t e = cudaFuncSetAttribute(k_num_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.bytes);
+  const size_t budget = wide_budget(ctx);
+  WideGeom g = wide_geom(words, budget, true);
+  const bool light = max_nnz <= g.vcap;  // every row of the bin fits: no more slots than it needs
+  if (light) g = wide_geom(words, g.val_off + (size_t)max_nnz * 8 < budget ? g.val_off + (size_t)max_nnz * 8 : budget, true);
+  const int block = wide_block(ctx, g.bytes, light);
+  if (block == 256) return num_wide<256>(ctx, A, B, words, g, c_rowptr, rows, nrows, c_colind, c_vals);
+  if (block == 512) return num_wide<512>(ctx, A, B, words, g, c_rowptr, rows, nrows, c_colind, c_vals);
+  return num_wide<kWideBlock>(ctx, A, B, words, g, c_rowptr, rows, nrows, c_colind, c_vals);
+}
+
+cudaError_t launch_num_chunk(const LaunchCtx& ctx, const CsrView& A, const CsrView& B, const int64_t* c_rowptr,
+                             int32_t* c_colind, double* c_vals) {
+  cudaError_t e = cudaFuncSetAttribute(k_num_chunk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ChunkSmem));
   if (e != cudaSuccess) return e;
-  k_num_wide<<<wide_grid(ctx, g.bytes, nrows), kWideBlock, g.bytes, ctx.stream>>>(
-      A, B, words, g.vcap, (uint32_t)g.sum_off, (uint32_t)g.reg_off, (uint32_t)g.val_off, c_rowptr,
-      ctx.flop, rows, nrows, c_colind, c_vals, ctx.keep, ctx.status);
+  e = cudaMemsetAsync(ctx.keep.next + 2, 0, sizeof(int32_t), ctx.stream);
+  if (e != cudaSuccess) return e;
+  timer_begin(ctx.timer, ctx.stream, "num_chunk");
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_num_chunk, kChunkThreads, sizeof(ChunkSmem)) != cudaSuccess ||
+      per_sm < 1) {
+    (void)cudaGetLastError();
+    per_sm = 1;
+  }
+  k_num_chunk<<<ctx.num_sms * per_sm, kChunkThreads, sizeof(ChunkSmem), ctx.stream>>>(A, B, wide_words(B.n), c_rowptr, c_colind,
+                                                                         c_vals, ctx.keep, ctx.status);
+  timer_end(ctx.timer, ctx.stream);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,64 @@
+"""GPU: chunked numeric phase of the wide tier's kept rows, at the edges of its
+chunks, of B's index and of the kept-row budget, against the oracle."""
+import numpy as np
+import pytest
+
+from oracle import jacobi as OJ
+from paper_2103_11991_gb300 import inputs as I
+from tests._gpu import check_against_oracle, run_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+# k: one to three 2,048-word parts of the bit vector, either side of the width
+# at which chunks end at coarser columns; lens: B rows without and with an index
+@pytest.mark.parametrize("k", [1500, 65536, 65537, 131072, 262144, 262145, 300000])
+@pytest.mark.parametrize("la,lb", [((30, 60), (40, 127)), ((4, 9), (500, 1400)), ((260, 300), (5, 40))])
+def test_chunks_match_oracle(k, la, lb):
+    n = 700
+    A = I.random_rows(60, n, *la, seed=k + la[0], purpose="chA")
+    B = I.random_rows(n, k, *lb, seed=k + lb[0], purpose="chB")
+    kept = run_gpu(A, B, force_tier=2, arith=1)
+    check_against_oracle(A, B, *kept[:3])
+    rebuilt = run_gpu(A, B, force_tier=2, arith=1, structure_cache=0)
+    assert np.array_equal(kept[0], rebuilt[0]) and np.array_equal(kept[1], rebuilt[1])
+    few = run_gpu(A, B, force_tier=2, arith=1, wide_cache_mb=1)
+    check_against_oracle(A, B, *few[:3])
+
+
+@pytest.mark.parametrize("count", [1024, 1025, 3071, 3072, 3073, 3584, 3585, 20000])
+def test_dense_columns_at_chunk_ends(count):
+    # neighbouring columns: every group of columns is full, chunks end between them
+    k = 70000
+    lens = np.array([count, count // 2, 7])
+    cols = np.concatenate([np.arange(count), np.arange(count // 2) * 2, np.arange(7) * 100]) + 300
+    B = I.ensure_csr(3, k, np.concatenate([[0], np.cumsum(lens)]), cols, I.uniform01(count, "ch.b", int(lens.sum())))
+    A = I.ensure_csr(4, 3, [0, 3, 5, 6, 9], [0, 1, 2, 0, 2, 0, 2, 1, 0], I.uniform01(count, "ch.a", 9) - 0.5)
+    rp, ci, va, _, _ = run_gpu(A, B, force_tier=2)
+    check_against_oracle(A, B, rp, ci, va)
+
+
+def test_chunks_refresh_other_arrays_and_jacobi():
+    import torch
+    from paper_2103_11991_gb300 import spgemm as K
+    A = I.with_diagonal(I.random_rows(500, 500, 30, 60, seed=3, purpose="chJ"), 4)
+    B = I.random_rows(500, 90000, 80, 200, seed=5, purpose="chK")
+    dA, dB = K.DeviceCSR.from_host(A), K.DeviceCSR.from_host(B)
+    with K.SpGEMM(force_tier=2) as op:
+        rp, nnz = op.symbolic(dA, dB)
+        for seed in (6, 7):  # new values on the kept structure
+            B.vals = I.uniform01(seed, "ch.v", B.nnz) - 0.5
+            dB.vals.copy_(torch.from_numpy(B.vals).cuda())
+            ci, va = op.numeric(dA, dB, rp, nnz)
+            op.sync()
+            check_against_oracle(A, B, rp.cpu().numpy(), ci.cpu().numpy(), va.cpu().numpy())
+        ci, va = op.jacobi_numeric(dA, dB, rp, nnz, 2.0 / 3.0)
+        op.sync()
+        ref = OJ.jacobi_spgemm(A, B, 2.0 / 3.0)
+        assert np.array_equal(ci.cpu().numpy(), ref.colind)
+        assert np.all(np.abs(va.cpu().numpy() - ref.vals) <= 1e-12 * OJ.jacobi_abs(A, B, 2.0 / 3.0))
+        # the same matrices in other arrays: nothing kept is used
+        dB2 = K.DeviceCSR(B.m, B.n, dB.rowptr.clone(), dB.colind.clone(), dB.vals.clone())
+        ci, va = op.numeric(dA, dB2, rp, nnz)
+        op.sync()
+        check_against_oracle(A, B, rp.cpu().numpy(), ci.cpu().numpy(), va.cpu().numpy())
