@@ -19,10 +19,14 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-template <int T, int U>
+// Rows of more than kLongRow entries are put on lr's list by teams of less than
+// a warp and walked by a second launch, a warp per listed row (LISTED): the
+// longest rows of a power-law graph kept single teams busy long after the others
+// had finished (0.95 ms for the scale-18 R-MAT graph's 3.9e6 entries).
+template <int T, int U, bool LISTED>
 __global__ void __launch_bounds__(256, 6)
 k_analyze_b(CsrView B, int32_t* sorted_flag, int* status, int2* __restrict__ bc,
-            int32_t* __restrict__ len, unsigned long long* pairs) {
+            int32_t* __restrict__ len, unsigned long long* pairs, LongRows lr) {
   const int lane = threadIdx.x & 31;
   const int tl = lane & (T - 1);
   const int tbase = lane & ~(T - 1);
@@ -33,26 +37,61 @@ k_analyze_b(CsrView B, int32_t* sorted_flag, int* status, int2* __restrict__ bc,
   int unsorted = 0, bad = 0;
   unsigned long long tot = 0;
   if (team0 == 0 && tl == 0 && B.rowptr[0] != 0) bad = 1;
-  long long r = team0;
-  int bs_n = 0, be_n = 0;
-  if (r < B.m) {
-    bs_n = B.rowptr[r];
-    be_n = B.rowptr[r + 1];
+  const int nrows = LISTED ? min(*lr.count, lr.most) : B.m;
+  long long t = team0;
+  int r_n = 0, bs_n = 0, be_n = 0;
+  if (t < nrows) {
+    r_n = LISTED ? lr.rows[t] : (int)t;
+    bs_n = B.rowptr[r_n];
+    be_n = B.rowptr[r_n + 1];
   }
-  for (; r < B.m; r += nteams) {
-    const int bs = bs_n, be = be_n;
-    if (r + nteams < B.m) {  // next row's bounds in flight while this row is walked
-      bs_n = B.rowptr[r + nteams];
-      be_n = B.rowptr[r + nteams + 1];
+  for (; t < nrows; t += nteams) {
+    const int r = r_n, bs = bs_n, be = be_n;
+    if (t + nteams < nrows) {  // next row's bounds in flight while this row is walked
+      r_n = LISTED ? lr.rows[t + nteams] : (int)(t + nteams);
+      bs_n = B.rowptr[r_n];
+      be_n = B.rowptr[r_n + 1];
     }
     if (bs < 0 || be < bs || be > B.nnz) {
       bad = 1;
       continue;
     }
+    if (!LISTED && lr.rows && be - bs > kLongRow) {
+      int at = 0;
+      if (tl == 0) at = atomicAdd(lr.count, 1);
+      at = __shfl_sync(mask, at, 0, T);
+      if (at < lr.most) {
+        if (tl == 0) lr.rows[at] = r;
+        continue;
+      }
+    }
     int cw = -1, n = 0;
     uint32_t cm = 0u;
     int prev = 0;  // last column of the previous chunk
-    for (int qb = bs; qb < be; qb += T * U) {
+    if constexpr (T == 1) {
+      // a thread per row: no lanes to combine (shuffles under single-lane masks
+      // run lane after lane: 91 us for a prolongator's 2.1e6 rows, now 14)
+      for (int qb = bs; qb < be; qb += U) {
+        int cu[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) cu[u] = qb + u < be ? B.colind[qb + u] : 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          if (qb + u < be) {
+            const int c = cu[u], w = c >> 5;
+            if ((unsigned)c >= (unsigned)B.n) bad = 1;
+            if (qb + u > bs && prev >= c) unsorted = 1;
+            prev = c;
+            if (w != cw) {
+              if (bc && cm) bc[bs + n++] = make_int2(cw, (int)cm);
+              cw = w;
+              cm = 0u;
+            }
+            cm |= 1u << (c & 31);
+          }
+        }
+      }
+    } else for (int qb = bs; qb < be; qb += T * U) {
       int cu[U];  // the columns of U chunks, loaded together
 #pragma unroll
       for (int u = 0; u < U; ++u) {
@@ -89,7 +128,8 @@ k_analyze_b(CsrView B, int32_t* sorted_flag, int* status, int2* __restrict__ bc,
         const uint32_t acc0 = __shfl_sync(mask, acc, 0, T);
         const bool cont0 = __shfl_sync(mask, (int)(valid && !head), 0, T) != 0;
         if (cont0) cm |= acc0;
-        const unsigned hm = (__ballot_sync(mask, head) >> tbase) & ((1u << T) - 1u);
+        unsigned hm = __ballot_sync(mask, head);
+        if constexpr (T < 32) hm = (hm >> tbase) & ((1u << T) - 1u);
         if (hm) {
           // a new word started: the carried pair is complete
           if (cm) {
@@ -129,32 +169,35 @@ k_analyze_b(CsrView B, int32_t* sorted_flag, int* status, int2* __restrict__ bc,
 
 }  // namespace
 
-template <int T, int U>
+template <int T, int U, bool LISTED = false>
 static cudaError_t analyze_b_tu(const LaunchCtx& ctx, const CsrView& B, int32_t* sorted_flag,
-                                int2* bc, int32_t* len, unsigned long long* pairs) {
+                                int2* bc, int32_t* len, unsigned long long* pairs, const LongRows& lr) {
   // one resident wave: the kernel strides over rows, so blocks beyond what the
   // SMs hold at once would only start late
   static int per_sm = 0;
   if (per_sm == 0 &&
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_analyze_b<T, U>, 256, 0) != cudaSuccess) {
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_analyze_b<T, U, LISTED>, 256, 0) != cudaSuccess) {
     (void)cudaGetLastError();
     per_sm = 4;
   }
-  long long blocks = ((long long)B.m * T + 255) / 256;
+  long long blocks = ((long long)(LISTED ? lr.most : B.m) * T + 255) / 256;
   const long long cap = (long long)ctx.num_sms * (per_sm > 0 ? per_sm : 1);
   if (blocks > cap) blocks = cap;
   if (blocks < 1) blocks = 1;
-  k_analyze_b<T, U><<<(int)blocks, 256, 0, ctx.stream>>>(B, sorted_flag, ctx.status, bc, len, pairs);
+  k_analyze_b<T, U, LISTED><<<(int)blocks, 256, 0, ctx.stream>>>(B, sorted_flag, ctx.status, bc, len, pairs, lr);
   return cudaGetLastError();
 }
 
 cudaError_t launch_analyze_b(const LaunchCtx& ctx, const CsrView& B, int32_t* sorted_flag,
-                             int2* bc, int32_t* len, unsigned long long* pairs) {
+                             int2* bc, int32_t* len, unsigned long long* pairs, const LongRows& lr) {
   if (B.m <= 0) return cudaSuccess;
   const long long avg = (long long)B.nnz / B.m;
-  if (avg <= 2) return analyze_b_tu<1, 2>(ctx, B, sorted_flag, bc, len, pairs);
-  if (avg <= 8) return analyze_b_tu<4, 2>(ctx, B, sorted_flag, bc, len, pairs);
-  return analyze_b_tu<8, 4>(ctx, B, sorted_flag, bc, len, pairs);
+  cudaError_t e;
+  if (avg <= 2) e = analyze_b_tu<1, 2>(ctx, B, sorted_flag, bc, len, pairs, lr);
+  else if (avg <= 8) e = analyze_b_tu<1, 8>(ctx, B, sorted_flag, bc, len, pairs, lr);
+  else e = analyze_b_tu<8, 4>(ctx, B, sorted_flag, bc, len, pairs, lr);
+  if (e != cudaSuccess || !lr.rows) return e;
+  return analyze_b_tu<32, 4, true>(ctx, B, sorted_flag, bc, len, pairs, lr);
 }
 
 }  // namespace kk

@@ -154,12 +154,13 @@ struct BinTable {
 __device__ __forceinline__ uint8_t classify(const BinTable& t, long long q, int flat, int span,
                                             long long flop, int sorted, bool kept) {
   if (q <= 0) return kSkipBin;
-  if (t.mode[0] == 3 && q <= t.hi[0] && flop <= t.thread_flop) return 0;
+  for (int b = 0; t.mode[b] == 3; ++b)
+    if (q <= t.hi[b] && flop <= t.thread_flop) return (uint8_t)b;
   const int sp = sorted ? span : t.cols;
   if (sp > 0) {
     for (int w = 0; w < t.nwin; ++w)
-      if (q <= t.win_q[w] && sp <= t.win_bits[w] && (sorted || t.win_any_order[w]) &&
-          (!t.win_kept[w] || kept) && (long long)t.win_bits[w] <= t.win_ratio[w] * flop)
+      if (q <= t.win_q[w] && sp <= t.win_bits[w] && (sorted || t.win_any_order[w]) && (!t.win_kept[w] || kept) &&
+          (long long)t.win_bits[w] <= (q > kRankMinNnz ? t.win_ratio[w] : (long long)kWindowFlopRatio) * flop)
         return (uint8_t)t.win_bin[w];
   }
   for (int b = 0; b < t.nb; ++b) {
@@ -178,7 +179,8 @@ __device__ __forceinline__ uint8_t classify(const BinTable& t, long long q, int 
 // those of U entries together and the next row's bounds are loaded while a row
 // is processed; T and U follow A's mean row length.  STATS (the learned
 // form): also the longest and shortest referenced B row of each row, to stat.
-template <int T, int U, bool STATS>
+// Long rows are listed for a second launch (LISTED), as in k_analyze_b.
+template <int T, int U, bool STATS, bool LISTED>
 __global__ void __launch_bounds__(256, 6)
 k_analyze_a(CsrView A, const int32_t* __restrict__ brp,
                             const int32_t* __restrict__ bcol, int32_t nb_rows,
@@ -186,31 +188,45 @@ k_analyze_a(CsrView A, const int32_t* __restrict__ brp,
                             int32_t vec_min_len, long long* __restrict__ flop,
                             uint8_t* __restrict__ bin, int32_t* __restrict__ row_lo,
                             int32_t* __restrict__ row_span, int2* __restrict__ stat,
-                            unsigned long long* total_flop, int* status) {
+                            unsigned long long* total_flop, int* status, LongRows lr) {
   const int sorted = *b_sorted;
   const int tl = threadIdx.x % T;
   const unsigned mask = team_mask<T>();
   const long long team0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / T;
   const long long nteams = (long long)gridDim.x * blockDim.x / T;
-  const long long iters = (A.m + nteams - 1) / nteams;
+  const int nrows = LISTED ? min(*lr.count, lr.most) : A.m;
+  const long long iters = (nrows + nteams - 1) / nteams;
   unsigned long long acc = 0;
-  long long r = team0;
-  int pa_n = 0, pe_n = 0;
-  if (r < A.m) {
-    pa_n = A.rowptr[r];
-    pe_n = A.rowptr[r + 1];
+  long long t = team0;
+  int r_n = 0, pa_n = 0, pe_n = 0;
+  if (t < nrows) {
+    r_n = LISTED ? lr.rows[t] : (int)t;
+    pa_n = A.rowptr[r_n];
+    pe_n = A.rowptr[r_n + 1];
   }
-  for (long long it = 0; it < iters; ++it, r += nteams) {
+  for (long long it = 0; it < iters; ++it, t += nteams) {
+    const int r = r_n;
     int pa = pa_n, pe = pe_n;
-    if (r + nteams < A.m) {
-      pa_n = A.rowptr[r + nteams];
-      pe_n = A.rowptr[r + nteams + 1];
+    bool on = t < nrows;
+    if (t + nteams < nrows) {
+      r_n = LISTED ? lr.rows[t + nteams] : (int)(t + nteams);
+      pa_n = A.rowptr[r_n];
+      pe_n = A.rowptr[r_n + 1];
+    }
+    if (!LISTED && on && lr.rows && pe - pa > kLongRow) {
+      int at = 0;
+      if (tl == 0) at = atomicAdd(lr.count, 1);
+      at = __shfl_sync(mask, at, 0, T);
+      if (at < lr.most) {
+        if (tl == 0) lr.rows[at] = r;
+        on = false;
+      }
     }
     long long f = 0;
     int bad = 0;
     int lo = 0x7fffffff, hi = -1;
     int mx = 0, mn = 0x7fffffff;
-    if (r < A.m) {
+    if (on) {
       if (pa < 0 || pe < pa || pe > A.nnz || (r == 0 && pa != 0)) {
         bad = 1;
         pe = pa;
@@ -260,7 +276,7 @@ k_analyze_a(CsrView A, const int32_t* __restrict__ brp,
       }
     }
     if (bad) set_status(status, KK_ERR_BAD_INDEX);
-    if (r < A.m && tl == 0) {
+    if (on && tl == 0) {
       flop[r] = f;
       const long long span = hi >= lo ? (long long)hi - lo + 1 : 0;
       const int sp = span > 0x7fffffff ? 0x7fffffff : (int)span;
@@ -278,11 +294,27 @@ k_analyze_a(CsrView A, const int32_t* __restrict__ brp,
 
 // ---------------------------------------------------------------------------
 // Stable binning: rows grouped by bin id, ascending row order within a bin.
+// Blocks of 2,048 rows: counts per bin and block, one CTA per bin scans its
+// blocks' counts (a single CTA over all bins took 29 us for 2.1e6 rows), and the
+// blocks place their rows.  Blocks whose rows share a bin, the common case, take
+// short cuts in the first and last step.
 // ---------------------------------------------------------------------------
 constexpr int kBinBlock = 256;
 constexpr int kBinPerThread = 8;
 constexpr int kBinRows = kBinBlock * kBinPerThread;
-constexpr int kBinScanPer = 8;  // counts per thread in the bin-offset scan
+
+// The bins of a thread's 8 consecutive rows, packed (kSkipBin past the end).
+__device__ __forceinline__ unsigned long long bin_bytes(const uint8_t* __restrict__ bin, long long r, int32_t m) {
+  if (r + kBinPerThread <= m) return *reinterpret_cast<const unsigned long long*>(bin + r);
+  unsigned long long v = ~0ull;
+  for (int t = 0; t < kBinPerThread && r + t < m; ++t)
+    v = (v & ~(0xFFull << (8 * t))) | (unsigned long long)bin[r + t] << (8 * t);
+  return v;
+}
+// Whether all eight equal the lowest one.
+__device__ __forceinline__ bool bin_uniform(unsigned long long v) {
+  return v == (v & 0xFFull) * 0x0101010101010101ull;
+}
 
 __global__ void __launch_bounds__(kBinBlock)
 k_bin_count(int32_t m, const uint8_t* __restrict__ bin, int32_t nb, int32_t nblk,
@@ -290,11 +322,16 @@ k_bin_count(int32_t m, const uint8_t* __restrict__ bin, int32_t nb, int32_t nblk
   __shared__ int c[kMaxBins];
   if (threadIdx.x < kMaxBins) c[threadIdx.x] = 0;
   __syncthreads();
-  const long long base = (long long)blockIdx.x * kBinRows;
-  for (int t = 0; t < kBinPerThread; ++t) {
-    const long long r = base + t * kBinBlock + threadIdx.x;
-    if (r < m) {
-      const uint8_t b = bin[r];
+  const long long r = (long long)blockIdx.x * kBinRows + (long long)threadIdx.x * kBinPerThread;
+  const unsigned long long v = bin_bytes(bin, r, m);
+  const int b0 = (int)(v & 0xFF);
+  int same = 0;
+  __match_all_sync(0xffffffffu, v, &same);
+  if (same && bin_uniform(v)) {
+    if ((threadIdx.x & 31) == 0 && b0 != kSkipBin) atomicAdd(&c[b0], 32 * kBinPerThread);
+  } else {
+    for (int t = 0; t < kBinPerThread; ++t) {
+      const int b = (int)(v >> (8 * t) & 0xFF);
       if (b != kSkipBin) atomicAdd(&c[b], 1);
     }
   }
@@ -302,65 +339,73 @@ k_bin_count(int32_t m, const uint8_t* __restrict__ bin, int32_t nb, int32_t nblk
   if (threadIdx.x < nb) blk_counts[(long long)threadIdx.x * nblk + blockIdx.x] = c[threadIdx.x];
 }
 
-// Single CTA: exclusive scan (bin-major) of the per-block counts in place;
-// bin_start[b] = first position of bin b, bin_start[nb] = total.
-__global__ void __launch_bounds__(1024)
-k_bin_scan(int32_t nb, int32_t nblk, int32_t* __restrict__ blk, int32_t* __restrict__ bin_start) {
-  // every thread scans kBinScanPer consecutive counts, so one pass of the
-  // 1024-thread block covers 8,192 (bin, block) counts (few barriers)
-  constexpr int P = kBinScanPer;
-  __shared__ int warp_tot[32];
-  __shared__ int carry;
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
-  const long long total = (long long)nb * nblk;
+// CTA b: exclusive scan of bin b's block counts in place, total to tot[b].
+__global__ void __launch_bounds__(kBinBlock)
+k_bin_scan(int32_t nblk, int32_t* __restrict__ blk, int32_t* __restrict__ tot) {
+  constexpr int P = 8;
+  __shared__ int warp_tot[kBinBlock / 32];
+  int32_t* mine = blk + (long long)blockIdx.x * nblk;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (long long c0 = 0; c0 < total; c0 += (long long)blockDim.x * P) {
-    const long long i0 = c0 + (long long)threadIdx.x * P;
-    int v[P];
-    int sum = 0;
+  int carry = 0;
+  for (int c0 = 0; c0 < nblk; c0 += kBinBlock * P) {
+    const int i0 = c0 + threadIdx.x * P;
+    int v[P], sum = 0;
 #pragma unroll
     for (int t = 0; t < P; ++t) {
-      v[t] = i0 + t < total ? blk[i0 + t] : 0;
+      v[t] = i0 + t < nblk ? mine[i0 + t] : 0;
       sum += v[t];
     }
     const int incl = team_inclusive_scan<32>(sum, lane, 0xffffffffu);
     if (lane == 31) warp_tot[warp] = incl;
     __syncthreads();
-    if (warp == 0) {
-      const int w = warp_tot[lane];
-      const int wi = team_inclusive_scan<32>(w, lane, 0xffffffffu);
-      warp_tot[lane] = wi - w;
+    int run = carry + incl - sum;
+#pragma unroll
+    for (int w = 0; w < kBinBlock / 32; ++w) {
+      run += w < warp ? warp_tot[w] : 0;
+      carry += warp_tot[w];
     }
-    __syncthreads();
-    int run = carry + warp_tot[warp] + incl - sum;
 #pragma unroll
     for (int t = 0; t < P; ++t) {
-      const long long idx = i0 + t;
-      if (idx < total) {
-        blk[idx] = run;
-        if (idx % nblk == 0) bin_start[idx / nblk] = run;
-      }
+      if (i0 + t < nblk) mine[i0 + t] = run;
       run += v[t];
     }
     __syncthreads();
-    if (threadIdx.x == blockDim.x - 1) carry = run;
-    __syncthreads();
   }
-  if (threadIdx.x == 0) bin_start[nb] = carry;
+  if (threadIdx.x == 0) tot[blockIdx.x] = carry;
 }
 
+// bin_start[b] = first position of bin b, bin_start[nb] = total.
 __global__ void __launch_bounds__(kBinBlock)
 k_bin_scatter(int32_t m, const uint8_t* __restrict__ bin, int32_t nb, int32_t nblk,
-              const int32_t* __restrict__ blk_off, int32_t* __restrict__ rows_out) {
+              const int32_t* __restrict__ blk_off, const int32_t* __restrict__ tot,
+              int32_t* __restrict__ rows_out, int32_t* __restrict__ bin_start) {
   constexpr int NW = kBinBlock / 32;
+  static_assert(kMaxBins <= 64, "two bins per lane");
   __shared__ int wcount[NW][kMaxBins];
-  __shared__ int running[kMaxBins];
+  __shared__ int running[64];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int t = threadIdx.x; t < NW * kMaxBins; t += blockDim.x) (&wcount[0][0])[t] = 0;
-  if (threadIdx.x < nb) running[threadIdx.x] = blk_off[(long long)threadIdx.x * nblk + blockIdx.x];
-  __syncthreads();
+  if (warp == 0) {  // the bins' first positions, and this block's in each
+    const int b0 = 2 * lane, b1 = 2 * lane + 1;
+    const int v0 = b0 < nb ? tot[b0] : 0, v1 = b1 < nb ? tot[b1] : 0;
+    const int incl = team_inclusive_scan<32>(v0 + v1, lane, 0xffffffffu);
+    const int s0 = incl - v0 - v1, s1 = incl - v1;
+    if (b0 < nb) running[b0] = s0 + blk_off[(long long)b0 * nblk + blockIdx.x];
+    if (b1 < nb) running[b1] = s1 + blk_off[(long long)b1 * nblk + blockIdx.x];
+    if (blockIdx.x == 0) {
+      if (b0 <= nb) bin_start[b0] = s0;
+      if (b1 <= nb) bin_start[b1] = s1;
+    }
+  }
   const long long base = (long long)blockIdx.x * kBinRows;
+  const unsigned long long v = bin_bytes(bin, base + (long long)threadIdx.x * kBinPerThread, m);
+  const int first = (int)bin[base];
+  if (__syncthreads_and(bin_uniform(v) && (int)(v & 0xFF) == first)) {
+    if (first != kSkipBin)
+      for (int t = threadIdx.x; t < kBinRows; t += kBinBlock) rows_out[running[first] + t] = (int32_t)(base + t);
+    return;
+  }
+  for (int t = threadIdx.x; t < NW * kMaxBins; t += blockDim.x) (&wcount[0][0])[t] = 0;
+  __syncthreads();
   const unsigned lt = (1u << lane) - 1u;
   for (int t = 0; t < kBinPerThread; ++t) {
     const long long r = base + t * kBinBlock + threadIdx.x;
@@ -377,11 +422,12 @@ k_bin_scatter(int32_t m, const uint8_t* __restrict__ bin, int32_t nb, int32_t nb
     __syncthreads();
     if (threadIdx.x < nb) {
       int s = 0;
-      for (int w = 0; w < NW; ++w) s += wcount[w][threadIdx.x];
+      for (int w = 0; w < NW; ++w) {
+        s += wcount[w][threadIdx.x];
+        wcount[w][threadIdx.x] = 0;
+      }
       running[threadIdx.x] += s;
     }
-    __syncthreads();
-    for (int q = threadIdx.x; q < NW * kMaxBins; q += blockDim.x) (&wcount[0][0])[q] = 0;
     __syncthreads();
   }
 }
@@ -390,7 +436,7 @@ k_bin_scatter(int32_t m, const uint8_t* __restrict__ bin, int32_t nb, int32_t nb
 // Scan of row counts into int64 row pointers, fused with numeric bin ids.
 // ---------------------------------------------------------------------------
 constexpr int kScanBlock = 256;
-constexpr int kScanPer = 8;
+constexpr int kScanPer = 2;  // few rows per thread: a row's classification is a chain of its own
 constexpr int kScanRows = kScanBlock * kScanPer;
 
 __device__ __forceinline__ long long block_excl_scan_ll(long long v, long long* scratch,
@@ -831,6 +877,7 @@ struct kk_spgemm_handle_s {
   bool cache_valid = false;
   // wide-tier bit vectors kept by the symbolic phase
   DevBuf d_wbits, d_wslot, d_wnext, d_wtasks, d_widx, d_wtab;
+  DevBuf d_along_rows, d_blong;  // long rows of A and of B (analysis)
   int32_t wide_kept = 0;  // rows kept with tasks by the last symbolic call
   bool b_overflow = false;             // the persistent batched form handed a batch to the packed form
   unsigned long long b_overflow_key = 0;  // ... the batch's key (pairs, output pointer, count)
@@ -864,6 +911,7 @@ struct Misc {
   unsigned long long fp[2];      // structure fingerprints: symbolic call, numeric call
   int32_t small_flags[4];        // small-product path: row beyond it, bad index, CTA ticket
   int32_t wide_kept;             // rows kept with chunk tasks
+  int32_t long_a, long_b;        // long rows listed by the analyses
   int32_t pad2;
 };
 static_assert(sizeof(Misc) <= 256, "the staging buffer's bin starts follow at byte 256");
@@ -936,8 +984,11 @@ void build_bins(const kk_spgemm_options& o, bool numeric, std::vector<BinSpec>& 
   out.clear();
   const int force = o.force_tier;
   // thread tier first (automatic tier choice only)
-  if (force == -1)
-    out.push_back(BinSpec{kTierThread, 1, 0, 0, 0, numeric ? kThreadNumMax : kThreadSymMax});
+  if (force == -1) {
+    const long long most = numeric ? kThreadNumMax : kThreadSymMax;
+    out.push_back(BinSpec{kTierThread, 1, 0, 0, 0, most / 2});
+    out.push_back(BinSpec{kTierThread, 1, 0, 0, 0, most});
+  }
   if (!numeric) {
     if (force < 1) {
       for (int ls = 5; ls <= 12; ++ls) {
@@ -1025,6 +1076,17 @@ LaunchCtx ctx_of(kk_spgemm_handle h) {
                    h->opt.stage_long_rows, nullptr, h->opt.arith == KK_ARITH_AUTO ? 1 : 0};
 }
 
+// The list of a matrix's long rows: matrices of fewer than 2^18 entries do
+// without (their longest row costs less than a launch).
+kk_status long_rows(kk_spgemm_handle h, const CsrView& M, DevBuf* buf, int32_t* count, LongRows* out) {
+  *out = LongRows{nullptr, nullptr, 0};
+  if (M.nnz < (1 << 18)) return KK_OK;
+  const int32_t most = M.nnz / kLongRow + 1;
+  KK_CUDA(h, buf->ensure(sizeof(int32_t) * (size_t)most), "alloc long rows");
+  *out = LongRows{buf->as<int32_t>(), count, most};
+  return KK_OK;
+}
+
 // Analysis of B at the start of a symbolic call; with the window tier on, the
 // same pass writes the compressed B (valid once B is known to be sorted, see
 // accept_bcomp).
@@ -1040,7 +1102,9 @@ kk_status analyze_b(kk_spgemm_handle h, const CsrView& bv) {
     len = h->d_bclen.as<int32_t>();
   }
   Misc* dm = h->d_misc.as<Misc>();
-  KK_CUDA(h, launch_analyze_b(ctx_of(h), bv, &dm->sorted, bc, len, &dm->bc_pairs), "analyze launch");
+  LongRows lr;
+  KK_TRY(long_rows(h, bv, &h->d_blong, &dm->long_b, &lr));
+  KK_CUDA(h, launch_analyze_b(ctx_of(h), bv, &dm->sorted, bc, len, &dm->bc_pairs, lr), "analyze launch");
   return KK_OK;
 }
 
@@ -1070,7 +1134,7 @@ kk_status ensure_bcomp(kk_spgemm_handle h, const CsrView& bv, BComp* out, int* b
     KK_CUDA(h, h->d_bclen.ensure(sizeof(int32_t) * (size_t)bv.m), "alloc compressed B");
     // sortedness is not re-decided here: the flag goes to a scratch word
     KK_CUDA(h, launch_analyze_b(ctx_of(h), bv, &h->d_misc.as<Misc>()->pad, h->d_bc.as<int2>(),
-                                h->d_bclen.as<int32_t>(), nullptr),
+                                h->d_bclen.as<int32_t>(), nullptr, LongRows{nullptr, nullptr, 0}),
             "compress launch");
     accept_bcomp(h, bv, true);
     *built = 1;
@@ -1276,12 +1340,13 @@ kk_status run_binning(kk_spgemm_handle h, int32_t m, const uint8_t* bin, int nb,
     KK_CUDA(h, cudaMemsetAsync(bin_start, 0, sizeof(int32_t) * (nb + 1), h->stream), "memset");
     return KK_OK;
   }
-  KK_CUDA(h, h->d_blk.ensure(sizeof(int32_t) * (size_t)nb * nblk), "alloc bins");
+  KK_CUDA(h, h->d_blk.ensure(sizeof(int32_t) * ((size_t)nb * nblk + kMaxBins)), "alloc bins");
   int32_t* blk = h->d_blk.as<int32_t>();
+  int32_t* tot = blk + (size_t)nb * nblk;
   timer_begin(h->timer, h->stream, "binning");
   k_bin_count<<<nblk, kBinBlock, 0, h->stream>>>(m, bin, nb, nblk, blk);
-  k_bin_scan<<<1, 1024, 0, h->stream>>>(nb, nblk, blk, bin_start);
-  k_bin_scatter<<<nblk, kBinBlock, 0, h->stream>>>(m, bin, nb, nblk, blk, rows_out);
+  k_bin_scan<<<nb, kBinBlock, 0, h->stream>>>(nblk, blk, tot);
+  k_bin_scatter<<<nblk, kBinBlock, 0, h->stream>>>(m, bin, nb, nblk, blk, tot, rows_out, bin_start);
   timer_end(h->timer, h->stream);
   KK_CUDA(h, cudaGetLastError(), "binning launch");
   return KK_OK;
@@ -1338,20 +1403,31 @@ static cudaError_t launch_jacobi_rows(kk_spgemm_handle h, const CsrView& av, con
 // strides over rows).
 // bin receives the symbolic bin ids; with STATS, stat the learned form's row
 // statistics.
-template <int T, int U, bool STATS = false>
-static void launch_analyze_a(kk_spgemm_handle h, const CsrView& av, const CsrView& bv, Misc* dm,
-                             cudaStream_t s, uint8_t* bin, int2* stat = nullptr) {
+template <int T, int U, bool STATS, bool LISTED>
+static void launch_analyze_a_t(kk_spgemm_handle h, const CsrView& av, const CsrView& bv, Misc* dm,
+                               cudaStream_t s, uint8_t* bin, int2* stat, const LongRows& lr) {
+  auto kern = k_analyze_a<T, U, STATS, LISTED>;
   static int per_sm = 0;
-  if (per_sm == 0 &&
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_analyze_a<T, U, STATS>, 256, 0) != cudaSuccess) {
+  if (per_sm == 0 && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, 0) != cudaSuccess) {
     (void)cudaGetLastError();
     per_sm = 4;
   }
-  const int64_t m = av.m;
-  k_analyze_a<T, U, STATS><<<grid_for(m * T, 256, h->num_sms * (per_sm > 0 ? per_sm : 1)), 256, 0, s>>>(
+  const int64_t m = LISTED ? lr.most : av.m;
+  kern<<<grid_for(m * T, 256, h->num_sms * (per_sm > 0 ? per_sm : 1)), 256, 0, s>>>(
       av, bv.rowptr, bv.colind, bv.m, &dm->sorted, to_table(h->sym_bins, false, bv.n), h->opt.team_vec_min_len,
       h->d_flop.as<long long>(), bin, h->d_rowlo.as<int32_t>(), h->d_span.as<int32_t>(), stat,
-      &dm->total_flop, &dm->status);
+      &dm->total_flop, &dm->status, lr);
+}
+
+// Teams by A's mean row length: the smallest whose U = 8 gathers per lane cover
+// a typical row in one round (more rows in flight per SM; measured against teams
+// of 4 and 8), then the listed long rows.
+template <bool STATS = false>
+static void launch_analyze_a(kk_spgemm_handle h, const CsrView& av, const CsrView& bv, Misc* dm,
+                             cudaStream_t s, uint8_t* bin, const LongRows& lr, int2* stat = nullptr) {
+  if ((long long)av.nnz / av.m <= 8) launch_analyze_a_t<1, 8, STATS, false>(h, av, bv, dm, s, bin, stat, lr);
+  else launch_analyze_a_t<4, 8, STATS, false>(h, av, bv, dm, s, bin, stat, lr);
+  if (lr.rows) launch_analyze_a_t<32, 8, STATS, true>(h, av, bv, dm, s, bin, stat, lr);
 }
 
 extern "C" {
@@ -1540,13 +1616,9 @@ kk_status kk_spgemm_symbolic(kk_spgemm_handle h, const kk_csr* A, const kk_csr* 
   if (m > 0) {
     timer_begin(h->timer, s, "analyze");
     if ((st = analyze_b(h, bv)) != KK_OK) return st;
-    // smallest team whose U = 8 gathers per lane cover a typical row in one
-    // round (more rows in flight per SM; measured against teams of 4 and 8)
-    const long long avg = m > 0 ? (long long)av.nnz / m : 0;
-    if (avg <= 8)
-      launch_analyze_a<1, 8>(h, av, bv, dm, s, h->d_sbin.as<uint8_t>());
-    else
-      launch_analyze_a<4, 8>(h, av, bv, dm, s, h->d_sbin.as<uint8_t>());
+    LongRows lr;
+    KK_TRY(long_rows(h, av, &h->d_along_rows, &dm->long_a, &lr));
+    launch_analyze_a(h, av, bv, dm, s, h->d_sbin.as<uint8_t>(), lr);
     timer_end(h->timer, s);
     KK_CUDA(h, cudaGetLastError(), "analyze launch");
     if ((st = run_binning(h, m, h->d_sbin.as<uint8_t>(), nbs, h->d_srows.as<int32_t>(), sym_start)) != KK_OK)
@@ -1693,7 +1765,20 @@ static kk_status numeric_impl(kk_spgemm_handle h, const kk_csr* A, const kk_csr*
   if (h->am == 0 || h->nnz_c == 0) return KK_OK;
   const float2* bsplit = nullptr;
   keep_for_numeric(h, av, bv);
-  if (arith == kArithDF32) {
+  // with the automatic arithmetic only the hash tiers run in DF32
+  bool df32 = arith == kArithDF32;
+  if (df32 && h->opt.arith == KK_ARITH_AUTO) {
+    const bool wide = wide_numeric_fits(ctx_of(h), bv.n);
+    df32 = false;
+    for (size_t b = 0; b < h->num_bins.size(); ++b) {
+      const int32_t tier = h->num_bins[b].tier;
+      if (h->num_start[b + 1] > h->num_start[b] &&
+          (tier == kTierTeam || (!wide && (tier == kTierCta || tier == kTierDense))))
+        df32 = true;
+    }
+    if (!df32) h->last_arith = kArithF64;
+  }
+  if (df32) {
     KK_CUDA(h, h->d_bsplit.ensure(sizeof(float2) * (size_t)(bv.nnz > 0 ? bv.nnz : 1)), "alloc split");
     KK_CUDA(h, cudaMemsetAsync(&dm->range_bad, 0, sizeof(int32_t), s), "memset");
     if (bv.nnz > 0) {
@@ -1707,7 +1792,7 @@ static kk_status numeric_impl(kk_spgemm_handle h, const kk_csr* A, const kk_csr*
   }
   LaunchCtx ctx = ctx_of(h);
   const int nbn = (int)h->num_bins.size();
-  h->stats[9] = (arith == kArithDF32 && bv.nnz > 0) ? 1 : 0;
+  h->stats[9] = (df32 && bv.nnz > 0) ? 1 : 0;
   bool any_win = false;
   for (int b = 0; b < nbn; ++b)
     if (stat_tier(h->num_bins[b].tier) == kTierWindow && h->num_start[b + 1] > h->num_start[b]) any_win = true;
@@ -1965,11 +2050,9 @@ kk_status kk_spgemm_learned_symbolic(kk_spgemm_handle h, const kk_csr* A, const 
     // the plain row analysis (flop bound, span, symbolic bin of every row,
     // the B-row statistics the features need), then the classification
     timer_begin(h->timer, s, "learned_analyze");
-    const long long avg = (long long)av.nnz / m;
-    if (avg <= 8)
-      launch_analyze_a<1, 8, true>(h, av, bv, dm, s, h->d_sball.as<uint8_t>(), h->d_lstat.as<int2>());
-    else
-      launch_analyze_a<4, 8, true>(h, av, bv, dm, s, h->d_sball.as<uint8_t>(), h->d_lstat.as<int2>());
+    LongRows lr;
+    KK_TRY(long_rows(h, av, &h->d_along_rows, &dm->long_a, &lr));
+    launch_analyze_a<true>(h, av, bv, dm, s, h->d_sball.as<uint8_t>(), lr, h->d_lstat.as<int2>());
     cudaError_t e = launch_learned_classify(
         ctx, av, bv.n, &dm->sorted, h->opt.use_window, h->opt.structure_cache ? 0 : 1,
         h->have_pred ? h->d_params.as<float>() : nullptr,
@@ -2398,7 +2481,7 @@ kk_status kk_spgemm_batched_symbolic(kk_spgemm_handle h, int32_t count, const kk
   KK_CUDA(h, h->d_bstart.ensure(sizeof(int32_t) * 2 * (kMaxBBins + 1)), "alloc batch");
   KK_CUDA(h, h->d_bqueue.ensure(sizeof(int) * 2), "alloc batch");
   KK_CUDA(h, h->d_boff.ensure(sizeof(int64_t) * ((size_t)count + 1)), "alloc batch");
-  KK_CUDA(h, h->d_blk.ensure(sizeof(int32_t) * (size_t)nbmax * (size_t)(nblk > 0 ? nblk : 1)), "alloc bins");
+  KK_CUDA(h, h->d_blk.ensure(sizeof(int32_t) * ((size_t)nbmax * (size_t)(nblk > 0 ? nblk : 1) + kMaxBins)), "alloc bins");
   KK_CUDA(h, h->d_scan.ensure(sizeof(long long) * (size_t)(nblk_scan > 0 ? nblk_scan : 1)), "alloc scan");
   if (h->d_span.bytes == 0) KK_CUDA(h, h->d_span.ensure(4), "alloc");
   if (h->d_flop.bytes == 0) KK_CUDA(h, h->d_flop.ensure(8), "alloc");
@@ -2605,7 +2688,7 @@ kk_status kk_spgemm_destroy(kk_spgemm_handle h) {
                     &h->d_bdesc, &h->d_rowpair, &h->d_bflop, &h->d_bsbin, &h->d_bnbin, &h->d_bsrows,
                     &h->d_bnrows, &h->d_bcnt, &h->d_btiles, &h->d_bstart, &h->d_bqueue, &h->d_bsplit2,
                     &h->d_boff, &h->d_bc, &h->d_bclen, &h->d_cw, &h->d_cm, &h->d_cn, &h->d_wbits,
-                    &h->d_wslot, &h->d_wnext, &h->d_wtasks, &h->d_widx, &h->d_wtab, &h->d_pa_rp, &h->d_pa_ci, &h->d_pa_v, &h->d_pb_rp, &h->d_pb_ci,
+                    &h->d_wslot, &h->d_wnext, &h->d_wtasks, &h->d_widx, &h->d_wtab, &h->d_along_rows, &h->d_blong, &h->d_pa_rp, &h->d_pa_ci, &h->d_pa_v, &h->d_pb_rp, &h->d_pb_ci,
                     &h->d_pb_v, &h->d_pbase})
     b->release();
   for (void* p : {h->h_bdesc, h->h_bdesc2, h->h_boff})

@@ -115,7 +115,7 @@ __host__ __device__ constexpr int32_t stat_tier(int32_t t) {
 // Thread tier (kk_thread.cu): one thread per row, accumulator in registers.
 constexpr int kThreadSymMax = 16;     // symbolic rows: flop bound <= this
 constexpr int kThreadNumMax = 8;      // numeric rows: nnz(C(i,:)) <= this ...
-constexpr int kThreadNumMaxFlop = 16; // ... and flop bound <= this
+constexpr int kThreadNumMaxFlop = 64; // ... and flop bound <= this
 // Small products (kk_small.cu): one launch per phase, a thread per row, for A
 // with at most options.small_max_rows rows (at most kSmallMaxRowsCap), C rows
 // of at most kSmallN columns, tried when A's rows average at most
@@ -142,7 +142,12 @@ constexpr long long kWindowMaxFlop = 4096;  // symbolic rows of a narrow B (k <=
 constexpr int kNumRankBits = 5, kNumRankNnz = 3;
 constexpr int32_t kRankBits[kNumRankBits] = {4096, 8192, 16384, 32768, 65536};
 constexpr int32_t kRankNnz[kNumRankNnz] = {256, 512, 1024};
-constexpr int32_t kRankFlopRatio = 512;  // rank tier used only when W <= ratio * flop
+// Rank tier used only when W <= kRankFlopRatio * flop, and for rows of at most
+// kRankMinNnz columns when W <= kWindowFlopRatio * flop: short rows share a warp
+// in the thread and team tiers (262,144 rows of 7 columns over 8,200: 130 us in
+// the team tier, 400 in the rank tier).
+constexpr int32_t kRankFlopRatio = 512;
+constexpr int32_t kRankMinNnz = 32;
 constexpr int kMaxWindowBins = kNumWindowClasses + kNumRankBits * kNumRankNnz;
 
 // Per-row structure kept by the symbolic window kernel for the numeric phase
@@ -197,8 +202,17 @@ cudaError_t launch_num_rank(const LaunchCtx& ctx, const BinSpec& bin, const CsrV
                             const int32_t* b_range_bad, int32_t arith, const int64_t* c_rowptr,
                             const int32_t* rows, int32_t nrows, int32_t* c_colind, double* c_vals);
 
+// Analysis kernels: rows of more than kLongRow entries, listed for a second
+// launch with a warp per row (rows null: no list).
+constexpr int kLongRow = 512;
+struct LongRows {
+  int32_t* rows;
+  int32_t* count;
+  int32_t most;
+};
+
 cudaError_t launch_analyze_b(const LaunchCtx& ctx, const CsrView& B, int32_t* sorted_flag,
-                             int2* bc, int32_t* len, unsigned long long* pairs);
+                             int2* bc, int32_t* len, unsigned long long* pairs, const LongRows& lr);
 
 // Arithmetic mode for the numeric kernels.
 enum ArithMode : int32_t { kArithF64 = 1, kArithDF32 = 2 };
@@ -240,14 +254,14 @@ cudaError_t launch_num_chunk(const LaunchCtx& ctx, const CsrView& A, const CsrVi
                              int32_t* c_colind, double* c_vals);
 
 cudaError_t launch_symbolic_thread(const LaunchCtx& ctx, const CsrView& A, const CsrView& B,
-                                   const int32_t* rows, int32_t nrows, int32_t* cnt);
+                                   const int32_t* rows, int32_t nrows, int32_t* cnt, long long max_flop);
 cudaError_t launch_small_symbolic(const LaunchCtx& ctx, const CsrView& A, const CsrView& B, int64_t* c_rowptr,
                                   int32_t* cnt, int32_t* flags, long long* out);
 cudaError_t launch_small_numeric(const LaunchCtx& ctx, const CsrView& A, const CsrView& B,
                                  const int64_t* c_rowptr, int32_t* c_colind, double* c_vals);
 cudaError_t launch_numeric_thread(const LaunchCtx& ctx, const CsrView& A, const CsrView& B,
                                   const int64_t* c_rowptr, const int32_t* rows, int32_t nrows,
-                                  int32_t* c_colind, double* c_vals);
+                                  int32_t* c_colind, double* c_vals, long long max_nnz);
 
 // Window-tier launches (kk_window.cu).
 cudaError_t launch_symbolic_window(const LaunchCtx& ctx, const BinSpec& bin, const CsrView& A,
