@@ -814,7 +814,8 @@ struct kk_spgemm_handle_s {
   DevBuf d_jpos;       // int32[m]: position of each row's first diagonal entry (Jacobi)
   DevBuf d_apos, d_bpos;  // SpAdd: slot in C's row of every entry of A and of B (int32)
   DevBuf d_acnt;          // SpAdd: nnz(C(i,:)) (int32[m])
-  DevBuf d_along;         // SpAdd: [0] long-row count, [1..] long rows (int32[m + 1])
+  DevBuf d_akind;         // SpAdd: 1 for a row merged by the numeric phase (uint8[m])
+  DevBuf d_along;         // SpAdd: long rows, their count first (int32[m + 1])
   // learned form
   DevBuf d_params;     // float[KK_MLP_NUM_PARAMS]
   bool have_pred = false;
@@ -1908,14 +1909,15 @@ kk_status kk_spadd_symbolic(kk_spgemm_handle h, const kk_csr* A, const kk_csr* B
   // only the status word is reset: the rest of the device record belongs to
   // the SpGEMM state of this handle (fingerprints, flags), which SpAdd leaves alone
   KK_CUDA(h, cudaMemsetAsync(&dm->status, 0, sizeof(int), s), "memset");
-  KK_CUDA(h, cudaMemsetAsync(h->d_along.p, 0, sizeof(int32_t), s), "memset");
+  KK_CUDA(h, h->d_akind.ensure((size_t)(m > 0 ? m : 1)), "alloc SpAdd");
+  int32_t* long_rows = h->d_along.as<int32_t>();
+  KK_CUDA(h, cudaMemsetAsync(long_rows, 0, sizeof(int32_t), s), "memset");
   int64_t nnz = 0;
   if (m > 0) {
     LaunchCtx ctx = ctx_of(h);
     timer_begin(h->timer, s, "spadd_symbolic");
     cudaError_t e = launch_spadd_symbolic(ctx, view(A), view(B), h->d_acnt.as<int32_t>(),
-                                          h->d_apos.as<int32_t>(), h->d_bpos.as<int32_t>(),
-                                          h->d_along.as<int32_t>() + 1, h->d_along.as<int32_t>());
+                                          h->d_apos.as<int32_t>(), h->d_bpos.as<int32_t>(), h->d_akind.as<uint8_t>(), long_rows);
     timer_end(h->timer, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "SpAdd symbolic launch");
     timer_begin(h->timer, s, "scan");
@@ -1960,9 +1962,9 @@ kk_status kk_spadd_numeric(kk_spgemm_handle h, double alpha, const kk_csr* A, do
   if (!c_colind || !c_vals) return fail(h, KK_ERR_INVALID_ARG, "C arrays are NULL");
   cudaStream_t s = h->stream;
   timer_begin(h->timer, s, "spadd_numeric");
-  KK_CUDA(h, cudaMemsetAsync(c_vals, 0, sizeof(double) * (size_t)h->add_nnzc, s), "memset");
   cudaError_t e = launch_spadd_numeric(ctx_of(h), view(A), view(B), alpha, beta, c_rowptr,
-                                       h->d_apos.as<int32_t>(), h->d_bpos.as<int32_t>(), c_colind, c_vals);
+                                       h->d_apos.as<int32_t>(), h->d_bpos.as<int32_t>(), h->d_akind.as<uint8_t>(),
+                                       c_colind, c_vals);
   timer_end(h->timer, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "SpAdd numeric launch");
   return KK_OK;

@@ -1,24 +1,32 @@
 // Sparse matrix addition C = alpha A + beta B (Kokkos Kernels paper, Sec.
 // "SpAdd"), symbolic and numeric phases.
 //
-// Symbolic, per row: the row's entries of A and B become 64-bit keys
+// Rows that are strictly ascending in both matrices, of up to kAddWarpMax combined
+// entries, are merged by binary search of each entry in the other row, staged in
+// shared memory: the symbolic phase counts the shared columns, the numeric phase
+// merges again and writes the row of C in one go.  Nothing is kept between the
+// phases for them: reading both rows' columns again, which C's columns need
+// anyway, costs less than writing and reading a slot per entry, adding into C
+// with atomics and zeroing it first (two matrices of 500,000 rows of 30: 286 us
+// symbolic and 217 numeric that way, 116 and 184 now; bound by issue and by the
+// latency of a row's loads, which prefetching the next row's did not shorten: it
+// costs a third of the warps in flight).
+//
+// Other rows: the entries of A and B become 64-bit keys
 // (column << 32 | source bit (B) << 31 | index within the source row) in
 // shared memory and are sorted by a bitonic network; equal columns are then
 // adjacent, so a scan of "first of its column" flags gives nnz(C(i,:)) and, for
 // every entry of A and of B, its slot in the row of C (the paper's Apos and
-// Bpos).  Rows that are both strictly ascending take their slots by binary
-// search of each entry in the other row (no sort).  When both rows are sorted
-// (repeats allowed) the keys are laid out as A ascending, then
-// padding, then B descending: a bitonic sequence, so only the final merge
-// stage runs (the paper's sorted-input method); otherwise the full sort runs
-// (its unsorted-input method).  Rows of up to kAddWarpMax combined entries take
-// one warp, rows of up to kAddCtaMax one CTA of 1024 threads; longer rows are
-// reported as KK_ERR_CAPACITY.
-//
-// Numeric: C's values are zeroed, then every entry of A and of B adds its
-// scaled value at its slot (float64 atomics: an entry of C with at most one
-// entry of A and one of B is the same sum in either order; repeated columns
-// within A or B are added in no fixed order) and writes its column.
+// Bpos; the sign bit marks all but the first entry of a column).  When both rows are sorted (repeats allowed) the keys are laid out as A
+// ascending, then padding, then B descending: a bitonic sequence, so only the
+// final merge stage runs (the paper's sorted-input method); otherwise the full
+// sort runs (its unsorted-input method).  Rows of up to kAddWarpMax combined
+// entries take one warp, rows of up to kAddCtaMax one CTA of 1024 threads; longer
+// rows are reported as KK_ERR_CAPACITY.  Their numeric phase zeroes the row of C,
+// then every entry of A and of B adds its scaled value at its slot (float64
+// atomics: an entry of C with at most one entry of A and one of B is the same
+// sum in either order; repeated columns within A or B are added in no fixed
+// order) and writes its column.
 #include "kk_internal.h"
 #include "kk_device.cuh"
 
@@ -29,7 +37,6 @@ using u64 = unsigned long long;
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kAddWarpMax = 256;
 constexpr int kAddCtaMax = 8192;
-constexpr int kAddWarps = 4;     // warps per CTA of the warp kernel
 constexpr int kAddCtaThreads = 1024;
 constexpr u64 kAddPad = ~0ull;
 
@@ -108,7 +115,7 @@ __device__ __forceinline__ void add_load(const CsrView& A, const CsrView& B, int
 }
 
 // First index in the sorted row x[0, len) whose column is >= c.
-__device__ __forceinline__ int add_lower_bound(const int32_t* __restrict__ x, int len, int c) {
+__device__ __forceinline__ int add_lower_bound(const int32_t* x, int len, int c) {
   int lo = 0, hi = len;
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
@@ -118,97 +125,227 @@ __device__ __forceinline__ int add_lower_bound(const int32_t* __restrict__ x, in
   return lo;
 }
 
-// Slots of one strictly ascending row against another (merge by binary
-// search, no sort): entry k of x at column c lands at
-//   k + #{y < c} - #{columns of x before k that are also in y},
-// the last term an exclusive scan of "found in y" flags.  Returns the number
-// of columns x shares with y.
-__device__ __forceinline__ int add_slots_sorted(const int32_t* __restrict__ x, int lx,
-                                                const int32_t* __restrict__ y, int ly,
-                                                int32_t* __restrict__ pos, int lane) {
+struct AddRow {
+  int pa, la, pb, lb;
+};
+
+// A row by a warp: its columns go to col (A's la, then B's lb); *strict: both
+// rows strictly ascending.
+__device__ __forceinline__ void add_stage(const CsrView& A, const CsrView& B, const AddRow& r, int32_t* col,
+                                          int lane, bool* strict, int* bad) {
+  __syncwarp();
+  for (int t = lane; t < r.la; t += 32) col[t] = A.colind[r.pa + t];
+  for (int t = lane; t < r.lb; t += 32) col[r.la + t] = B.colind[r.pb + t];
+  __syncwarp();
+  bool off = false;
+  for (int t = lane; t < r.la + r.lb; t += 32) {
+    const int c = col[t];
+    if ((unsigned)c >= (unsigned)A.n) *bad = 1;  // (A and B have the same columns)
+    off |= t > 0 && t != r.la && col[t - 1] >= c;
+  }
+  *strict = !__any_sync(kFull, off);
+}
+
+// Columns that strictly ascending staged rows share.
+__device__ __forceinline__ int add_common(const AddRow& r, const int32_t* col, int lane) {
   int common = 0;
-  for (int t0 = 0; t0 < lx; t0 += 32) {
+  for (int t0 = 0; t0 < r.la; t0 += 32) {
     const int t = t0 + lane;
-    int lb = 0, found = 0;
-    if (t < lx) {
-      const int c = x[t];
-      lb = add_lower_bound(y, ly, c);
-      found = (lb < ly && y[lb] == c) ? 1 : 0;
+    bool found = false;
+    if (t < r.la) {
+      const int c = col[t], k = add_lower_bound(col + r.la, r.lb, c);
+      found = k < r.lb && col[r.la + k] == c;
     }
-    const int incl = team_inclusive_scan<32>(found, lane, kFull);
-    if (t < lx) pos[t] = t + lb - (common + incl - found);
-    common += __shfl_sync(kFull, incl, 31);
+    common += __popc(__ballot_sync(kFull, found));
   }
   return common;
 }
 
-// One warp per row; rows longer than kAddWarpMax go to the long-row list.
-__global__ void __launch_bounds__(kAddWarps * 32)
-k_spadd_sym_warp(CsrView A, CsrView B, int32_t* __restrict__ cnt, int32_t* __restrict__ apos,
-                 int32_t* __restrict__ bpos, int32_t* __restrict__ long_rows,
-                 int32_t* __restrict__ long_count, int* status) {
-  __shared__ u64 keys[kAddWarps][kAddWarpMax];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  u64* key = keys[warp];
-  const long long nw = (long long)gridDim.x * kAddWarps;
+// Strictly ascending staged rows into row off .. off + n of C; returns the merged
+// length.  Entry k of a row lands at k + #{other < its column} - #{shared columns
+// before it}; a shared column is summed by A's entry.
+__device__ __forceinline__ int add_merge(const CsrView& A, const CsrView& B, double alpha, double beta,
+                                         const AddRow& r, const int32_t* col, int64_t off, int n,
+                                         int32_t* __restrict__ c_colind, double* __restrict__ c_vals, int lane) {
+  const unsigned before = (1u << lane) - 1u;
+  const int32_t* ca = col;
+  const int32_t* cb = col + r.la;
+  int common = 0, seen = 0;
+  for (int t0 = 0; t0 < r.la; t0 += 32) {
+    const int t = t0 + lane;
+    bool found = false;
+    int c = 0, k = 0;
+    double v = 0.0;
+    if (t < r.la) {
+      v = A.vals[r.pa + t];
+      c = ca[t];
+      k = add_lower_bound(cb, r.lb, c);
+      found = k < r.lb && cb[k] == c;
+    }
+    if (alpha != 1.0) v *= alpha;
+    if (found) {
+      const double w = B.vals[r.pb + k];
+      v += beta == 1.0 ? w : beta * w;
+    }
+    const unsigned f = __ballot_sync(kFull, found);
+    const int s = t + k - common - __popc(f & before);
+    if (t < r.la && s < n) {
+      c_colind[off + s] = c;
+      c_vals[off + s] = v;
+    }
+    common += __popc(f);
+  }
+  for (int t0 = 0; t0 < r.lb; t0 += 32) {
+    const int t = t0 + lane;
+    bool found = false;
+    int c = 0, k = 0;
+    double v = 0.0;
+    if (t < r.lb) {
+      v = B.vals[r.pb + t];
+      c = cb[t];
+      k = add_lower_bound(ca, r.la, c);
+      found = k < r.la && ca[k] == c;
+    }
+    if (beta != 1.0) v *= beta;
+    const unsigned f = __ballot_sync(kFull, found);
+    const int s = t + k - seen - __popc(f & before);
+    if (t < r.lb && !found && s < n) {
+      c_colind[off + s] = c;
+      c_vals[off + s] = v;
+    }
+    seen += __popc(f);
+  }
+  return r.la + r.lb - common;
+}
+
+// Rows of up to T entries in each matrix: a lane holds one entry of each, and the
+// searches go through shuffles (110 instructions a row instead of 330 through
+// shared memory).
+// Whether the team's rows, one entry of each in a lane (INT_MAX past their ends),
+// are strictly ascending.
+template <int T>
+__device__ __forceinline__ bool add_strict(int ca, int cb, const AddRow& r, int ncols, int tl, unsigned team, int* bad) {
+  if ((tl < r.la && (unsigned)ca >= (unsigned)ncols) || (tl < r.lb && (unsigned)cb >= (unsigned)ncols)) *bad = 1;
+  const int ua = __shfl_up_sync(kFull, ca, 1, T), ub = __shfl_up_sync(kFull, cb, 1, T);
+  const bool off = tl > 0 && ((tl < r.la && ua >= ca) || (tl < r.lb && ub >= cb));
+  return (__ballot_sync(kFull, off) & team) == 0u;
+}
+// Columns below c in the team's sorted x (padded with INT_MAX); *at: x holds c there.
+template <int T>
+__device__ __forceinline__ int add_search(int x, int c, bool* at) {
+  int pos = 0;
+#pragma unroll
+  for (int st = T / 2; st > 0; st >>= 1)
+    if (__shfl_sync(kFull, x, pos + st - 1, T) < c) pos += st;
+  const int v = __shfl_sync(kFull, x, pos, T);
+  *at = v == c;
+  return pos + (v < c ? 1 : 0);
+}
+
+// Slots of a row that is not strictly ascending, sorted by one warp; returns
+// nnz(C(i,:)).
+__device__ __forceinline__ int add_sort_row(const CsrView& A, const CsrView& B, const AddRow& r, u64* key,
+                                            int32_t* __restrict__ apos, int32_t* __restrict__ bpos, int lane,
+                                            int& bad) {
+  const int L = r.la + r.lb, n = next_pow2(L);
+  int unsorted = 0;
+  add_load<32>(A, B, r.pa, r.la, r.pb, r.lb, n, key, lane, unsorted, bad);
+  unsorted = __any_sync(kFull, unsorted);
+  __syncwarp();
+  add_sort<32>(key, n, lane, !unsorted);
+  // slots: scan of "first of its column" flags over the L sorted keys
+  int run = 0;
+  for (int t0 = 0; t0 < L; t0 += 32) {
+    const int t = t0 + lane;
+    u64 k = 0;
+    int first = 0;
+    if (t < L) {
+      k = key[t];
+      first = (t == 0 || (key[t - 1] >> 32) != (k >> 32)) ? 1 : 0;
+    }
+    const int incl = team_inclusive_scan<32>(first, lane, kFull);
+    if (t < L) {
+      const int slot = (run + incl - 1) | (first ? 0 : (int)0x80000000u);
+      const int idx = (int)(k & 0x7fffffffull);
+      if (k & (1ull << 31)) bpos[r.pb + idx] = slot;
+      else apos[r.pa + idx] = slot;
+    }
+    run += __shfl_sync(kFull, incl, 31);
+  }
+  __syncwarp();
+  return run;
+}
+
+// Symbolic, T lanes per row: rows that do not fit the team, or are not strictly
+// ascending, are taken by the whole warp afterwards; rows of more than
+// kAddWarpMax entries go to long_rows (count first).  kind: 1 for a row that the
+// numeric phase merges, 0 for one with slots.
+constexpr int kAddRowWarps = 8;
+template <int T>
+__global__ void __launch_bounds__(kAddRowWarps * 32)
+k_spadd_count(CsrView A, CsrView B, int32_t* __restrict__ cnt, int32_t* __restrict__ apos,
+              int32_t* __restrict__ bpos, uint8_t* __restrict__ kind, int32_t* __restrict__ long_rows,
+              int* status) {
+  __shared__ u64 keys[kAddRowWarps][kAddWarpMax];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tl = lane % T, tm = lane / T;
+  const unsigned team = team_mask<T>();
+  const long long stride = (long long)gridDim.x * kAddRowWarps * (32 / T);
   int bad = 0;
-  for (long long r = (long long)blockIdx.x * kAddWarps + warp; r < A.m; r += nw) {
-    const int pa = A.rowptr[r], la = A.rowptr[r + 1] - pa;
-    const int pb = B.rowptr[r], lb = B.rowptr[r + 1] - pb;
-    const int L = la + lb;
-    if (L > kAddWarpMax) {
-      if (lane == 0) long_rows[atomicAdd(long_count, 1)] = (int32_t)r;
-      continue;
-    }
-    if (L == 0) {
-      if (lane == 0) cnt[r] = 0;
-      continue;
-    }
-    // both rows strictly ascending (no repeated column): slots by binary search
-    int strict_bad = 0;
-    for (int t = lane; t < la; t += 32) {
-      const int c = A.colind[pa + t];
-      if ((unsigned)c >= (unsigned)A.n) bad = 1;
-      if (t > 0 && A.colind[pa + t - 1] >= c) strict_bad = 1;
-    }
-    for (int t = lane; t < lb; t += 32) {
-      const int c = B.colind[pb + t];
-      if ((unsigned)c >= (unsigned)B.n) bad = 1;
-      if (t > 0 && B.colind[pb + t - 1] >= c) strict_bad = 1;
-    }
-    if (!__any_sync(kFull, strict_bad)) {
-      const int common = add_slots_sorted(A.colind + pa, la, B.colind + pb, lb, apos + pa, lane);
-      add_slots_sorted(B.colind + pb, lb, A.colind + pa, la, bpos + pb, lane);
-      if (lane == 0) cnt[r] = la + lb - common;
-      continue;
-    }
-    const int n = next_pow2(L);
-    int unsorted = 0;
-    add_load<32>(A, B, pa, la, pb, lb, n, key, lane, unsorted, bad);
-    unsorted = __any_sync(kFull, unsorted);
-    __syncwarp();
-    add_sort<32>(key, n, lane, !unsorted);
-    // slots: scan of "first of its column" flags over the L sorted keys
-    int run = 0;
-    for (int t0 = 0; t0 < L; t0 += 32) {
-      const int t = t0 + lane;
-      u64 k = 0;
-      int first = 0;
-      if (t < L) {
-        k = key[t];
-        first = (t == 0 || (key[t - 1] >> 32) != (k >> 32)) ? 1 : 0;
+  auto bounds = [&](long long row) -> AddRow {
+    AddRow r{0, 0, 0, 0};
+    if (row < A.m) {
+      r.pa = A.rowptr[row];
+      r.la = A.rowptr[row + 1] - r.pa;
+      r.pb = B.rowptr[row];
+      r.lb = B.rowptr[row + 1] - r.pb;
+      if (r.la < 0 || r.lb < 0) {
+        bad = 1;
+        r.la = r.lb = 0;
       }
-      const int incl = team_inclusive_scan<32>(first, lane, kFull);
-      if (t < L) {
-        const int slot = run + incl - 1;
-        const int idx = (int)(k & 0x7fffffffull);
-        if (k & (1ull << 31)) bpos[pb + idx] = slot;
-        else apos[pa + idx] = slot;
-      }
-      run += __shfl_sync(kFull, incl, 31);
     }
-    if (lane == 0) cnt[r] = run;
-    __syncwarp();
+    return r;
+  };
+  const long long first = ((long long)blockIdx.x * kAddRowWarps + warp) * (32 / T);
+  for (long long r0 = first; r0 < A.m; r0 += stride) {
+    const long long row = r0 + tm;
+    const AddRow all = bounds(row);
+    AddRow r = all;
+    const int L = r.la + r.lb;
+    const bool big = r.la > T || r.lb > T;
+    if (big) r.la = r.lb = 0;
+    const int ca = tl < r.la ? A.colind[r.pa + tl] : 0x7fffffff;
+    const int cb = tl < r.lb ? B.colind[r.pb + tl] : 0x7fffffff;
+    const bool ok = add_strict<T>(ca, cb, r, A.n, tl, team, &bad);
+    bool found;
+    add_search<T>(cb, ca, &found);
+    const int common = __popc(__ballot_sync(kFull, found && tl < r.la) & team);
+    if (row < A.m && !big && ok && tl == 0) {
+      cnt[row] = L - common;
+      kind[row] = 1;
+    }
+    for (unsigned m = __ballot_sync(kFull, (big || !ok) && tl == 0); m; m &= m - 1) {
+      const int src = __ffs(m) - 1;
+      const AddRow w{__shfl_sync(kFull, all.pa, src), __shfl_sync(kFull, all.la, src),
+                     __shfl_sync(kFull, all.pb, src), __shfl_sync(kFull, all.lb, src)};
+      const long long wrow = r0 + src / T;
+      if (w.la + w.lb > kAddWarpMax) {
+        if (lane == 0) {
+          long_rows[1 + atomicAdd(long_rows, 1)] = (int32_t)wrow;
+          kind[wrow] = 0;
+        }
+        continue;
+      }
+      bool strict = false;
+      int32_t* col = reinterpret_cast<int32_t*>(keys[warp]);
+      if (__shfl_sync(kFull, (int)big, src)) add_stage(A, B, w, col, lane, &strict, &bad);
+      const int n = strict ? w.la + w.lb - add_common(w, col, lane)
+                           : add_sort_row(A, B, w, keys[warp], apos, bpos, lane, bad);
+      if (lane == 0) {
+        cnt[wrow] = n;
+        kind[wrow] = strict ? 1 : 0;
+      }
+      __syncwarp();
+    }
   }
   if (bad) set_status(status, KK_ERR_BAD_INDEX);
 }
@@ -216,16 +353,15 @@ k_spadd_sym_warp(CsrView A, CsrView B, int32_t* __restrict__ cnt, int32_t* __res
 // One CTA of kAddCtaThreads per long row (dynamic shared memory kAddCtaMax keys).
 __global__ void __launch_bounds__(kAddCtaThreads)
 k_spadd_sym_cta(CsrView A, CsrView B, int32_t* __restrict__ cnt, int32_t* __restrict__ apos,
-                int32_t* __restrict__ bpos, const int32_t* __restrict__ rows,
-                const int32_t* __restrict__ nrows_dev, int* status) {
+                int32_t* __restrict__ bpos, const int32_t* __restrict__ long_rows, int* status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   u64* key = reinterpret_cast<u64*>(smem_raw);
   __shared__ int scratch[33];
   __shared__ int flags[2];
   const int tid = threadIdx.x;
-  const int nrows = *nrows_dev;
+  const int nrows = long_rows[0];
   for (int q = blockIdx.x; q < nrows; q += gridDim.x) {
-    const int r = rows[q];
+    const int r = long_rows[1 + q];
     const int pa = A.rowptr[r], la = A.rowptr[r + 1] - pa;
     const int pb = B.rowptr[r], lb = B.rowptr[r + 1] - pb;
     const int L = la + lb;
@@ -259,7 +395,7 @@ k_spadd_sym_cta(CsrView A, CsrView B, int32_t* __restrict__ cnt, int32_t* __rest
       int tot;
       const int ex = add_block_scan(first, scratch, &tot);
       if (t < L) {
-        const int slot = run + ex + first - 1;
+        const int slot = (run + ex + first - 1) | (first ? 0 : (int)0x80000000u);
         const int idx = (int)(k & 0x7fffffffull);
         if (k & (1ull << 31)) bpos[pb + idx] = slot;
         else apos[pa + idx] = slot;
@@ -271,80 +407,179 @@ k_spadd_sym_cta(CsrView A, CsrView B, int32_t* __restrict__ cnt, int32_t* __rest
   }
 }
 
-// Numeric: one warp per row; every entry adds its scaled value at its slot.
-__global__ void __launch_bounds__(256)
-k_spadd_num(CsrView A, CsrView B, double alpha, double beta, const int64_t* __restrict__ c_rowptr,
-            const int32_t* __restrict__ apos, const int32_t* __restrict__ bpos,
-            int32_t* __restrict__ c_colind, double* __restrict__ c_vals) {
-  const int lane = threadIdx.x & 31;
-  const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
-  // coefficients of 1 skip the float64 multiply (FP64 is the scarce pipe): the
-  // branches are uniform over the grid, so no multiply is issued at all
-  const bool a1 = alpha == 1.0, b1 = beta == 1.0;
-  for (long long r = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < A.m; r += nw) {
-    const int64_t off = c_rowptr[r];
-    const int pa = A.rowptr[r], pae = A.rowptr[r + 1];
-    if (a1) {
-      for (int p = pa + lane; p < pae; p += 32) {
-        const int64_t s = off + apos[p];
-        c_colind[s] = A.colind[p];
-        atomicAdd(&c_vals[s], A.vals[p]);
-      }
+// Numeric of a row through its slots, by one warp: the first entry of every
+// column is stored, the others are added to it.
+__device__ __forceinline__ void add_scatter(const CsrView& A, const CsrView& B, double alpha, double beta,
+                                            const AddRow& r, const int32_t* __restrict__ apos,
+                                            const int32_t* __restrict__ bpos, int64_t off, int n,
+                                            int32_t* __restrict__ c_colind, double* __restrict__ c_vals, int lane,
+                                            int& mismatch) {
+  bool more = false;
+  auto put = [&](int s, int c, double v) {
+    const int at = s & 0x7fffffff;
+    if (at >= n) {
+      mismatch = 1;
+    } else if (s < 0) {
+      more = true;
     } else {
-      for (int p = pa + lane; p < pae; p += 32) {
-        const int64_t s = off + apos[p];
-        c_colind[s] = A.colind[p];
-        atomicAdd(&c_vals[s], alpha * A.vals[p]);
+      c_colind[off + at] = c;
+      c_vals[off + at] = v;
+    }
+  };
+  for (int t = lane; t < max(r.la, r.lb); t += 32) {
+    const bool a = t < r.la, b = t < r.lb;
+    const int sa = a ? apos[r.pa + t] : 0, sb = b ? bpos[r.pb + t] : 0;
+    const int ca = a ? A.colind[r.pa + t] : 0, cb = b ? B.colind[r.pb + t] : 0;
+    double va = a ? A.vals[r.pa + t] : 0.0, vb = b ? B.vals[r.pb + t] : 0.0;
+    if (alpha != 1.0) va *= alpha;
+    if (beta != 1.0) vb *= beta;
+    if (a) put(sa, ca, va);
+    if (b) put(sb, cb, vb);
+  }
+  __syncwarp();
+  if (!__any_sync(kFull, more)) return;
+  auto add = [&](int s, double v) {
+    const int at = s & 0x7fffffff;
+    if (s < 0 && at < n) atomicAdd(&c_vals[off + at], v);
+  };
+  for (int t = lane; t < r.la; t += 32) add(apos[r.pa + t], alpha == 1.0 ? A.vals[r.pa + t] : alpha * A.vals[r.pa + t]);
+  for (int t = lane; t < r.lb; t += 32) add(bpos[r.pb + t], beta == 1.0 ? B.vals[r.pb + t] : beta * B.vals[r.pb + t]);
+}
+
+// Numeric, T lanes per row as in k_spadd_count.
+template <int T>
+__global__ void __launch_bounds__(kAddRowWarps * 32)
+k_spadd_num(CsrView A, CsrView B, double alpha, double beta, const int64_t* __restrict__ c_rowptr,
+            const int32_t* __restrict__ apos, const int32_t* __restrict__ bpos, const uint8_t* __restrict__ kind,
+            int32_t* __restrict__ c_colind, double* __restrict__ c_vals, int* status) {
+  __shared__ int32_t cols[kAddRowWarps][kAddWarpMax];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tl = lane % T, tm = lane / T;
+  const unsigned team = team_mask<T>(), before = (1u << lane) - 1u;
+  const long long stride = (long long)gridDim.x * kAddRowWarps * (32 / T);
+  int bad = 0, mismatch = 0;
+  struct Row {
+    AddRow r;
+    int n;        // the row's length in C
+    int64_t off;  // ... and its start
+    bool fits, merge;
+  };
+  auto bounds = [&](long long row) -> Row {
+    Row x{{0, 0, 0, 0}, 0, 0, true, true};
+    if (row < A.m) {
+      x.r.pa = A.rowptr[row];
+      x.r.la = A.rowptr[row + 1] - x.r.pa;
+      x.r.pb = B.rowptr[row];
+      x.r.lb = B.rowptr[row + 1] - x.r.pb;
+      x.off = c_rowptr[row];
+      x.n = (int)(c_rowptr[row + 1] - x.off);
+      x.merge = kind[row] != 0;
+      if (x.r.la < 0 || x.r.lb < 0) {
+        mismatch = 1;
+        x.r.la = x.r.lb = 0;
+      }
+      x.fits = x.r.la <= T && x.r.lb <= T && x.merge;
+    }
+    return x;
+  };
+  const long long first = ((long long)blockIdx.x * kAddRowWarps + warp) * (32 / T);
+  for (long long r0 = first; r0 < A.m; r0 += stride) {
+    const long long row = r0 + tm;
+    const Row cur = bounds(row);
+    AddRow r = cur.r;
+    if (!cur.fits) r.la = r.lb = 0;
+    const int64_t off = cur.off;
+    const int n = cur.n;
+    const int ca = tl < r.la ? A.colind[r.pa + tl] : 0x7fffffff;
+    const int cb = tl < r.lb ? B.colind[r.pb + tl] : 0x7fffffff;
+    double va = tl < r.la ? A.vals[r.pa + tl] : 0.0, vb = tl < r.lb ? B.vals[r.pb + tl] : 0.0;
+    if (__any_sync(kFull, cur.fits)) {
+      const bool strict = add_strict<T>(ca, cb, r, A.n, tl, team, &bad);
+      if (!strict) mismatch = 1;  // not the rows of the symbolic call
+      // coefficients of 1 skip the float64 multiply (FP64 is the scarce pipe): the
+      // branches are uniform over the grid
+      if (alpha != 1.0) va *= alpha;
+      if (beta != 1.0) vb *= beta;
+      bool fa, fb;
+      const int ka = add_search<T>(cb, ca, &fa), kb = add_search<T>(ca, cb, &fb);
+      fa = fa && tl < r.la;
+      fb = fb && tl < r.lb;
+      const unsigned ma = __ballot_sync(kFull, fa) & team, mb = __ballot_sync(kFull, fb) & team;
+      if (__any_sync(kFull, fa)) {  // shared columns: A's entry takes the sum
+        const double w = __shfl_sync(kFull, vb, min(ka, T - 1), T);
+        if (fa) va += w;
+      }
+      if (cur.fits) {
+        if (row < A.m && r.la + r.lb - __popc(ma) != n) mismatch = 1;
+        const int sa = tl + ka - __popc(ma & before), sb = tl + kb - __popc(mb & before);
+        if (tl < r.la && sa < n) {
+          c_colind[off + sa] = ca;
+          c_vals[off + sa] = va;
+        }
+        if (tl < r.lb && !fb && sb < n) {
+          c_colind[off + sb] = cb;
+          c_vals[off + sb] = vb;
+        }
       }
     }
-    const int pb = B.rowptr[r], pbe = B.rowptr[r + 1];
-    if (b1) {
-      for (int p = pb + lane; p < pbe; p += 32) {
-        const int64_t s = off + bpos[p];
-        c_colind[s] = B.colind[p];
-        atomicAdd(&c_vals[s], B.vals[p]);
-      }
-    } else {
-      for (int p = pb + lane; p < pbe; p += 32) {
-        const int64_t s = off + bpos[p];
-        c_colind[s] = B.colind[p];
-        atomicAdd(&c_vals[s], beta * B.vals[p]);
+    for (unsigned m = __ballot_sync(kFull, !cur.fits && tl == 0); m; m &= m - 1) {
+      const int src = __ffs(m) - 1;
+      const AddRow w{__shfl_sync(kFull, cur.r.pa, src), __shfl_sync(kFull, cur.r.la, src),
+                     __shfl_sync(kFull, cur.r.pb, src), __shfl_sync(kFull, cur.r.lb, src)};
+      const int64_t woff = __shfl_sync(kFull, (long long)off, src);
+      const int wn = __shfl_sync(kFull, n, src);
+      if (!__shfl_sync(kFull, (int)cur.merge, src)) {
+        add_scatter(A, B, alpha, beta, w, apos, bpos, woff, wn, c_colind, c_vals, lane, mismatch);
+      } else if (w.la + w.lb > kAddWarpMax) {
+        mismatch = 1;
+      } else {
+        bool ok;
+        add_stage(A, B, w, cols[warp], lane, &ok, &bad);
+        if (!ok || add_merge(A, B, alpha, beta, w, cols[warp], woff, wn, c_colind, c_vals, lane) != wn) mismatch = 1;
       }
     }
   }
+  if (mismatch || bad) set_status(status, KK_ERR_STRUCTURE_MISMATCH);
+}
+
+// Lanes per row: enough for the typical row of either matrix.
+int add_team(const CsrView& A, const CsrView& B) {
+  const long long avg = (A.nnz > B.nnz ? A.nnz : B.nnz) / A.m;
+  return avg <= 7 ? 8 : avg <= 14 ? 16 : 32;
+}
+
+int add_grid(const LaunchCtx& ctx, int m, int rows_per_cta) {
+  long long blocks = ((long long)m + rows_per_cta - 1) / rows_per_cta;
+  const long long cap = (long long)ctx.num_sms * 32;
+  return (int)(blocks > cap ? cap : blocks);
 }
 
 }  // namespace
 
 cudaError_t launch_spadd_symbolic(const LaunchCtx& ctx, const CsrView& A, const CsrView& B, int32_t* cnt,
-                                  int32_t* apos, int32_t* bpos, int32_t* long_rows,
-                                  int32_t* long_count) {
+                                  int32_t* apos, int32_t* bpos, uint8_t* kind, int32_t* long_rows) {
   if (A.m <= 0) return cudaSuccess;
-  long long blocks = ((long long)A.m + kAddWarps - 1) / kAddWarps;
-  const long long cap = (long long)ctx.num_sms * 16;
-  if (blocks > cap) blocks = cap;
-  k_spadd_sym_warp<<<(int)blocks, kAddWarps * 32, 0, ctx.stream>>>(A, B, cnt, apos, bpos, long_rows,
-                                                                   long_count, ctx.status);
+  const int T = add_team(A, B), grid = add_grid(ctx, A.m, kAddRowWarps * 32 / T);
+  auto kern = T == 8 ? k_spadd_count<8> : T == 16 ? k_spadd_count<16> : k_spadd_count<32>;
+  kern<<<grid, kAddRowWarps * 32, 0, ctx.stream>>>(A, B, cnt, apos, bpos, kind, long_rows, ctx.status);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
+  // the list's length is on the device: one wave of CTAs strides over it
   const size_t smem = (size_t)kAddCtaMax * 8;
   e = cudaFuncSetAttribute(k_spadd_sym_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  // the long-row count is on the device: one wave of CTAs strides over it
   k_spadd_sym_cta<<<ctx.num_sms * 2, kAddCtaThreads, smem, ctx.stream>>>(A, B, cnt, apos, bpos, long_rows,
-                                                                         long_count, ctx.status);
+                                                                         ctx.status);
   return cudaGetLastError();
 }
 
 cudaError_t launch_spadd_numeric(const LaunchCtx& ctx, const CsrView& A, const CsrView& B, double alpha,
                                  double beta, const int64_t* c_rowptr, const int32_t* apos,
-                                 const int32_t* bpos, int32_t* c_colind, double* c_vals) {
+                                 const int32_t* bpos, const uint8_t* kind, int32_t* c_colind, double* c_vals) {
   if (A.m <= 0) return cudaSuccess;
-  long long blocks = ((long long)A.m * 32 + 255) / 256;
-  const long long cap = (long long)ctx.num_sms * 8;
-  if (blocks > cap) blocks = cap;
-  k_spadd_num<<<(int)blocks, 256, 0, ctx.stream>>>(A, B, alpha, beta, c_rowptr, apos, bpos, c_colind,
-                                                   c_vals);
+  const int T = add_team(A, B), grid = add_grid(ctx, A.m, kAddRowWarps * 32 / T);
+  auto kern = T == 8 ? k_spadd_num<8> : T == 16 ? k_spadd_num<16> : k_spadd_num<32>;
+  kern<<<grid, kAddRowWarps * 32, 0, ctx.stream>>>(A, B, alpha, beta, c_rowptr, apos, bpos, kind, c_colind, c_vals,
+                                                   ctx.status);
   return cudaGetLastError();
 }
 

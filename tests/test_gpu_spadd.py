@@ -135,3 +135,23 @@ def test_spadd_edge_and_interleaved_spgemm():
         ci, va = op.numeric(dA, dA, rp, nnz)
         op.sync()
         check_against_oracle(A, A, rp.cpu().numpy(), ci.cpu().numpy(), va.cpu().numpy())
+
+
+@pytest.mark.parametrize("len_a,len_b", [((0, 8), (0, 8)), ((7, 9), (1, 3)), ((15, 17), (14, 18)), ((31, 33), (30, 34)),
+                                         ((1, 60), (0, 5)), ((100, 128), (100, 128)), ((120, 140), (120, 140))])
+@pytest.mark.parametrize("order", ["sorted", "unsorted", "mixed"])
+def test_spadd_row_lengths(len_a, len_b, order):
+    # rows at either side of what a team's lanes, a warp's shared memory and the
+    # merge hold; mixed: every third row out of order, so a warp has both kinds
+    m, n = 333, 700
+    A = I.random_rows(m, n, *len_a, seed=len_a[1], purpose="rlA")
+    B = I.random_rows(m, n, *len_b, seed=len_b[1] + 7, purpose="rlB")
+    if order != "sorted":
+        for M in (A, B):
+            for r in range(0, m, 1 if order == "unsorted" else 3):
+                s, e = M.rowptr[r], M.rowptr[r + 1]
+                M.colind[s:e] = M.colind[s:e][::-1].copy()
+                M.vals[s:e] = M.vals[s:e][::-1].copy()
+    for al, be in ((1.0, 1.0), (1.5, -0.5)):
+        rp, ci, va = _run(A, B, al, be)
+        _check(A, B, al, be, rp, ci, va, exact=True)
