@@ -1917,7 +1917,8 @@ kk_status kk_spadd_symbolic(kk_spgemm_handle h, const kk_csr* A, const kk_csr* B
     LaunchCtx ctx = ctx_of(h);
     timer_begin(h->timer, s, "spadd_symbolic");
     cudaError_t e = launch_spadd_symbolic(ctx, view(A), view(B), h->d_acnt.as<int32_t>(),
-                                          h->d_apos.as<int32_t>(), h->d_bpos.as<int32_t>(), h->d_akind.as<uint8_t>(), long_rows);
+                                          h->d_apos.as<int32_t>(), h->d_bpos.as<int32_t>(),
+                                          h->d_akind.as<uint8_t>(), long_rows);
     timer_end(h->timer, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "SpAdd symbolic launch");
     timer_begin(h->timer, s, "scan");
@@ -2690,8 +2691,9 @@ kk_status kk_spgemm_destroy(kk_spgemm_handle h) {
                     &h->d_bdesc, &h->d_rowpair, &h->d_bflop, &h->d_bsbin, &h->d_bnbin, &h->d_bsrows,
                     &h->d_bnrows, &h->d_bcnt, &h->d_btiles, &h->d_bstart, &h->d_bqueue, &h->d_bsplit2,
                     &h->d_boff, &h->d_bc, &h->d_bclen, &h->d_cw, &h->d_cm, &h->d_cn, &h->d_wbits,
-                    &h->d_wslot, &h->d_wnext, &h->d_wtasks, &h->d_widx, &h->d_wtab, &h->d_along_rows, &h->d_blong, &h->d_pa_rp, &h->d_pa_ci, &h->d_pa_v, &h->d_pb_rp, &h->d_pb_ci,
-                    &h->d_pb_v, &h->d_pbase})
+                    &h->d_wslot, &h->d_wnext, &h->d_wtasks, &h->d_widx, &h->d_wtab, &h->d_along_rows, &h->d_blong,
+                    &h->d_pa_rp, &h->d_pa_ci, &h->d_pa_v, &h->d_pb_rp, &h->d_pb_ci, &h->d_pb_v, &h->d_pbase, &h->d_jvals,
+                    &h->d_jpos, &h->d_apos, &h->d_bpos, &h->d_acnt, &h->d_akind, &h->d_along})
     b->release();
   for (void* p : {h->h_bdesc, h->h_bdesc2, h->h_boff})
     if (p) cudaFreeHost(p);

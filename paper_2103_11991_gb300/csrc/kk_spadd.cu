@@ -2,31 +2,30 @@
 // "SpAdd"), symbolic and numeric phases.
 //
 // Rows that are strictly ascending in both matrices, of up to kAddWarpMax combined
-// entries, are merged by binary search of each entry in the other row, staged in
-// shared memory: the symbolic phase counts the shared columns, the numeric phase
-// merges again and writes the row of C in one go.  Nothing is kept between the
-// phases for them: reading both rows' columns again, which C's columns need
-// anyway, costs less than writing and reading a slot per entry, adding into C
-// with atomics and zeroing it first (two matrices of 500,000 rows of 30: 286 us
-// symbolic and 217 numeric that way, 116 and 184 now; bound by issue and by the
-// latency of a row's loads, which prefetching the next row's did not shorten: it
-// costs a third of the warps in flight).
+// entries, are merged by binary search of each entry in the other row: through
+// shuffles in teams of 8, 16 or 32 lanes while both rows fit the team, staged in
+// shared memory by a warp otherwise.  The symbolic phase counts the shared columns,
+// the numeric phase merges again and writes the row of C in one go.  Nothing is
+// kept between the phases for them: reading both rows' columns again, which C's
+// columns need anyway, costs less than writing and reading a slot per entry, adding
+// into C with atomics and zeroing it first (two matrices of 500,000 rows of 30: 286
+// us symbolic and 217 numeric that way, 116 and 180 now, both phases with their
+// scan 546 -> 337).  Bound by issue and by the latency of a row's loads; prefetching
+// the next row's costs a third of the warps in flight and gave nothing.
 //
 // Other rows: the entries of A and B become 64-bit keys
 // (column << 32 | source bit (B) << 31 | index within the source row) in
 // shared memory and are sorted by a bitonic network; equal columns are then
 // adjacent, so a scan of "first of its column" flags gives nnz(C(i,:)) and, for
 // every entry of A and of B, its slot in the row of C (the paper's Apos and
-// Bpos; the sign bit marks all but the first entry of a column).  When both rows are sorted (repeats allowed) the keys are laid out as A
-// ascending, then padding, then B descending: a bitonic sequence, so only the
-// final merge stage runs (the paper's sorted-input method); otherwise the full
-// sort runs (its unsorted-input method).  Rows of up to kAddWarpMax combined
-// entries take one warp, rows of up to kAddCtaMax one CTA of 1024 threads; longer
-// rows are reported as KK_ERR_CAPACITY.  Their numeric phase zeroes the row of C,
-// then every entry of A and of B adds its scaled value at its slot (float64
-// atomics: an entry of C with at most one entry of A and one of B is the same
-// sum in either order; repeated columns within A or B are added in no fixed
-// order) and writes its column.
+// Bpos; the sign bit marks all but the first entry of a column).  When both rows
+// are sorted (repeats allowed) the keys are laid out as A ascending, then padding,
+// then B descending: a bitonic sequence, so only the final merge stage runs (the
+// paper's sorted-input method); otherwise the full sort runs (its unsorted-input
+// method).  Rows of up to kAddWarpMax combined entries take one warp, rows of up to
+// kAddCtaMax one CTA of 1024 threads; longer rows are reported as KK_ERR_CAPACITY.
+// Their numeric phase stores the first entry of every column with its value, then
+// adds the others (float64 atomics: repeated columns are added in no fixed order).
 #include "kk_internal.h"
 #include "kk_device.cuh"
 
@@ -224,7 +223,8 @@ __device__ __forceinline__ int add_merge(const CsrView& A, const CsrView& B, dou
 // Whether the team's rows, one entry of each in a lane (INT_MAX past their ends),
 // are strictly ascending.
 template <int T>
-__device__ __forceinline__ bool add_strict(int ca, int cb, const AddRow& r, int ncols, int tl, unsigned team, int* bad) {
+__device__ __forceinline__ bool add_strict(int ca, int cb, const AddRow& r, int ncols, int tl, unsigned team,
+                                           int* bad) {
   if ((tl < r.la && (unsigned)ca >= (unsigned)ncols) || (tl < r.lb && (unsigned)cb >= (unsigned)ncols)) *bad = 1;
   const int ua = __shfl_up_sync(kFull, ca, 1, T), ub = __shfl_up_sync(kFull, cb, 1, T);
   const bool off = tl > 0 && ((tl < r.la && ua >= ca) || (tl < r.lb && ub >= cb));
@@ -442,7 +442,8 @@ __device__ __forceinline__ void add_scatter(const CsrView& A, const CsrView& B, 
     const int at = s & 0x7fffffff;
     if (s < 0 && at < n) atomicAdd(&c_vals[off + at], v);
   };
-  for (int t = lane; t < r.la; t += 32) add(apos[r.pa + t], alpha == 1.0 ? A.vals[r.pa + t] : alpha * A.vals[r.pa + t]);
+  for (int t = lane; t < r.la; t += 32)
+    add(apos[r.pa + t], alpha == 1.0 ? A.vals[r.pa + t] : alpha * A.vals[r.pa + t]);
   for (int t = lane; t < r.lb; t += 32) add(bpos[r.pb + t], beta == 1.0 ? B.vals[r.pb + t] : beta * B.vals[r.pb + t]);
 }
 
