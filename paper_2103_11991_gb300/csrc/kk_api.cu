@@ -146,7 +146,7 @@ struct BinTable {
   int32_t win_bits[kMaxWindowBins];
   int32_t win_bin[kMaxWindowBins];
   int32_t win_kept[kMaxWindowBins];     // 1: rows with kept structure only
-  int32_t win_any_order[kMaxWindowBins];
+  int32_t win_order[kMaxWindowBins];    // 0: sorted B only, 1: any, 2: unsorted only
   long long win_q[kMaxWindowBins];      // largest binning quantity of each window bin
   long long win_ratio[kMaxWindowBins];  // window W only when W <= ratio * flop
 };
@@ -159,7 +159,7 @@ __device__ __forceinline__ uint8_t classify(const BinTable& t, long long q, int 
   const int sp = sorted ? span : t.cols;
   if (sp > 0) {
     for (int w = 0; w < t.nwin; ++w)
-      if (q <= t.win_q[w] && sp <= t.win_bits[w] && (sorted || t.win_any_order[w]) && (!t.win_kept[w] || kept) &&
+      if (q <= t.win_q[w] && sp <= t.win_bits[w] && t.win_order[w] != (sorted ? 2 : 0) && (!t.win_kept[w] || kept) &&
           (long long)t.win_bits[w] <= (q > kRankMinNnz ? t.win_ratio[w] : (long long)kWindowFlopRatio) * flop)
         return (uint8_t)t.win_bin[w];
   }
@@ -1036,7 +1036,9 @@ void build_bins(const kk_spgemm_options& o, bool numeric, std::vector<BinSpec>& 
       out.push_back(BinSpec{kTierWindow, 128, kWindowBits[w], 0, 0,
                             numeric ? kWindowMaxNnz : (long long)9e18});
     // numeric rows without kept structure: by slots, then by window
-    if (numeric)
+    if (!numeric)
+      for (const int32_t bits : kRankBits) out.push_back(BinSpec{kTierRank, 128, bits, 0, 0, kRankMaxFlop});
+    else
       for (const int32_t vmax : kRankNnz)
         for (const int32_t bits : kRankBits) out.push_back(BinSpec{kTierRank, 64, bits, 0, 0, vmax});
   }
@@ -1054,9 +1056,10 @@ BinTable to_table(const std::vector<BinSpec>& bins, bool numeric, int32_t cols) 
       t.win_bin[t.nwin] = (int32_t)b;
       // a heavy row's products are too many for the window's one warp where the
       // wide tier's bit vector is no larger than a window
-      t.win_q[t.nwin] = !numeric && cols <= kWindowBits[kNumWindowClasses - 1] ? kWindowMaxFlop : bins[b].hi;
+      t.win_q[t.nwin] =
+          !numeric && !rank && cols <= kWindowBits[kNumWindowClasses - 1] ? kWindowMaxFlop : bins[b].hi;
       t.win_kept[t.nwin] = numeric && !rank ? 1 : 0;
-      t.win_any_order[t.nwin] = rank ? 1 : 0;
+      t.win_order[t.nwin] = !rank ? 0 : numeric ? 1 : 2;
       t.win_ratio[t.nwin] = rank ? kRankFlopRatio : kWindowFlopRatio;
       ++t.nwin;
     } else {

@@ -138,7 +138,8 @@ constexpr int32_t kWindowFlopRatio = 128;  // window used only when W <= ratio *
 constexpr long long kWindowMaxFlop = 4096;  // symbolic rows of a narrow B (k <= 65,536): flop bound <= this
 
 // Rank tier (kk_rank.cu): numeric rows without kept structure, nnz(C(i,:)) at
-// most kRankNnz[2], span at most kRankBits of the bin.
+// most kRankNnz[2], span at most kRankBits of the bin; symbolic rows of an
+// unsorted B (span: B's columns).
 constexpr int kNumRankBits = 5, kNumRankNnz = 3;
 constexpr int32_t kRankBits[kNumRankBits] = {4096, 8192, 16384, 32768, 65536};
 constexpr int32_t kRankNnz[kNumRankNnz] = {256, 512, 1024};
@@ -148,6 +149,9 @@ constexpr int32_t kRankNnz[kNumRankNnz] = {256, 512, 1024};
 // the team tier, 400 in the rank tier).
 constexpr int32_t kRankFlopRatio = 512;
 constexpr int32_t kRankMinNnz = 32;
+// Symbolic rank rows: flop bound <= this, the line of the window tier for a B as
+// narrow; heavier rows are too many products for one warp and stay where they were.
+constexpr long long kRankMaxFlop = 4096;
 constexpr int kMaxWindowBins = kNumWindowClasses + kNumRankBits * kNumRankNnz;
 
 // Per-row structure kept by the symbolic window kernel for the numeric phase
@@ -193,6 +197,10 @@ cudaError_t launch_num_kept(const LaunchCtx& ctx, const CsrView& A, const CsrVie
                             const WinCacheView& cache, const float2* b_split, const int32_t* b_range_bad,
                             int32_t arith, const int64_t* c_rowptr, const int32_t* rows, int32_t nrows,
                             int32_t* c_colind, double* c_vals);
+
+// Symbolic phase of the rank tier's rows (unsorted B): window of bin.slots columns.
+cudaError_t launch_sym_rank(const LaunchCtx& ctx, const BinSpec& bin, const CsrView& A, const CsrView& B,
+                            const int32_t* rows, int32_t nrows, int32_t* cnt);
 
 // Numeric phase of the rank tier's rows (kk_rank.cu): window of bin.slots
 // columns, at most bin.hi columns of C per row.

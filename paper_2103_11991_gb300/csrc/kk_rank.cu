@@ -128,6 +128,62 @@ __device__ __forceinline__ u64 rank_add(u64 v, bool df, int2 a, float2 b) {
   return (u64)__double_as_longlong(fma(x, y, __longlong_as_double((long long)v)));
 }
 
+// Symbolic phase of rows of an unsorted B: the row's column bits as in k_num_rank,
+// counted as they are set (those that an OR finds clear), one warp per row.  A hash
+// set takes a chain of probes for every product; here the products of four steps
+// are loaded together and each costs one OR (90,666 rows of 510 products in 60,013
+// columns: 657 us by hash, 123 so; bound by the ORs and the load latency).
+constexpr int kSymRankWarps = 4;
+__global__ void __launch_bounds__(kSymRankWarps * 32)
+k_sym_rank(CsrView A, CsrView B, const int32_t* __restrict__ rows, int32_t nrows, int32_t nwords,
+           int32_t* __restrict__ cnt, int* status) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int qbase[kSymRankWarps][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint32_t* bits = reinterpret_cast<uint32_t*>(smem_raw) + (size_t)warp * nwords;
+  uint4* bits4 = reinterpret_cast<uint4*>(bits);
+  int* qb = qbase[warp];
+  const uint32_t words = (uint32_t)nwords;
+  int bad = 0;
+  for (int r = blockIdx.x * kSymRankWarps + warp; r < nrows; r += gridDim.x * kSymRankWarps) {
+    const int i = rows[r];
+    const int pa = A.rowptr[i], pe = A.rowptr[i + 1];
+    for (int q = lane; q < nwords / 4; q += 32) bits4[q] = make_uint4(0u, 0u, 0u, 0u);
+    int c = 0;
+    for (int p0 = pa; p0 < pe; p0 += 32) {
+      int xs = 0, ys = 0;
+      if (p0 + lane < pe) {
+        const int j = A.colind[p0 + lane];
+        xs = B.rowptr[j];
+        ys = B.rowptr[j + 1] - xs;
+      }
+      const FlatRows f = flat_rows(ys, lane);
+      __syncwarp();
+      if (ys > 0) qb[f.k] = xs - f.start;
+      __syncwarp();
+      int seen = 0;
+      for (int f0 = 0; f0 < f.total; f0 += 32 * kRankBatch) {
+        int v[kRankBatch];
+#pragma unroll
+        for (int u = 0; u < kRankBatch; ++u) {
+          const int fl = min(f0 + u * 32 + lane, f.total - 1);
+          v[u] = B.colind[qb[flat_owner(f, f0 + u * 32, lane, seen)] + fl];
+        }
+#pragma unroll
+        for (int u = 0; u < kRankBatch; ++u) {
+          const uint32_t w = (uint32_t)v[u] >> 5, bit = 1u << (v[u] & 31);
+          bad |= w >= words;
+          if (w < words) c += !(atomicOr(&bits[w], bit) & bit);
+        }
+      }
+    }
+    c = team_sum<32>(c, kFull);
+    if (lane == 0) cnt[i] = c;
+    __syncwarp();
+  }
+  if (bad) set_status(status, KK_ERR_CAPACITY);
+}
+
 // SORTED: B's rows strictly ascending; the bits come from the compressed B and
 // a product outside them means that B's structure is not the one they were
 // built from (KK_ERR_STRUCTURE_MISMATCH).  Otherwise the bits come from B's
@@ -420,6 +476,27 @@ __global__ void __launch_bounds__(kRankThreads, 14) k_num_rank(RankArgs g, RankG
 }
 
 }  // namespace
+
+cudaError_t launch_sym_rank(const LaunchCtx& ctx, const BinSpec& bin, const CsrView& A, const CsrView& B,
+                            const int32_t* rows, int32_t nrows, int32_t* cnt) {
+  if (nrows <= 0) return cudaSuccess;
+  const int nwords = rank_geom(B.n < bin.slots ? B.n : bin.slots, 0, 1).words;
+  const size_t smem = (size_t)kSymRankWarps * nwords * 4;
+  cudaError_t e = cudaFuncSetAttribute(k_sym_rank, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sym_rank, kSymRankWarps * 32, smem) != cudaSuccess ||
+      per_sm < 1) {
+    (void)cudaGetLastError();
+    per_sm = 1;
+  }
+  long long blocks = ((long long)nrows + kSymRankWarps - 1) / kSymRankWarps;
+  if (blocks > (long long)ctx.num_sms * per_sm) blocks = (long long)ctx.num_sms * per_sm;
+  timer_begin(ctx.timer, ctx.stream, "sym_rank");
+  k_sym_rank<<<(int)blocks, kSymRankWarps * 32, smem, ctx.stream>>>(A, B, rows, nrows, nwords, cnt, ctx.status);
+  timer_end(ctx.timer, ctx.stream);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_num_rank(const LaunchCtx& ctx, const BinSpec& bin, const CsrView& A, const CsrView& B,
                             int32_t b_sorted, const BComp& bcomp, const float2* b_split,

@@ -303,6 +303,7 @@ cudaError_t launch_symbolic_bin(const LaunchCtx& ctx, const BinSpec& bin, const 
                                 const CsrView& B, int32_t b_sorted, const int32_t* rows,
                                 int32_t nrows, int32_t* cnt) {
   if (nrows <= 0) return cudaSuccess;
+  if (bin.tier == kTierRank) return launch_sym_rank(ctx, bin, A, B, rows, nrows, cnt);
   if (bin.tier == kTierThread) return launch_symbolic_thread(ctx, A, B, rows, nrows, cnt, bin.hi);
   int log2s = 0;
   while ((1 << log2s) < bin.slots) ++log2s;

@@ -58,3 +58,21 @@ def test_rank_rows_at_slot_counts(count, arith):
     assert np.all(np.diff(rp) == count)
     assert (st["num_window_rows"] == m) == (count <= 1024)
     check_against_oracle(A, B, rp, ci, va, exact=count <= 1024 and arith != 2)
+
+
+# the symbolic phase of unsorted rows: word edges of its windows, the largest one,
+# the first size beyond it, and products to either side of its limit
+@pytest.mark.parametrize("n", [4096, 4097, 32768, 65535, 65536, 65537])
+@pytest.mark.parametrize("flop", [510, 4095, 4096, 4097])
+def test_unsorted_symbolic_counts(n, flop):
+    lens = np.array([flop // 8] * 7 + [flop - 7 * (flop // 8)], np.int64)
+    k = 8 * 24
+    lb = np.tile(lens, 24)
+    cols = (I.uniform01(n + flop, "rk.uc", int(lb.sum())) * n).astype(np.int64)
+    cols[:2] = 0, n - 1
+    B = I._from_sorted_coo(k, n, np.repeat(np.arange(k), lb), cols, I.uniform01(flop, "rk.uv", len(cols)) * 2 - 1)
+    A = I.ensure_csr(24, k, np.arange(25) * 8, np.arange(k), I.uniform01(n, "rk.ua", k) * 2 - 1)
+    rp, ci, va, _, st = run_gpu(A, B, arith=1, small_max_rows=0)
+    want = [0] + [len(np.unique(cols[B.rowptr[8 * i]:B.rowptr[8 * i + 8]])) for i in range(24)]
+    assert np.array_equal(rp, np.cumsum(want))
+    check_against_oracle(A, B, rp, ci, va, exact=False)
