@@ -141,7 +141,8 @@ struct BinTable {
   long long hi[kMaxBins];
   int32_t mode[kMaxBins];  // 0 vector, 1 flattened, 2 either, 3 thread tier (flop capped too)
   long long thread_flop;
-  int32_t cols;  // columns of B
+  long long team_max;  // sorted B: rows beyond it leave the team tier
+  int32_t cols;        // columns of B
   int32_t nwin;
   int32_t win_bits[kMaxWindowBins];
   int32_t win_bin[kMaxWindowBins];
@@ -164,7 +165,7 @@ __device__ __forceinline__ uint8_t classify(const BinTable& t, long long q, int 
         return (uint8_t)t.win_bin[w];
   }
   for (int b = 0; b < t.nb; ++b) {
-    if (t.mode[b] == 3) continue;
+    if (t.mode[b] == 3 || (t.mode[b] < 2 && sorted && q > t.team_max)) continue;
     if (q <= t.hi[b] && (t.mode[b] == 2 || t.mode[b] == flat)) return (uint8_t)b;
   }
   return (uint8_t)(t.nb - 1);
@@ -505,7 +506,7 @@ k_scan_final(int32_t m, const int32_t* __restrict__ cnt, const long long* __rest
              const long long* __restrict__ flop, const int32_t* __restrict__ arp,
              const int32_t* __restrict__ row_span, const int32_t* __restrict__ b_sorted,
              int32_t vec_min_len, BinTable ntab, const int32_t* __restrict__ kept_n,
-             int64_t* __restrict__ rowptr, uint8_t* __restrict__ nbin) {
+             const int32_t* __restrict__ wide_slot, int64_t* __restrict__ rowptr, uint8_t* __restrict__ nbin) {
   const int sorted = *b_sorted;
   __shared__ long long scratch[33];
   const long long base = (long long)blockIdx.x * kScanRows + (long long)threadIdx.x * kScanPer;
@@ -524,7 +525,9 @@ k_scan_final(int32_t m, const int32_t* __restrict__ cnt, const long long* __rest
       if (nbin) {
         const int nza = arp[r + 1] - arp[r];
         const int flat = (flop[r] < (long long)vec_min_len * nza) ? 1 : 0;
-        nbin[r] = classify(ntab, v[t], flat, row_span[r], flop[r], sorted, kept_n != nullptr && kept_n[r] >= 0);
+        nbin[r] = wide_slot != nullptr && wide_slot[r] >= 0
+                      ? (uint8_t)(ntab.nb - 1)  // kept bits: chunk tasks
+                      : classify(ntab, v[t], flat, row_span[r], flop[r], sorted, kept_n != nullptr && kept_n[r] >= 0);
       }
       if (r == m - 1) rowptr[m] = run + v[t];
     }
@@ -1048,6 +1051,7 @@ BinTable to_table(const std::vector<BinSpec>& bins, bool numeric, int32_t cols) 
   BinTable t{};
   t.nb = 0;
   t.nwin = 0;
+  t.team_max = (long long)9e18;
   t.cols = cols;
   for (size_t b = 0; b < bins.size(); ++b) {
     const bool rank = bins[b].tier == kTierRank;
@@ -1237,7 +1241,9 @@ kk_status keep_for_symbolic(kk_spgemm_handle h, int32_t m, int64_t wide_rows, co
   h->keep.tasks = tasks ? h->d_wtasks.as<int2>() : nullptr;
   h->keep.kept = &h->d_misc.as<Misc>()->wide_kept;
   h->keep.max_slots = (int32_t)slots;
-  h->keep.min_cnt = tasks ? kRankNnz[kNumRankNnz - 1] : wide_keep_min_cnt(probe, bv.n);
+  h->keep.min_cnt = !tasks                                ? wide_keep_min_cnt(probe, bv.n)
+                    : bv.n <= kRankBits[kNumRankBits - 1] ? kRankNnz[kNumRankNnz - 1]
+                                                          : kRankNnz[0];
   h->keep.stride = (int32_t)stride;
   h->keep.max_chunks = chunks;
   h->keep.max_tasks = (int32_t)ntasks;
@@ -1272,6 +1278,9 @@ void keep_for_numeric(kk_spgemm_handle h, const CsrView& av, const CsrView& bv) 
 // Kept word counts of the rows of this symbolic call (-1: no kept structure),
 // null when it keeps none.
 const int32_t* kept_counts(kk_spgemm_handle h) { return h->cache_valid ? h->d_cn.as<int32_t>() : nullptr; }
+
+// Slots of the rows of this symbolic call kept with chunk tasks (-1: none).
+const int32_t* kept_slots(kk_spgemm_handle h) { return h->keep.tasks ? h->keep.slot : nullptr; }
 
 // The kept structure, if it belongs to these index arrays.  Unless options.debug_checks asks for a check of
 // every product, the arrays' fingerprint is taken again and ctx->fingerprint
@@ -1403,6 +1412,18 @@ static cudaError_t launch_jacobi_rows(kk_spgemm_handle h, const CsrView& av, con
   return cudaGetLastError();
 }
 
+// The symbolic bins' table: rows that the wide tier's kept chunks serve better
+// than the hash kernels leave the team tier.
+static BinTable symbolic_table(kk_spgemm_handle h, int32_t cols) {
+  BinTable t = to_table(h->sym_bins, false, cols);
+  if (h->opt.structure_cache && h->opt.wide_cache_mb >= 0 && wide_symbolic_fits(ctx_of(h), cols) &&
+      wide_numeric_fits(ctx_of(h), cols)) {
+    const long long least = wide_keep_min_flop(wide_word_count(cols)) - 1;
+    t.team_max = least > kKeepEarlyFlop ? least : kKeepEarlyFlop;
+  }
+  return t;
+}
+
 // Analysis of A with teams of T lanes, one resident wave of blocks (the kernel
 // strides over rows).
 // bin receives the symbolic bin ids; with STATS, stat the learned form's row
@@ -1418,7 +1439,7 @@ static void launch_analyze_a_t(kk_spgemm_handle h, const CsrView& av, const CsrV
   }
   const int64_t m = LISTED ? lr.most : av.m;
   kern<<<grid_for(m * T, 256, h->num_sms * (per_sm > 0 ? per_sm : 1)), 256, 0, s>>>(
-      av, bv.rowptr, bv.colind, bv.m, &dm->sorted, to_table(h->sym_bins, false, bv.n), h->opt.team_vec_min_len,
+      av, bv.rowptr, bv.colind, bv.m, &dm->sorted, symbolic_table(h, bv.n), h->opt.team_vec_min_len,
       h->d_flop.as<long long>(), bin, h->d_rowlo.as<int32_t>(), h->d_span.as<int32_t>(), stat,
       &dm->total_flop, &dm->status, lr);
 }
@@ -1683,7 +1704,8 @@ kk_status kk_spgemm_symbolic(kk_spgemm_handle h, const kk_csr* A, const kk_csr* 
     k_scan_final<<<nblk_scan, kScanBlock, 0, s>>>(
         m, h->d_cnt.as<int32_t>(), h->d_scan.as<long long>(), h->d_flop.as<long long>(), av.rowptr,
         h->d_span.as<int32_t>(), &dm->sorted, h->opt.team_vec_min_len,
-        to_table(h->num_bins, true, bv.n), kept_counts(h), c_rowptr, h->d_nbin.as<uint8_t>());
+        to_table(h->num_bins, true, bv.n), kept_counts(h), kept_slots(h), c_rowptr,
+        h->d_nbin.as<uint8_t>());
     timer_end(h->timer, s);
     KK_CUDA(h, cudaGetLastError(), "scan launch");
     if ((st = run_binning(h, m, h->d_nbin.as<uint8_t>(), nbn, h->d_nrows.as<int32_t>(), num_start)) != KK_OK)
@@ -1880,7 +1902,8 @@ kk_status run_scan(kk_spgemm_handle h, int32_t m, const int32_t* cnt, int64_t* o
   k_scan_final<<<nblk, kScanBlock, 0, s>>>(m, cnt, h->d_scan.as<long long>(), h->d_flop.as<long long>(),
                                            av.rowptr, h->d_span.as<int32_t>(), &dm->sorted,
                                            h->opt.team_vec_min_len, to_table(h->num_bins, true, cols),
-                                           nbin ? kept_counts(h) : nullptr, out, nbin);
+                                           nbin ? kept_counts(h) : nullptr, nbin ? kept_slots(h) : nullptr,
+                                           out, nbin);
   KK_CUDA(h, cudaGetLastError(), "scan launch");
   return KK_OK;
 }

@@ -224,6 +224,15 @@ cudaError_t launch_analyze_b(const LaunchCtx& ctx, const CsrView& B, int32_t* so
 // Arithmetic mode for the numeric kernels.
 enum ArithMode : int32_t { kArithF64 = 1, kArithDF32 = 2 };
 
+// Sorted B: symbolic rows of more than kKeepEarlyFlop products that the wide tier
+// would keep (wide_keep_min_flop) leave the team tier for it, because its chunks
+// serve their numeric phase (scale-18 R-MAT square 31.2 -> 30.1 ms, learned scale-15
+// form 2.15 -> 1.97).
+constexpr long long kKeepEarlyFlop = 768;
+// Products from which k_sym_wide keeps a row's bits for chunk tasks: fewer leave
+// most words empty, and it walks a summary instead.
+__host__ __device__ inline int wide_keep_min_flop(int words) { return words / 4; }
+
 // Symbolic launch: rows[0..nrows) of A (a device array) get cnt[i] = nnz(C(i,:)).
 cudaError_t launch_symbolic_bin(const LaunchCtx& ctx, const BinSpec& bin, const CsrView& A,
                                 const CsrView& B, int32_t b_sorted, const int32_t* rows,

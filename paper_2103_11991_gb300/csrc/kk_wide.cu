@@ -534,7 +534,7 @@ k_sym_wide(CsrView A, CsrView B, BComp bc, int32_t words, uint32_t sum_off, uint
     // few words touched: walk the summary instead of all words.  Such a row
     // keeps nothing; with chunk tasks the line lies lower, because a kept row's
     // numeric phase is much the faster one.
-    const bool sparse = flop[i] < (long long)(keep.tasks ? words / 4 : words);
+    const bool sparse = flop[i] < (long long)(keep.tasks ? wide_keep_min_flop(words) : words);
     const int lng = wide_piece(flop, i, A.rowptr[i], A.rowptr[i + 1]);
     int c = 0;
     if (sparse) {

@@ -62,3 +62,32 @@ def test_chunks_refresh_other_arrays_and_jacobi():
         ci, va = op.numeric(dA, dB2, rp, nnz)
         op.sync()
         check_against_oracle(A, B, rp.cpu().numpy(), ci.cpu().numpy(), va.cpu().numpy())
+
+
+# rows that leave the hash kernels for the chunks by their products: either side of
+# that line (769 or a 128th of B's columns) and of the columns a kept row needs
+@pytest.mark.parametrize("k", [65536, 65537, 98304, 131072, 262144, 262145])
+@pytest.mark.parametrize("flop,count", [(767, 767), (768, 256), (768, 257), (769, 256), (769, 257), (1023, 400), (1024, 400), (1040, 520),
+                                        (2047, 700), (2048, 700)])
+def test_rows_beyond_the_hash_kernels(k, flop, count):
+    m = 40
+    full, rest = divmod(flop, count)
+    lens = np.tile([count] * full + ([rest] if rest else []), m)
+    per = len(lens) // m
+    pick = [np.sort(np.argsort(I.uniform01(i, "ch.p%d" % flop, k))[:count]) for i in range(m)]
+    cols = np.concatenate([np.concatenate([pick[i]] * full + ([pick[i][:rest]] if rest else [])) for i in range(m)])
+    B = I.ensure_csr(m * per, k, np.concatenate([[0], np.cumsum(lens)]), cols,
+                     I.uniform01(k, "ch.q", len(cols)) * 2 - 1)
+    A = I.ensure_csr(m, m * per, np.arange(m + 1) * per, np.arange(m * per),
+                     I.uniform01(flop, "ch.r", m * per) * 2 - 1)
+    rp, ci, va, _, st = run_gpu(A, B, arith=1, small_max_rows=0)
+    assert np.all(np.diff(rp) == count)
+    early = flop >= max(769, k // 128)
+    if k in (98304, 131072, 262144):  # every row's span is beyond the window tier's
+        assert (st["sym_cta_rows"] + st["sym_dense_rows"] == m) == early
+        assert st["num_dense_rows"] == (m if early and count > 256 else 0)
+    check_against_oracle(A, B, rp, ci, va)
+    few = run_gpu(A, B, arith=1, small_max_rows=0, wide_cache_mb=1)  # most rows find no slot
+    check_against_oracle(A, B, *few[:3])
+    plain = run_gpu(A, B, arith=1, small_max_rows=0, structure_cache=0)
+    assert np.array_equal(rp, plain[0]) and np.array_equal(ci, plain[1])
