@@ -226,12 +226,14 @@ enum ArithMode : int32_t { kArithF64 = 1, kArithDF32 = 2 };
 
 // Sorted B: symbolic rows of more than kKeepEarlyFlop products that the wide tier
 // would keep (wide_keep_min_flop) leave the team tier for it, because its chunks
-// serve their numeric phase (scale-18 R-MAT square 31.2 -> 30.1 ms, learned scale-15
-// form 2.15 -> 1.97).
-constexpr long long kKeepEarlyFlop = 768;
+// serve their numeric phase.
+constexpr long long kKeepEarlyFlop = 512;
 // Products from which k_sym_wide keeps a row's bits for chunk tasks: fewer leave
-// most words empty, and it walks a summary instead.
-__host__ __device__ inline int wide_keep_min_flop(int words) { return words / 4; }
+// most words empty, and it walks a summary instead.  Measured with the line above,
+// R-MAT squares of scale 18 and 19: words / 4 and 768 30.4 and 92.6 ms, words / 11
+// and 768 28.7 and 91.7, words / 16 and 512 28.5 and 91.0, words / 24 and 384 28.4
+// and 90.8 (hardly less, for more rows to hold).
+__host__ __device__ inline int wide_keep_min_flop(int words) { return words / 16; }
 
 // Symbolic launch: rows[0..nrows) of A (a device array) get cnt[i] = nnz(C(i,:)).
 cudaError_t launch_symbolic_bin(const LaunchCtx& ctx, const BinSpec& bin, const CsrView& A,

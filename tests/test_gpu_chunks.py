@@ -65,9 +65,10 @@ def test_chunks_refresh_other_arrays_and_jacobi():
 
 
 # rows that leave the hash kernels for the chunks by their products: either side of
-# that line (769 or a 128th of B's columns) and of the columns a kept row needs
+# that line (513 or a 512th of B's columns) and of the columns a kept row needs
 @pytest.mark.parametrize("k", [65536, 65537, 98304, 131072, 262144, 262145])
-@pytest.mark.parametrize("flop,count", [(767, 767), (768, 256), (768, 257), (769, 256), (769, 257), (1023, 400), (1024, 400), (1040, 520),
+@pytest.mark.parametrize("flop,count", [(511, 300), (512, 257), (513, 256), (513, 257), (767, 767),
+                                        (768, 256), (768, 257), (769, 256), (769, 257), (1023, 400), (1024, 400), (1040, 520),
                                         (2047, 700), (2048, 700)])
 def test_rows_beyond_the_hash_kernels(k, flop, count):
     m = 40
@@ -82,7 +83,7 @@ def test_rows_beyond_the_hash_kernels(k, flop, count):
                      I.uniform01(flop, "ch.r", m * per) * 2 - 1)
     rp, ci, va, _, st = run_gpu(A, B, arith=1, small_max_rows=0)
     assert np.all(np.diff(rp) == count)
-    early = flop >= max(769, k // 128)
+    early = flop >= max(513, k // 512)
     if k in (98304, 131072, 262144):  # every row's span is beyond the window tier's
         assert (st["sym_cta_rows"] + st["sym_dense_rows"] == m) == early
         assert st["num_dense_rows"] == (m if early and count > 256 else 0)
