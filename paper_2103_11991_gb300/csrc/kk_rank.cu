@@ -1,5 +1,5 @@
-// Rank tier of the numeric phase: rows of up to kRankMaxNnz columns whose span
-// fits a bit vector of at most 65,536 columns, one warp per row.
+// Rank tier: numeric rows of up to 1,024 columns whose span fits a bit vector of at
+// most 65,536 columns, one or two warps per row; symbolic rows of an unsorted B.
 //
 // The paper's dense accumulator (Sec. "Standard SpGEMM Kernel": bit vector and
 // scalar array) over the row's span: the row's column bits are set, one pass
@@ -13,10 +13,11 @@
 // 16-byte piece of 128 columns, two pieces per warp scan (their counts packed
 // into one register), about 25 instructions per 8,192 columns.  A list of the
 // non-empty words costs more than that (summary bits, ordered list, a scan and
-// an expansion per word; with a CTA of four warps per row and three barriers it
-// took 106 us for the 2,993 rows of a 3,001-row random product and 8.9 ms for
-// the window rows of a 256-pair batch, see the design notes for this kernel's
-// figures).  C's columns come from the products themselves (each writes its
+// an expansion per word; with a CTA of four warps per row and three barriers the
+// window rows of a 256-pair batch took 8.9 ms and its hash rows 4.6, together 5.2
+// here).  90,666 rows of about 500 columns of an unsorted B take 592 us: 1,250 with
+// an entry of A at a time, 905 flattened, 800 without branches, then two warps per
+// row where a row's shared memory leaves few of them on an SM.  C's columns come from the products themselves (each writes its
 // column's offset beside its value), not from expanding the bits.
 //
 // The row's products are walked flattened, 32 per step whatever the lengths of

@@ -862,10 +862,12 @@ k_num_wide(CsrView A, CsrView B, int32_t words, int32_t vcap, uint32_t sum_off, 
       }
     };
     if (sparse) {
-      if (lng) wide_walk_long<BLOCK, true, false>(A, B, none, pa, pe, walk.ls, lng, bad, add_smem, nullptr, nullptr, i);
+      if (lng)
+        wide_walk_long<BLOCK, true, false>(A, B, none, pa, pe, walk.ls, lng, bad, add_smem, nullptr, nullptr, i);
       else wide_walk<BLOCK, true, false>(A, B, none, pa, pe, walk.ws, bad, add_smem, i);
     } else {
-      if (lng) wide_walk_long<BLOCK, true, false>(A, B, none, pa, pe, walk.ls, lng, bad, add_glob, nullptr, nullptr, i);
+      if (lng)
+        wide_walk_long<BLOCK, true, false>(A, B, none, pa, pe, walk.ls, lng, bad, add_glob, nullptr, nullptr, i);
       else wide_walk<BLOCK, true, false>(A, B, none, pa, pe, walk.ws, bad, add_glob, i);
     }
     if (sparse) {
