@@ -1218,8 +1218,8 @@ kk_status keep_for_symbolic(kk_spgemm_handle h, int32_t m, int64_t wide_rows, co
   if (!wide_symbolic_fits(probe, bv.n) || !wide_numeric_fits(probe, bv.n)) return KK_OK;
   const size_t words = (size_t)wide_word_count(bv.n);
   // sorted B: rows of more columns than the rank tier takes, computed in chunks;
-  // unsorted B: rows whose values do not fit the wide kernel's shared memory
-  const bool tasks = h->b_sorted != 0;
+  // otherwise: rows whose values do not fit the wide kernel's shared memory
+  const bool tasks = h->b_sorted != 0 && bv.n <= kChunkMaxCols;
   const int32_t chunks = tasks ? wide_max_chunks(bv.n) : 0;
   const size_t stride = words + ((size_t)chunks * 2 + 3) / 4 * 4;
   const size_t budget = h->opt.wide_cache_mb > 0 ? ((size_t)h->opt.wide_cache_mb << 20) : h->dev_total / 8;
@@ -1416,8 +1416,8 @@ static cudaError_t launch_jacobi_rows(kk_spgemm_handle h, const CsrView& av, con
 // than the hash kernels leave the team tier.
 static BinTable symbolic_table(kk_spgemm_handle h, int32_t cols) {
   BinTable t = to_table(h->sym_bins, false, cols);
-  if (h->opt.structure_cache && h->opt.wide_cache_mb >= 0 && wide_symbolic_fits(ctx_of(h), cols) &&
-      wide_numeric_fits(ctx_of(h), cols)) {
+  if (cols <= kChunkMaxCols && h->opt.structure_cache && h->opt.wide_cache_mb >= 0 &&
+      wide_symbolic_fits(ctx_of(h), cols) && wide_numeric_fits(ctx_of(h), cols)) {
     const long long least = wide_keep_min_flop(wide_word_count(cols)) - 1;
     t.team_max = least > kKeepEarlyFlop ? least : kKeepEarlyFlop;
   }

@@ -224,6 +224,11 @@ cudaError_t launch_analyze_b(const LaunchCtx& ctx, const CsrView& B, int32_t* so
 // Arithmetic mode for the numeric kernels.
 enum ArithMode : int32_t { kArithF64 = 1, kArithDF32 = 2 };
 
+// Column chunks only where B has at most this many columns: R-MAT square of scale 19
+// (2^19 columns) 91.0 ms with them, 102.1 with one CTA per row; of scale 20 296.5 and
+// 273.0 (chunks also end every 65,536 columns, so a wide B has more of them per row,
+// and each walks all of the row's entries of A).
+constexpr int32_t kChunkMaxCols = 1 << 19;
 // Sorted B: symbolic rows of more than kKeepEarlyFlop products that the wide tier
 // would keep (wide_keep_min_flop) leave the team tier for it, because its chunks
 // serve their numeric phase.

@@ -92,3 +92,18 @@ def test_rows_beyond_the_hash_kernels(k, flop, count):
     check_against_oracle(A, B, *few[:3])
     plain = run_gpu(A, B, arith=1, small_max_rows=0, structure_cache=0)
     assert np.array_equal(rp, plain[0]) and np.array_equal(ci, plain[1])
+
+
+# the widest B whose kept rows are computed in chunks, and the next: rows with few
+# and with many columns, kept, without room to keep them, and with nothing kept
+@pytest.mark.parametrize("k", [524288, 524289])
+@pytest.mark.parametrize("la,lb", [((6, 9), (300, 500)), ((200, 300), (40, 80))])
+def test_chunks_at_the_widest_b(k, la, lb):
+    A = I.random_rows(50, 600, *la, seed=k + la[0], purpose="chX")
+    B = I.random_rows(600, k, *lb, seed=k + lb[0], purpose="chY")
+    kept = run_gpu(A, B, arith=1, small_max_rows=0)
+    check_against_oracle(A, B, *kept[:3])
+    for other in (dict(wide_cache_mb=1), dict(structure_cache=0)):
+        got = run_gpu(A, B, arith=1, small_max_rows=0, **other)
+        check_against_oracle(A, B, *got[:3])
+        assert np.array_equal(kept[0], got[0]) and np.array_equal(kept[1], got[1])
