@@ -1,6 +1,8 @@
 // Learned row-capacity predictor: row features, capacity labels, and the
 // training kernels (forward, backward, Adam) and inference of the MLP
 // declared in kk_learned.h.  Everything runs on the GPU in float32.
+#include <cooperative_groups.h>
+
 #include <cmath>
 #include <cstdio>
 #include <vector>
@@ -134,14 +136,19 @@ constexpr int kMlpBlock = 128;
 // 16-byte reads along the samples are aligned and spread over the banks; a
 // layer's weights are broadcasts).  The gradient of a weight is then the inner
 // product of two rows, and every thread owns the same weights for all of the
-// CTA's tiles: 4 of W2, 2 of W3, 1 of W1 and one bias, in registers, added to
-// grad once at the end.
+// CTA's tiles: 4 of W2, 2 of W3, 1 of W1 and one bias, in registers.  At the end a
+// cluster of 8 CTAs adds its sums as a tree through distributed shared memory, then
+// to grad: a chain of 128 to 608 float32 additions, one per CTA, cost 2.2 us less at
+// 4,096 samples but was 1.8 times further from the float64 gradient than a warp sum
+// per weight (relative error at 4,096 and 20,001 samples, mean of 12 seeds: warp sums
+// 9.5e-8 and 2.0e-7, the chain 1.7e-7 and 3.4e-7, this 8.0e-8 and 1.4e-7).
 // What bounds it: issue and shared-memory reads; a tile is about 1,000
 // instructions a warp.  A thread per sample with a warp sum per weight (1,872 of
-// five shuffles, then atomics) took 252 us for 4,096 samples; this takes 13.6.
+// five shuffles, then atomics) took 252 us for 4,096 samples; this takes 14.8.
 constexpr int kGradThreads = 256;
 constexpr int kGradLd = 36;
 constexpr int kGradMaxCtas = 608;
+constexpr int kGradCluster = 8;
 struct GradSmem {
   float P[kMlpParams];
   float x[kMlpF][kGradLd];
@@ -149,22 +156,23 @@ struct GradSmem {
   float z[kMlpC][kGradLd];
   float dz[kMlpC][kGradLd];
   float dh2[kMlpH][kGradLd], dh1[kMlpH][kGradLd];
+  float loss;
 };
 
 __device__ __forceinline__ float row_dot(const float* a, const float* b) {
-  float s = 0.0f;
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
   for (int t = 0; t < 32; t += 4) {
     const float4 u = *reinterpret_cast<const float4*>(a + t), v = *reinterpret_cast<const float4*>(b + t);
-    s = fmaf(u.x, v.x, s);
-    s = fmaf(u.y, v.y, s);
-    s = fmaf(u.z, v.z, s);
-    s = fmaf(u.w, v.w, s);
+    s.x = fmaf(u.x, v.x, s.x);
+    s.y = fmaf(u.y, v.y, s.y);
+    s.z = fmaf(u.z, v.z, s.z);
+    s.w = fmaf(u.w, v.w, s.w);
   }
-  return s;
+  return (s.x + s.y) + (s.z + s.w);
 }
 
-__global__ void __launch_bounds__(kGradThreads)
+__global__ void __cluster_dims__(kGradCluster) __launch_bounds__(kGradThreads)
 k_mlp_loss_grad(int32_t n, int32_t start, int32_t count, long long pa, long long pb,
                 const float* __restrict__ X, const int32_t* __restrict__ y,
                 const float* __restrict__ Pg, float* __restrict__ grad, float* __restrict__ loss) {
@@ -304,32 +312,53 @@ k_mlp_loss_grad(int32_t n, int32_t start, int32_t count, long long pa, long long
     g1 += row_dot(sm.x[w], sm.dh1[lane]);
     if (tid < 2 * kMlpH + kMlpC) {
       const float* row = tid < kMlpH ? sm.dh1[tid] : tid < 2 * kMlpH ? sm.dh2[tid - kMlpH] : sm.dz[tid - 2 * kMlpH];
-      float a = 0.0f;
+      float a[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int t = 0; t < 32; ++t) a += row[t];
-      gb += a;
+      for (int t = 0; t < 32; ++t) a[t & 3] += row[t];
+      gb += (a[0] + a[1]) + (a[2] + a[3]);
     }
     __syncthreads();
   }
+  __syncthreads();
+  // this CTA's sums in the place of the weights, then the cluster's as a tree
 #pragma unroll
   for (int u = 0; u < 2; ++u)
 #pragma unroll
-    for (int v = 0; v < 2; ++v) atomicAdd(&grad[kOffW2 + (j2 + u) * kMlpH + k2 + v], g2[2 * u + v]);
+    for (int v = 0; v < 2; ++v) sm.P[kOffW2 + (j2 + u) * kMlpH + k2 + v] = g2[2 * u + v];
 #pragma unroll
-  for (int v = 0; v < 2; ++v) atomicAdd(&grad[kOffW3 + k3 * kMlpC + c3 + v], g3[v]);
-  atomicAdd(&grad[kOffW1 + w * kMlpH + lane], g1);
-  if (tid < 2 * kMlpH + kMlpC)
-    atomicAdd(&grad[tid < kMlpH ? kOffB1 + tid : tid < 2 * kMlpH ? kOffB2 + tid - kMlpH : kOffB3 + tid - 2 * kMlpH], gb);
+  for (int v = 0; v < 2; ++v) sm.P[kOffW3 + k3 * kMlpC + c3 + v] = g3[v];
+  sm.P[kOffW1 + w * kMlpH + lane] = g1;
+  if (tid < kMlpH) sm.P[kOffB1 + tid] = gb;
+  else if (tid < 2 * kMlpH) sm.P[kOffB2 + tid - kMlpH] = gb;
+  else if (tid < 2 * kMlpH + kMlpC) sm.P[kOffB3 + tid - 2 * kMlpH] = gb;
   if (w == 0) {
     lsum = warp_sum_f(lsum);
-    if (lane == 0) atomicAdd(loss, lsum);
+    if (lane == 0) sm.loss = lsum;
   }
+  auto cluster = cooperative_groups::this_cluster();
+  cluster.sync();
+  auto sum = [&](float* at) {
+    float v[kGradCluster];
+#pragma unroll
+    for (int c = 0; c < kGradCluster; ++c) v[c] = *cluster.map_shared_rank(at, c);
+#pragma unroll
+    for (int o = kGradCluster / 2; o > 0; o >>= 1)
+#pragma unroll
+      for (int c = 0; c < o; ++c) v[c] += v[c + o];
+    return v[0];
+  };
+  const int rank = (int)cluster.block_rank();
+  for (int i = rank * kGradThreads + tid; i < kMlpParams; i += kGradCluster * kGradThreads)
+    atomicAdd(&grad[i], sum(&sm.P[i]));
+  if (rank == kGradCluster - 1 && tid == kGradThreads - 1) atomicAdd(loss, sum(&sm.loss));
+  cluster.sync();  // the peers' shared memory is read until here
 }
 
-// CTAs of k_mlp_loss_grad: one per tile up to four per SM.
+// CTAs of k_mlp_loss_grad: one per tile up to four per SM, in whole clusters.
 int grad_ctas(int count) {
   const int tiles = (count + 31) / 32;
-  return tiles < kGradMaxCtas ? tiles : kGradMaxCtas;
+  const int ctas = (tiles + kGradCluster - 1) / kGradCluster * kGradCluster;
+  return ctas < kGradMaxCtas ? ctas : kGradMaxCtas;
 }
 
 // grad and loss to zero, in one launch.
