@@ -24,6 +24,7 @@
 // the row's barrier; each lane issues kWideU loads before it uses them.
 #include "kk_internal.h"
 #include "kk_device.cuh"
+#include "kk_walk.h"
 
 namespace kk {
 namespace {
@@ -1080,12 +1081,11 @@ k_num_chunk(CsrView A, CsrView B, int32_t words, const int64_t* __restrict__ c_r
 #pragma unroll
         for (int u = 0; u < kChunkU; ++u) {
           const int fb = f + u * 32;
-          const unsigned at = (unsigned)(sm.start[min(seen + lane, np)] - fb);
-          const unsigned m = __reduce_or_sync(kFull, at < 32u ? 1u << at : 0u);
-          const int own = min(seen + __popc(m & (0xffffffffu >> (31 - lane))) - 1, np - 1);
+          const unsigned m = __reduce_or_sync(kFull, walk_start_bit(sm.start[min(seen + lane, np)], fb, f_hi));
+          const int own = seen + __popc(m & walk_upto(lane)) - 1;
           seen += __popc(m);
           const int4 in = sm.piece[own];
-          const int q = in.x + min(fb + lane, f_hi - 1);
+          const int q = in.x + walk_product(fb, lane, f_hi);  // an entry of the piece, past the run too
           c[u] = bcol[q];
           y[u] = bval[q];
           x[u] = __hiloint2double(in.w, in.z);
