@@ -879,6 +879,7 @@ struct kk_spgemm_handle_s {
   DevBuf d_cm;         // uint32[m * kCacheWords]
   DevBuf d_cn;         // int32[m]
   bool cache_valid = false;
+  bool fp_taken = false;  // the symbolic call's fingerprint is in d_misc
   // wide-tier bit vectors kept by the symbolic phase
   DevBuf d_wbits, d_wslot, d_wnext, d_wtasks, d_widx, d_wtab;
   DevBuf d_along_rows, d_blong;  // long rows of A and of B (analysis)
@@ -1182,6 +1183,15 @@ kk_status fingerprint(kk_spgemm_handle h, const CsrView& av, const CsrView& bv,
   return KK_OK;
 }
 
+// The fingerprint of a symbolic call's index arrays, once per call: with it the
+// numeric phase knows whether what was kept is still that of its arrays.
+kk_status symbolic_fingerprint(kk_spgemm_handle h, const CsrView& av, const CsrView& bv) {
+  if (h->fp_taken) return KK_OK;
+  KK_TRY(fingerprint(h, av, bv, &h->d_misc.as<Misc>()->fp[0]));
+  h->fp_taken = true;
+  return KK_OK;
+}
+
 // Structure cache for the symbolic window kernel: every row starts without
 // kept structure (n = -1); null pointers when the option is off or no row of
 // the call takes the window tier.  The index arrays' fingerprint is recorded
@@ -1197,8 +1207,7 @@ kk_status cache_for_symbolic(kk_spgemm_handle h, int32_t m, bool any_window, con
   KK_CUDA(h, cudaMemsetAsync(h->d_cn.p, 0xFF, sizeof(int32_t) * (size_t)m, h->stream), "memset cache");
   *out = WinCache{h->d_cw.as<uint16_t>(), h->d_cm.as<uint32_t>(), h->d_cn.as<int32_t>(),
                   &h->d_misc.as<Misc>()->kept};
-  kk_status st = fingerprint(h, av, bv, &h->d_misc.as<Misc>()->fp[0]);
-  if (st != KK_OK) return st;
+  KK_TRY(symbolic_fingerprint(h, av, bv));
   h->cache_valid = true;
   h->cache_key[0] = av.rowptr;
   h->cache_key[1] = av.colind;
@@ -1258,6 +1267,7 @@ kk_status keep_for_symbolic(kk_spgemm_handle h, int32_t m, int64_t wide_rows, co
     KK_CUDA(h, launch_chunk_index(ctx_of(h), bv, h->d_widx.as<int32_t>(), h->d_widx.as<int32_t>() + bv.m,
                                   h->d_wtab.as<int32_t>()),
             "index launch");
+    KK_TRY(symbolic_fingerprint(h, av, bv));
   }
   h->keep_valid = true;
   h->keep_key[0] = av.rowptr;
@@ -1301,13 +1311,17 @@ kk_status cache_view(kk_spgemm_handle h, const CsrView& av, const CsrView& bv, W
 }
 
 // The rows kept with chunk tasks; *skip_wide = true when no row of the wide
-// tier is left (start: the bins' row starts).
+// tier is left (start: the bins' row starts).  Their bits and the positions in
+// B's rows are read as they were kept, so the kernel compares the index arrays'
+// fingerprints first, whatever options.debug_checks says.
 kk_status launch_kept_chunks(kk_spgemm_handle h, const LaunchCtx& ctx, const CsrView& av, const CsrView& bv,
                              const std::vector<int32_t>& start, const int64_t* c_rowptr, int32_t* c_colind,
                              double* c_vals, bool* skip_wide) {
   *skip_wide = false;
   if (!ctx.keep.tasks || h->wide_kept <= 0) return KK_OK;
-  KK_CUDA(h, launch_num_chunk(ctx, av, bv, c_rowptr, c_colind, c_vals), "chunk launch");
+  Misc* dm = h->d_misc.as<Misc>();
+  if (!ctx.fingerprint) KK_TRY(fingerprint(h, av, bv, &dm->fp[1]));
+  KK_CUDA(h, launch_num_chunk(ctx, av, bv, dm->fp, c_rowptr, c_colind, c_vals), "chunk launch");
   h->stats[9] += 1;
   int64_t wide = 0;
   for (size_t b = 0; b < h->num_bins.size(); ++b)
@@ -1568,6 +1582,7 @@ kk_status kk_spgemm_symbolic(kk_spgemm_handle h, const kk_csr* A, const kk_csr* 
   if (A->n != B->m) return fail(h, KK_ERR_INVALID_ARG, "A.n != B.m");
   if (!c_rowptr || !nnz_c) return fail(h, KK_ERR_INVALID_ARG, "c_rowptr / nnz_c is NULL");
   h->have_symbolic = false;
+  h->fp_taken = false;
   const int32_t m = A->m;
   const CsrView av = view(A), bv = view(B);
   cudaStream_t s = h->stream;
@@ -2037,6 +2052,7 @@ kk_status kk_spgemm_learned_symbolic(kk_spgemm_handle h, const kk_csr* A, const 
   if (A->n != B->m) return fail(h, KK_ERR_INVALID_ARG, "A.n != B.m");
   if (!c_rowptr || !nnz_c) return fail(h, KK_ERR_INVALID_ARG, "c_rowptr / nnz_c is NULL");
   h->have_symbolic = false;
+  h->fp_taken = false;
   h->small = false;
   h->learned_valid = false;
   h->keep = WideKeep{};

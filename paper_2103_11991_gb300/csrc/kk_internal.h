@@ -273,8 +273,9 @@ long long wide_max_tasks(int32_t k, long long flops, long long slots);  // of `s
 int32_t wide_index_stride(int32_t k);
 int32_t wide_index_slots(const CsrView& B);
 cudaError_t launch_chunk_index(const LaunchCtx& ctx, const CsrView& B, int32_t* slot, int32_t* row, int32_t* tab);
-cudaError_t launch_num_chunk(const LaunchCtx& ctx, const CsrView& A, const CsrView& B, const int64_t* c_rowptr,
-                             int32_t* c_colind, double* c_vals);
+// (fp: structure fingerprints of the symbolic call and of this one).
+cudaError_t launch_num_chunk(const LaunchCtx& ctx, const CsrView& A, const CsrView& B, const unsigned long long* fp,
+                             const int64_t* c_rowptr, int32_t* c_colind, double* c_vals);
 
 cudaError_t launch_symbolic_thread(const LaunchCtx& ctx, const CsrView& A, const CsrView& B,
                                    const int32_t* rows, int32_t nrows, int32_t* cnt, long long max_flop);

@@ -981,8 +981,15 @@ k_index_fill(CsrView B, int32_t shift, int32_t stride, int32_t max_slots, const 
 }
 
 __global__ void __launch_bounds__(kChunkThreads, 1024 / kChunkThreads)
-k_num_chunk(CsrView A, CsrView B, int32_t words, const int64_t* __restrict__ c_rowptr,
-            int32_t* __restrict__ c_colind, double* __restrict__ c_vals, WideKeep keep, int* status) {
+k_num_chunk(CsrView A, CsrView B, int32_t words, const unsigned long long* __restrict__ fp,
+            const int64_t* __restrict__ c_rowptr, int32_t* __restrict__ c_colind, double* __restrict__ c_vals,
+            WideKeep keep, int* status) {
+  // other index arrays than the symbolic call's: what was kept of them says
+  // neither where to read nor which columns have a product
+  if (fp[0] != fp[1]) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) set_status(status, KK_ERR_STRUCTURE_MISMATCH);
+    return;
+  }
   extern __shared__ __align__(16) unsigned char wsm[];
   ChunkSmem& sm = *reinterpret_cast<ChunkSmem*>(wsm);
   const uint32_t* bits = reinterpret_cast<const uint32_t*>(sm.bits);
@@ -991,7 +998,7 @@ k_num_chunk(CsrView A, CsrView B, int32_t words, const int64_t* __restrict__ c_r
   const int32_t* __restrict__ bcol = B.colind;
   const double* __restrict__ bval = B.vals;
   const int ntasks = min(keep.next[1], keep.max_tasks);
-  int mismatch = 0;
+  int mismatch = 0, bad = 0;
   bool ok = true;
   for (;;) {
     __syncthreads();  // the last task's shared memory is free
@@ -1049,11 +1056,15 @@ k_num_chunk(CsrView A, CsrView B, int32_t words, const int64_t* __restrict__ c_r
       double a = 0.0;
       if (p < pe) {
         const int j = A.colind[p];
-        const int bs = B.rowptr[j], be = B.rowptr[j + 1], x = keep.bidx[j];
-        const int32_t* tab = keep.btab + (size_t)(x < 0 ? 0 : x) * keep.tab_stride;
-        s = beg.x == 0 ? bs : x >= 0 ? tab[c0 >> keep.shift] : chunk_bound(bcol, bs, be, c0);
-        len = (last ? be : x >= 0 ? tab[c1 >> keep.shift] : chunk_bound(bcol, s, be, c1)) - s;
-        a = a_value(A, i, p);
+        if ((unsigned)j < (unsigned)B.m) {
+          const int bs = B.rowptr[j], be = B.rowptr[j + 1], x = keep.bidx[j];
+          const int32_t* tab = keep.btab + (size_t)(x < 0 ? 0 : x) * keep.tab_stride;
+          s = beg.x == 0 ? bs : x >= 0 ? tab[c0 >> keep.shift] : chunk_bound(bcol, bs, be, c0);
+          len = (last ? be : x >= 0 ? tab[c1 >> keep.shift] : chunk_bound(bcol, s, be, c1)) - s;
+          a = a_value(A, i, p);
+        } else {
+          bad = 1;
+        }
       }
       long long tot;
       const long long ex = block_exscan<long long>(len > 0 ? (1ll << 40) + len : 0ll, sm.tmp, &tot);
@@ -1103,6 +1114,7 @@ k_num_chunk(CsrView A, CsrView B, int32_t words, const int64_t* __restrict__ c_r
       __stcs(&c_vals[off + e], sm.vals[e]);
     }
   }
+  if (bad) set_status(status, KK_ERR_BAD_INDEX);
   if (mismatch) set_status(status, KK_ERR_STRUCTURE_MISMATCH);
   if (!ok) set_status(status, KK_ERR_TIMEOUT);
 }
@@ -1245,8 +1257,8 @@ cudaError_t launch_numeric_wide(const LaunchCtx& ctx, const CsrView& A, const Cs
   return num_wide<kWideBlock>(ctx, A, B, words, g, c_rowptr, rows, nrows, c_colind, c_vals);
 }
 
-cudaError_t launch_num_chunk(const LaunchCtx& ctx, const CsrView& A, const CsrView& B, const int64_t* c_rowptr,
-                             int32_t* c_colind, double* c_vals) {
+cudaError_t launch_num_chunk(const LaunchCtx& ctx, const CsrView& A, const CsrView& B, const unsigned long long* fp,
+                             const int64_t* c_rowptr, int32_t* c_colind, double* c_vals) {
   cudaError_t e = cudaFuncSetAttribute(k_num_chunk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ChunkSmem));
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(ctx.keep.next + 2, 0, sizeof(int32_t), ctx.stream);
@@ -1258,8 +1270,8 @@ cudaError_t launch_num_chunk(const LaunchCtx& ctx, const CsrView& A, const CsrVi
     (void)cudaGetLastError();
     per_sm = 1;
   }
-  k_num_chunk<<<ctx.num_sms * per_sm, kChunkThreads, sizeof(ChunkSmem), ctx.stream>>>(A, B, wide_words(B.n), c_rowptr, c_colind,
-                                                                         c_vals, ctx.keep, ctx.status);
+  k_num_chunk<<<ctx.num_sms * per_sm, kChunkThreads, sizeof(ChunkSmem), ctx.stream>>>(
+      A, B, wide_words(B.n), fp, c_rowptr, c_colind, c_vals, ctx.keep, ctx.status);
   timer_end(ctx.timer, ctx.stream);
   return cudaGetLastError();
 }
