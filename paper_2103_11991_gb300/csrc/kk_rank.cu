@@ -18,7 +18,8 @@
 // here).  90,666 rows of about 500 columns of an unsorted B take 592 us: 1,250 with
 // an entry of A at a time, 905 flattened, 800 without branches, then two warps per
 // row where a row's shared memory leaves few of them on an SM.  C's columns come from the products themselves (each writes its
-// column's offset beside its value), not from expanding the bits.
+// column's offset beside its value), not from expanding the bits; a slot that no
+// product wrote means that B is not the one whose compressed rows gave the bits.
 //
 // The row's products are walked flattened, 32 per step whatever the lengths of
 // the B rows (an entry at a time left lanes idle and, for B rows of more than
@@ -302,7 +303,12 @@ __global__ void __launch_bounds__(kRankThreads, 14) k_num_rank(RankArgs g, RankG
       __syncwarp();
     }
     const int nout = min(cnt, vmax);
-    for (int e = tid; e < nout; e += NT) vals[e] = 0ull;
+    // a slot's column comes from its products: offset 0 stands for none yet (the
+    // offsets ascend; that of a sorted B's slot 0 is 0, so 1 stands for it there)
+    for (int e = tid; e < nout; e += NT) {
+      vals[e] = 0ull;
+      cols[e] = SORTED && e == 0 ? 1 : 0;
+    }
     if (NW > 1) sync();
     int j_n = -1;
     if (i_n >= 0 && pa_n + lane < pe_n) j_n = acol[pa_n + lane];
@@ -458,11 +464,13 @@ __global__ void __launch_bounds__(kRankThreads, 14) k_num_rank(RankArgs g, RankG
       y_n = brp[j_n + 1] - x_n;
       z_n = SORTED ? g.bcomp.len[j_n] : y_n;
     }
-    if (bad) set_status(g.status, KK_ERR_STRUCTURE_MISMATCH);
     for (int e = tid; e < nout; e += NT) {
-      g.c_colind[off + e] = lo + (int)cols[e];
+      const int o = (int)cols[e];
+      bad |= SORTED && (e == 0) != (o == 0);  // a column of the bits without a product
+      g.c_colind[off + e] = lo + (SORTED && e == 0 ? 0 : o);
       g.c_vals[off + e] = out_value(vals[e], DFM && df);
     }
+    if (bad) set_status(g.status, KK_ERR_STRUCTURE_MISMATCH);
     for (int q = tid; q < n4; q += NT) bits4[q] = make_uint4(0u, 0u, 0u, 0u);
     sync();
     i = i_n;
