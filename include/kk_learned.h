@@ -56,7 +56,8 @@ kk_status kk_mlp_init(void* cuda_stream, float* params, uint64_t seed);
 
 /* Mean softmax cross-entropy of the n samples X (float32[n*8]) with labels y
  * (int32[n]) and its gradient with respect to params: grad (float32[1872]) and
- * loss (float32[1]) are overwritten. */
+ * loss (float32[1]) are overwritten.  A label outside 0..15 names no class: its
+ * sample's loss is the log of the sum of exponentials, its target is zero. */
 kk_status kk_mlp_loss_grad(void* cuda_stream, int32_t n, const float* X, const int32_t* y,
                            const float* params, float* grad, float* loss);
 

@@ -261,7 +261,8 @@ k_mlp_loss_grad(int32_t n, int32_t start, int32_t count, long long pa, long long
         const int c = 2 * w + u;
         sm.dz[c][lane] = (__expf(sm.z[c][lane] - lse) - (c == label ? 1.0f : 0.0f)) * inv;
       }
-      if (w == 0) lsum += (lse - sm.z[label][lane]) * inv;
+      // a label that is no class has no unit of z to read: its loss is lse
+      if (w == 0) lsum += (lse - ((unsigned)label < (unsigned)kMlpC ? sm.z[label][lane] : 0.0f)) * inv;
     }
     __syncthreads();
     {  // dh2, units 4 w .. 4 w + 3
