@@ -10,6 +10,7 @@
 #include "kk_internal.h"
 #include "kk_learned.h"
 #include "kk_mlp.cuh"
+#include "kk_walk.h"
 
 namespace kk {
 namespace {
@@ -184,7 +185,7 @@ k_mlp_loss_grad(int32_t n, int32_t start, int32_t count, long long pa, long long
   const int j2 = (w * 2 + (lane >> 4)) * 2, k2 = (lane & 15) * 2;  // W2 block of this thread
   const int k3 = tid >> 3, c3 = (tid & 7) * 2;                      // W3 pair
   const float inv_count = 1.0f / (float)count;
-  for (int t0 = blockIdx.x * 32; t0 < count; t0 += gridDim.x * 32) {
+  for (int t0 = blockIdx.x * 32; t0 < count; t0 = walk_next_tile(t0, gridDim.x * 32, count)) {
     const bool active = t0 + lane < count;
     const float inv = active ? inv_count : 0.0f;
     int label = 0;
@@ -357,7 +358,7 @@ k_mlp_loss_grad(int32_t n, int32_t start, int32_t count, long long pa, long long
 
 // CTAs of k_mlp_loss_grad: one per tile up to four per SM, in whole clusters.
 int grad_ctas(int count) {
-  const int tiles = (count + 31) / 32;
+  const int tiles = count / 32 + (count % 32 != 0);
   const int ctas = (tiles + kGradCluster - 1) / kGradCluster * kGradCluster;
   return ctas < kGradMaxCtas ? ctas : kGradMaxCtas;
 }

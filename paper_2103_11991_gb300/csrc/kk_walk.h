@@ -29,4 +29,8 @@ KK_WALK uint32_t walk_upto(int lane) { return 0xffffffffu >> (31 - lane); }
 // The product that a lane of the step from f on takes.
 KK_WALK int walk_product(int f, int lane, int f_hi) { return f + lane < f_hi ? f + lane : f_hi - 1; }
 
+// k_mlp_loss_grad: the next tile of samples of a CTA, count when there is none (the
+// sum may lie beyond int for counts near its largest).
+KK_WALK int walk_next_tile(int t0, int step, int count) { return count - t0 > step ? t0 + step : count; }
+
 }  // namespace kk

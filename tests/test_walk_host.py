@@ -44,6 +44,18 @@ extern "C" int replay(int np, const int* first, const int* len, int warps, int u
   for (int p = 0; p < total; ++p) if (taken[p] != 1) return -1;
   return 0;
 }
+
+// The tiles that CTA `cta` of `ctas` takes of `count` samples; -1 when one begins
+// outside them or before the one before.
+extern "C" int tiles(int cta, int ctas, int count) {
+  int n = 0, last = -1;
+  for (int t0 = cta * 32; t0 < count; t0 = walk_next_tile(t0, ctas * 32, count)) {
+    if (t0 <= last) return -1;
+    last = t0;
+    ++n;
+  }
+  return n;
+}
 """
 
 
@@ -76,3 +88,10 @@ def test_lanes_past_a_run_stay_in_its_pieces(replay, order, high):
             np.cumsum(lens[::-1])[::-1] - lens if order == "descending" else np.zeros(len(lens), int)
         for u in (1, 2, 4):
             assert _walk(replay, first, lens, u) == 0
+
+
+@pytest.mark.parametrize("count", [1, 32, 33, 19456, 19457, 2 ** 31 - 19457, 2 ** 31 - 19456, 2 ** 31 - 1])
+def test_tiles_of_samples_end(replay, count):
+    for ctas in (8, 608):
+        got = [replay.tiles(c, ctas, count) for c in (0, 1, ctas - 1)]
+        assert got == [max(0, -(-(-(-count // 32) - c) // ctas)) for c in (0, 1, ctas - 1)]
