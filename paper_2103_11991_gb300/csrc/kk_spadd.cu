@@ -128,6 +128,14 @@ struct AddRow {
   int pa, la, pb, lb;
 };
 
+// coefficient * value, rounded once.  A coefficient of 1 skips the float64 multiply
+// (FP64 is the scarce pipe; the branch is uniform over the grid).  Products and sums
+// are the rounded intrinsics: the compiler may contract plain ones into one fma, and
+// a row's values would then depend on which of the paths below it takes.
+__device__ __forceinline__ double add_scaled(double coefficient, double v) {
+  return coefficient == 1.0 ? v : __dmul_rn(coefficient, v);
+}
+
 // A row by a warp: its columns go to col (A's la, then B's lb); *strict: both
 // rows strictly ascending.
 __device__ __forceinline__ void add_stage(const CsrView& A, const CsrView& B, const AddRow& r, int32_t* col,
@@ -181,11 +189,8 @@ __device__ __forceinline__ int add_merge(const CsrView& A, const CsrView& B, dou
       k = add_lower_bound(cb, r.lb, c);
       found = k < r.lb && cb[k] == c;
     }
-    if (alpha != 1.0) v *= alpha;
-    if (found) {
-      const double w = B.vals[r.pb + k];
-      v += beta == 1.0 ? w : beta * w;
-    }
+    v = add_scaled(alpha, v);
+    if (found) v = __dadd_rn(v, add_scaled(beta, B.vals[r.pb + k]));
     const unsigned f = __ballot_sync(kFull, found);
     const int s = t + k - common - __popc(f & before);
     if (t < r.la && s < n) {
@@ -205,7 +210,7 @@ __device__ __forceinline__ int add_merge(const CsrView& A, const CsrView& B, dou
       k = add_lower_bound(ca, r.la, c);
       found = k < r.la && ca[k] == c;
     }
-    if (beta != 1.0) v *= beta;
+    v = add_scaled(beta, v);
     const unsigned f = __ballot_sync(kFull, found);
     const int s = t + k - seen - __popc(f & before);
     if (t < r.lb && !found && s < n) {
@@ -430,9 +435,7 @@ __device__ __forceinline__ void add_scatter(const CsrView& A, const CsrView& B, 
     const bool a = t < r.la, b = t < r.lb;
     const int sa = a ? apos[r.pa + t] : 0, sb = b ? bpos[r.pb + t] : 0;
     const int ca = a ? A.colind[r.pa + t] : 0, cb = b ? B.colind[r.pb + t] : 0;
-    double va = a ? A.vals[r.pa + t] : 0.0, vb = b ? B.vals[r.pb + t] : 0.0;
-    if (alpha != 1.0) va *= alpha;
-    if (beta != 1.0) vb *= beta;
+    const double va = a ? add_scaled(alpha, A.vals[r.pa + t]) : 0.0, vb = b ? add_scaled(beta, B.vals[r.pb + t]) : 0.0;
     if (a) put(sa, ca, va);
     if (b) put(sb, cb, vb);
   }
@@ -442,9 +445,8 @@ __device__ __forceinline__ void add_scatter(const CsrView& A, const CsrView& B, 
     const int at = s & 0x7fffffff;
     if (s < 0 && at < n) atomicAdd(&c_vals[off + at], v);
   };
-  for (int t = lane; t < r.la; t += 32)
-    add(apos[r.pa + t], alpha == 1.0 ? A.vals[r.pa + t] : alpha * A.vals[r.pa + t]);
-  for (int t = lane; t < r.lb; t += 32) add(bpos[r.pb + t], beta == 1.0 ? B.vals[r.pb + t] : beta * B.vals[r.pb + t]);
+  for (int t = lane; t < r.la; t += 32) add(apos[r.pa + t], add_scaled(alpha, A.vals[r.pa + t]));
+  for (int t = lane; t < r.lb; t += 32) add(bpos[r.pb + t], add_scaled(beta, B.vals[r.pb + t]));
 }
 
 // Numeric, T lanes per row as in k_spadd_count.
@@ -496,10 +498,8 @@ k_spadd_num(CsrView A, CsrView B, double alpha, double beta, const int64_t* __re
     if (__any_sync(kFull, cur.fits)) {
       const bool strict = add_strict<T>(ca, cb, r, A.n, tl, team, &bad);
       if (!strict) mismatch = 1;  // not the rows of the symbolic call
-      // coefficients of 1 skip the float64 multiply (FP64 is the scarce pipe): the
-      // branches are uniform over the grid
-      if (alpha != 1.0) va *= alpha;
-      if (beta != 1.0) vb *= beta;
+      va = add_scaled(alpha, va);
+      vb = add_scaled(beta, vb);
       bool fa, fb;
       const int ka = add_search<T>(cb, ca, &fa), kb = add_search<T>(ca, cb, &fb);
       fa = fa && tl < r.la;
@@ -507,7 +507,7 @@ k_spadd_num(CsrView A, CsrView B, double alpha, double beta, const int64_t* __re
       const unsigned ma = __ballot_sync(kFull, fa) & team, mb = __ballot_sync(kFull, fb) & team;
       if (__any_sync(kFull, fa)) {  // shared columns: A's entry takes the sum
         const double w = __shfl_sync(kFull, vb, min(ka, T - 1), T);
-        if (fa) va += w;
+        if (fa) va = __dadd_rn(va, w);
       }
       if (cur.fits) {
         if (row < A.m && r.la + r.lb - __popc(ma) != n) mismatch = 1;
