@@ -81,11 +81,15 @@ typedef struct {
   int32_t timing;         /* 1: record CUDA events around every kernel (see kk_spgemm_kernel_times)
                              and count the per-tier statistics (kk_spgemm_stats) */
   int32_t force_tier;     /* testing: -1 = automatic; 0 = team hash, 1 = CTA hash, 2 = dense chunks,
-                             3 = window wherever a row qualifies (team hash elsewhere) */
+                             3 = window wherever a row qualifies (dense chunks elsewhere) */
   int32_t team_vec_min_len; /* mean B-row length from which a team walks B rows lane-parallel (else flattened) */
-  int32_t sym_team_max_flop;  /* rows up to this flop bound use a team hash in the symbolic phase */
+  int32_t sym_team_max_flop;  /* rows up to this flop bound use a team hash in the symbolic phase
+                                 (default 3072; with the default, rows whose numeric phase the wide
+                                 tier's kept bits serve leave it earlier) */
   int32_t sym_cta_max_flop;   /* rows up to this flop bound use a CTA hash; above it dense chunks */
-  int32_t num_team_max_nnz;   /* rows up to this nnz(C(i,:)) use a team hash in the numeric phase */
+  int32_t num_team_max_nnz;   /* rows up to this nnz(C(i,:)) use a team hash in the numeric phase
+                                 (default 1024; with the default, not those whose bits the wide tier
+                                 kept) */
   int32_t num_cta_max_nnz;    /* rows up to this nnz use a CTA hash; above it dense chunks */
   int32_t use_window;         /* 1: rows whose column span fits a shared-memory window use the
                                  dense window accumulator (needs B rows sorted) */

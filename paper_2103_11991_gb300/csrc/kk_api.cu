@@ -1048,7 +1048,7 @@ void build_bins(const kk_spgemm_options& o, bool numeric, std::vector<BinSpec>& 
   }
 }
 
-BinTable to_table(const std::vector<BinSpec>& bins, bool numeric, int32_t cols) {
+BinTable to_table(const std::vector<BinSpec>& bins, bool numeric, int32_t cols, bool automatic) {
   BinTable t{};
   t.nb = 0;
   t.nwin = 0;
@@ -1060,9 +1060,9 @@ BinTable to_table(const std::vector<BinSpec>& bins, bool numeric, int32_t cols) 
       t.win_bits[t.nwin] = bins[b].slots;
       t.win_bin[t.nwin] = (int32_t)b;
       // a heavy row's products are too many for the window's one warp where the
-      // wide tier's bit vector is no larger than a window
-      t.win_q[t.nwin] =
-          !numeric && !rank && cols <= kWindowBits[kNumWindowClasses - 1] ? kWindowMaxFlop : bins[b].hi;
+      // wide tier's bit vector is no larger than a window (automatic tiers only)
+      t.win_q[t.nwin] = automatic && !numeric && !rank && cols <= kWindowBits[kNumWindowClasses - 1] ? kWindowMaxFlop
+                                                                                                     : bins[b].hi;
       t.win_kept[t.nwin] = numeric && !rank ? 1 : 0;
       t.win_order[t.nwin] = !rank ? 0 : numeric ? 1 : 2;
       t.win_ratio[t.nwin] = rank ? kRankFlopRatio : kWindowFlopRatio;
@@ -1227,8 +1227,9 @@ kk_status keep_for_symbolic(kk_spgemm_handle h, int32_t m, int64_t wide_rows, co
   if (!wide_symbolic_fits(probe, bv.n) || !wide_numeric_fits(probe, bv.n)) return KK_OK;
   const size_t words = (size_t)wide_word_count(bv.n);
   // sorted B: rows of more columns than the rank tier takes, computed in chunks;
-  // otherwise: rows whose values do not fit the wide kernel's shared memory
-  const bool tasks = h->b_sorted != 0 && bv.n <= kChunkMaxCols;
+  // otherwise: rows whose values do not fit the wide kernel's shared memory.  A
+  // forced team tier keeps the rows that fit its tables.
+  const bool tasks = h->b_sorted != 0 && bv.n <= kChunkMaxCols && h->opt.force_tier != 0;
   const int32_t chunks = tasks ? wide_max_chunks(bv.n) : 0;
   const size_t stride = words + ((size_t)chunks * 2 + 3) / 4 * 4;
   const size_t budget = h->opt.wide_cache_mb > 0 ? ((size_t)h->opt.wide_cache_mb << 20) : h->dev_total / 8;
@@ -1253,6 +1254,9 @@ kk_status keep_for_symbolic(kk_spgemm_handle h, int32_t m, int64_t wide_rows, co
   h->keep.min_cnt = !tasks                                ? wide_keep_min_cnt(probe, bv.n)
                     : bv.n <= kRankBits[kNumRankBits - 1] ? kRankNnz[kNumRankNnz - 1]
                                                           : kRankNnz[0];
+  // (num_team_max_nnz as asked for: those rows stay in the team tier)
+  if (tasks && h->opt.num_team_max_nnz != kNumTeamMaxNnz && h->keep.min_cnt < h->opt.num_team_max_nnz)
+    h->keep.min_cnt = h->opt.num_team_max_nnz;
   h->keep.stride = (int32_t)stride;
   h->keep.max_chunks = chunks;
   h->keep.max_tasks = (int32_t)ntasks;
@@ -1426,12 +1430,15 @@ static cudaError_t launch_jacobi_rows(kk_spgemm_handle h, const CsrView& av, con
   return cudaGetLastError();
 }
 
-// The symbolic bins' table: rows that the wide tier's kept chunks serve better
-// than the hash kernels leave the team tier.
+// The symbolic bins' table: with the tiers chosen automatically, rows that the
+// wide tier's kept chunks serve better than the hash kernels leave the team tier.
+// A forced tier, or another sym_team_max_flop than the default, says which rows
+// the team tier takes, and that is then so.
 static BinTable symbolic_table(kk_spgemm_handle h, int32_t cols) {
-  BinTable t = to_table(h->sym_bins, false, cols);
-  if (cols <= kChunkMaxCols && h->opt.structure_cache && h->opt.wide_cache_mb >= 0 &&
-      wide_symbolic_fits(ctx_of(h), cols) && wide_numeric_fits(ctx_of(h), cols)) {
+  const bool automatic = h->opt.force_tier == -1;
+  BinTable t = to_table(h->sym_bins, false, cols, automatic);
+  if (automatic && h->opt.sym_team_max_flop == kSymTeamMaxFlop && cols <= kChunkMaxCols && h->opt.structure_cache &&
+      h->opt.wide_cache_mb >= 0 && wide_symbolic_fits(ctx_of(h), cols) && wide_numeric_fits(ctx_of(h), cols)) {
     const long long least = wide_keep_min_flop(wide_word_count(cols)) - 1;
     t.team_max = least > kKeepEarlyFlop ? least : kKeepEarlyFlop;
   }
@@ -1495,9 +1502,9 @@ kk_status kk_spgemm_options_default(kk_spgemm_options* opt) {
   opt->timing = 0;
   opt->force_tier = -1;
   opt->team_vec_min_len = 12;
-  opt->sym_team_max_flop = 3072;
+  opt->sym_team_max_flop = kSymTeamMaxFlop;
   opt->sym_cta_max_flop = 24576;
-  opt->num_team_max_nnz = 1024;
+  opt->num_team_max_nnz = kNumTeamMaxNnz;
   opt->num_cta_max_nnz = 4096;
   opt->use_window = 1;
   opt->batched_graph = 1;
@@ -1719,7 +1726,7 @@ kk_status kk_spgemm_symbolic(kk_spgemm_handle h, const kk_csr* A, const kk_csr* 
     k_scan_final<<<nblk_scan, kScanBlock, 0, s>>>(
         m, h->d_cnt.as<int32_t>(), h->d_scan.as<long long>(), h->d_flop.as<long long>(), av.rowptr,
         h->d_span.as<int32_t>(), &dm->sorted, h->opt.team_vec_min_len,
-        to_table(h->num_bins, true, bv.n), kept_counts(h), kept_slots(h), c_rowptr,
+        to_table(h->num_bins, true, bv.n, h->opt.force_tier == -1), kept_counts(h), kept_slots(h), c_rowptr,
         h->d_nbin.as<uint8_t>());
     timer_end(h->timer, s);
     KK_CUDA(h, cudaGetLastError(), "scan launch");
@@ -1916,7 +1923,8 @@ kk_status run_scan(kk_spgemm_handle h, int32_t m, const int32_t* cnt, int64_t* o
   k_scan_top<<<1, 1024, 0, s>>>(nblk, h->d_scan.as<long long>(), grand);
   k_scan_final<<<nblk, kScanBlock, 0, s>>>(m, cnt, h->d_scan.as<long long>(), h->d_flop.as<long long>(),
                                            av.rowptr, h->d_span.as<int32_t>(), &dm->sorted,
-                                           h->opt.team_vec_min_len, to_table(h->num_bins, true, cols),
+                                           h->opt.team_vec_min_len,
+                                           to_table(h->num_bins, true, cols, h->opt.force_tier == -1),
                                            nbin ? kept_counts(h) : nullptr, nbin ? kept_slots(h) : nullptr,
                                            out, nbin);
   KK_CUDA(h, cudaGetLastError(), "scan launch");

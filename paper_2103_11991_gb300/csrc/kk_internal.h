@@ -229,6 +229,9 @@ enum ArithMode : int32_t { kArithF64 = 1, kArithDF32 = 2 };
 // 273.0 (chunks also end every 65,536 columns, so a wide B has more of them per row,
 // and each walks all of the row's entries of A).
 constexpr int32_t kChunkMaxCols = 1 << 19;
+// Defaults of options.sym_team_max_flop and options.num_team_max_nnz: with these the
+// lines to the chunks are the library's, any other value holds as it was given.
+constexpr int32_t kSymTeamMaxFlop = 3072, kNumTeamMaxNnz = 1024;
 // Sorted B: symbolic rows of more than kKeepEarlyFlop products that the wide tier
 // would keep (wide_keep_min_flop) leave the team tier for it, because its chunks
 // serve their numeric phase.
