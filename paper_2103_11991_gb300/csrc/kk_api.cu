@@ -135,7 +135,8 @@ constexpr uint8_t kSkipBin = 0xFF;
 // qualifies for one when its span fits win_bits, the window is not too wide for
 // its flop count and q lies in the bin's range.  Kept bins (numeric) also need
 // the structure kept by the symbolic phase; the others take unsorted B too
-// (any_order), over all of its columns.
+// (any_order), over all of its columns.  wq is the quantity of the window bins: q,
+// or less for a row whose work there is not its products.
 struct BinTable {
   int32_t nb;
   long long hi[kMaxBins];
@@ -143,6 +144,7 @@ struct BinTable {
   long long thread_flop;
   long long team_max;  // sorted B: rows beyond it leave the team tier
   int32_t cols;        // columns of B
+  long long pair_flop; // symbolic rows of more products: the window bins go by wq (see k_analyze_a)
   int32_t nwin;
   int32_t win_bits[kMaxWindowBins];
   int32_t win_bin[kMaxWindowBins];
@@ -153,14 +155,14 @@ struct BinTable {
 };
 
 __device__ __forceinline__ uint8_t classify(const BinTable& t, long long q, int flat, int span,
-                                            long long flop, int sorted, bool kept) {
+                                            long long flop, int sorted, bool kept, long long wq) {
   if (q <= 0) return kSkipBin;
   for (int b = 0; t.mode[b] == 3; ++b)
     if (q <= t.hi[b] && flop <= t.thread_flop) return (uint8_t)b;
   const int sp = sorted ? span : t.cols;
   if (sp > 0) {
     for (int w = 0; w < t.nwin; ++w)
-      if (q <= t.win_q[w] && sp <= t.win_bits[w] && t.win_order[w] != (sorted ? 2 : 0) && (!t.win_kept[w] || kept) &&
+      if (wq <= t.win_q[w] && sp <= t.win_bits[w] && t.win_order[w] != (sorted ? 2 : 0) && (!t.win_kept[w] || kept) &&
           (long long)t.win_bits[w] <= (q > kRankMinNnz ? t.win_ratio[w] : (long long)kWindowFlopRatio) * flop)
         return (uint8_t)t.win_bin[w];
   }
@@ -181,10 +183,14 @@ __device__ __forceinline__ uint8_t classify(const BinTable& t, long long q, int 
 // is processed; T and U follow A's mean row length.  STATS (the learned
 // form): also the longest and shortest referenced B row of each row, to stat.
 // Long rows are listed for a second launch (LISTED), as in k_analyze_b.
+// Rows of more than tab.pair_flop products of a sorted B are binned for the window
+// by the compressed pairs of their B rows (blen, null: not known) where these hold
+// kWindowDense columns or more each; a second walk over the row's entries of A adds
+// the pairs up.  The others are binned by their products.
 template <int T, int U, bool STATS, bool LISTED>
 __global__ void __launch_bounds__(256, 6)
 k_analyze_a(CsrView A, const int32_t* __restrict__ brp,
-                            const int32_t* __restrict__ bcol, int32_t nb_rows,
+                            const int32_t* __restrict__ bcol, const int32_t* __restrict__ blen, int32_t nb_rows,
                             const int32_t* __restrict__ b_sorted, BinTable tab,
                             int32_t vec_min_len, long long* __restrict__ flop,
                             uint8_t* __restrict__ bin, int32_t* __restrict__ row_lo,
@@ -277,14 +283,32 @@ k_analyze_a(CsrView A, const int32_t* __restrict__ brp,
       }
     }
     if (bad) set_status(status, KK_ERR_BAD_INDEX);
+    const long long span = hi >= lo ? (long long)hi - lo + 1 : 0;
+    long long wq = f;
+    if (on && sorted && f > tab.pair_flop) {  // (the same for all lanes of a team)
+      if (span <= kWindowFreeSpan) {
+        wq = 1;
+      } else if (blen) {
+        long long pairs = 0;
+        for (int p0 = pa; p0 < pe; p0 += T * U) {
+          int j[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) j[u] = p0 + u * T + tl < pe ? A.colind[p0 + u * T + tl] : -1;
+#pragma unroll
+          for (int u = 0; u < U; ++u) pairs += (unsigned)j[u] < (unsigned)nb_rows ? blen[j[u]] : 0;
+        }
+#pragma unroll
+        for (int o = T / 2; o > 0; o >>= 1) pairs += __shfl_xor_sync(mask, pairs, o, T);
+        if (pairs * kWindowDense <= f) wq = pairs;
+      }
+    }
     if (on && tl == 0) {
       flop[r] = f;
-      const long long span = hi >= lo ? (long long)hi - lo + 1 : 0;
       const int sp = span > 0x7fffffff ? 0x7fffffff : (int)span;
       row_lo[r] = hi >= lo ? lo : 0;
       row_span[r] = sp;
       const int flat = (f < (long long)vec_min_len * (pe - pa)) ? 1 : 0;
-      bin[r] = classify(tab, f, flat, sp, f, sorted, false);
+      bin[r] = classify(tab, f, flat, sp, f, sorted, false, wq);
       if (STATS) stat[r] = make_int2(mx, pe > pa ? mn : 0);
       acc += (unsigned long long)f;
     }
@@ -527,7 +551,8 @@ k_scan_final(int32_t m, const int32_t* __restrict__ cnt, const long long* __rest
         const int flat = (flop[r] < (long long)vec_min_len * nza) ? 1 : 0;
         nbin[r] = wide_slot != nullptr && wide_slot[r] >= 0
                       ? (uint8_t)(ntab.nb - 1)  // kept bits: chunk tasks
-                      : classify(ntab, v[t], flat, row_span[r], flop[r], sorted, kept_n != nullptr && kept_n[r] >= 0);
+                      : classify(ntab, v[t], flat, row_span[r], flop[r], sorted, kept_n != nullptr && kept_n[r] >= 0,
+                                 v[t]);
       }
       if (r == m - 1) rowptr[m] = run + v[t];
     }
@@ -1054,15 +1079,17 @@ BinTable to_table(const std::vector<BinSpec>& bins, bool numeric, int32_t cols, 
   t.nwin = 0;
   t.team_max = (long long)9e18;
   t.cols = cols;
+  t.pair_flop = (long long)9e18;
   for (size_t b = 0; b < bins.size(); ++b) {
     const bool rank = bins[b].tier == kTierRank;
     if (rank || bins[b].tier == kTierWindow) {
       t.win_bits[t.nwin] = bins[b].slots;
       t.win_bin[t.nwin] = (int32_t)b;
-      // a heavy row's products are too many for the window's one warp where the
-      // wide tier's bit vector is no larger than a window (automatic tiers only)
-      t.win_q[t.nwin] = automatic && !numeric && !rank && cols <= kWindowBits[kNumWindowClasses - 1] ? kWindowMaxFlop
-                                                                                                     : bins[b].hi;
+      // a heavy row is too much for the window's one warp where the wide tier's bit
+      // vector is no larger than a window (automatic tiers only)
+      const bool narrow = automatic && !numeric && !rank && cols <= kWindowBits[kNumWindowClasses - 1];
+      t.win_q[t.nwin] = narrow ? kWindowMaxFlop : bins[b].hi;
+      if (narrow) t.pair_flop = kWindowMaxFlop;
       t.win_kept[t.nwin] = numeric && !rank ? 1 : 0;
       t.win_order[t.nwin] = !rank ? 0 : numeric ? 1 : 2;
       t.win_ratio[t.nwin] = rank ? kRankFlopRatio : kWindowFlopRatio;
@@ -1460,7 +1487,7 @@ static void launch_analyze_a_t(kk_spgemm_handle h, const CsrView& av, const CsrV
   }
   const int64_t m = LISTED ? lr.most : av.m;
   kern<<<grid_for(m * T, 256, h->num_sms * (per_sm > 0 ? per_sm : 1)), 256, 0, s>>>(
-      av, bv.rowptr, bv.colind, bv.m, &dm->sorted, symbolic_table(h, bv.n), h->opt.team_vec_min_len,
+      av, bv.rowptr, bv.colind, h->opt.use_window ? h->d_bclen.as<int32_t>() : nullptr, bv.m, &dm->sorted, symbolic_table(h, bv.n), h->opt.team_vec_min_len,
       h->d_flop.as<long long>(), bin, h->d_rowlo.as<int32_t>(), h->d_span.as<int32_t>(), stat,
       &dm->total_flop, &dm->status, lr);
 }

@@ -135,7 +135,20 @@ __host__ __device__ constexpr int32_t window_bits(int w) {
 }
 constexpr int32_t kWindowMaxNnz = 256;   // numeric window rows: nnz(C(i,:)) <= this
 constexpr int32_t kWindowFlopRatio = 128;  // window used only when W <= ratio * flop
-constexpr long long kWindowMaxFlop = 4096;  // symbolic rows of a narrow B (k <= 65,536): flop bound <= this
+// Symbolic rows of a narrow B (k <= 65,536) with more than kWindowMaxFlop products
+// leave the window tier, because the wide tier's chunks serve their numeric phase
+// (60,000 random rows of 4,900 products: 2.9 ms, 7.9 without) - but for rows with
+// few columns, whose numeric phase is the kept rows' or the rank tier's either way:
+// those of a span up to kWindowFreeSpan, and those whose B rows hold kWindowDense
+// columns or more to a word, while the pairs that the window's warp walks are no
+// more than kWindowMaxFlop.  (Rows of small dense blocks, 81 x 81: 6,561 products,
+// 283 pairs.  59,940 of them, both phases: 1.50 ms in the window, 4.43 in the wide
+// tier without kept structure.)  Power-law rows have 2 to 5 columns to a word: all
+// of them by their pairs took the scale-15 R-MAT square from 1.98 to 2.62 ms, those
+// of 4 or more to 2.09.
+constexpr long long kWindowMaxFlop = 4096;
+constexpr int32_t kWindowFreeSpan = 1024;
+constexpr int kWindowDense = 6;
 
 // Rank tier (kk_rank.cu): numeric rows without kept structure, nnz(C(i,:)) at
 // most kRankNnz[2], span at most kRankBits of the bin; symbolic rows of an
@@ -152,6 +165,7 @@ constexpr int32_t kRankMinNnz = 32;
 // Symbolic rank rows: flop bound <= this, the line of the window tier for a B as
 // narrow; heavier rows are too many products for one warp and stay where they were.
 constexpr long long kRankMaxFlop = 4096;
+static_assert(kWindowFreeSpan <= kRankNnz[kNumRankNnz - 1], "their numeric phase is the rank tier's or the kept rows'");
 constexpr int kMaxWindowBins = kNumWindowClasses + kNumRankBits * kNumRankNnz;
 
 // Per-row structure kept by the symbolic window kernel for the numeric phase
