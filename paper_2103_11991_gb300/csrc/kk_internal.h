@@ -254,8 +254,14 @@ constexpr long long kKeepEarlyFlop = 512;
 // most words empty, and it walks a summary instead.  Measured with the line above,
 // R-MAT squares of scale 18 and 19: words / 4 and 768 30.4 and 92.6 ms, words / 11
 // and 768 28.7 and 91.7, words / 16 and 512 28.5 and 91.0, words / 24 and 384 28.4
-// and 90.8 (hardly less, for more rows to hold).
-__host__ __device__ inline int wide_keep_min_flop(int words) { return words / 16; }
+// and 90.8 (hardly less, for more rows to hold).  A row has a chunk for every 2,048
+// words at least, and each walks all of its entries of A: beyond five of them (k >
+// 327,680) spread rows of words / 16 products are the hash kernels' (both phases of
+// random rows, hash and chunks: k = 520,000, 1,089 products 55.4 and 71.1 ms, 1,600
+// products 72.5 and 74.6, 2,116 products 84.3 and 77.8; k = 400,000, 1,296 products
+// 45.3 and 48.7, 1,764 products 57.1 and 51.2; k = 300,000, 900 products 39.5 and
+// 25.4), so the line is words / 8 there.
+__host__ __device__ inline int wide_keep_min_flop(int words) { return words <= 10240 ? words / 16 : words / 8; }
 
 // Symbolic launch: rows[0..nrows) of A (a device array) get cnt[i] = nnz(C(i,:)).
 cudaError_t launch_symbolic_bin(const LaunchCtx& ctx, const BinSpec& bin, const CsrView& A,

@@ -48,3 +48,13 @@ def test_forced_window_takes_every_row_of_a_narrow_b(flop):
     rp, ci, va, _, st = run_gpu(A, B, arith=1, force_tier=3)
     assert st["sym_window_rows"] == M
     check_against_oracle(A, B, rp, ci, va)
+
+
+# beyond five pieces of 2,048 words a row's chunks pay from more products on
+@pytest.mark.parametrize("k,flop,wide", [(327680, 690, True), (327681, 690, False), (400000, 1300, False),
+                                         (400000, 1800, True), (520000, 2010, False), (520000, 2100, True)])
+def test_line_by_columns_of_b(k, flop, wide):
+    A, B = _rows(k, flop)
+    rp, ci, va, _, st = run_gpu(A, B, arith=1, small_max_rows=0)
+    assert st["sym_cta_rows"] + st["sym_dense_rows"] == (M if wide else 0)
+    check_against_oracle(A, B, rp, ci, va)
