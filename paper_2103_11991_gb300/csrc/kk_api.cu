@@ -136,13 +136,14 @@ constexpr uint8_t kSkipBin = 0xFF;
 // its flop count and q lies in the bin's range.  Kept bins (numeric) also need
 // the structure kept by the symbolic phase; the others take unsorted B too
 // (any_order), over all of its columns.  wq is the quantity of the window bins: q,
-// or less for a row whose work there is not its products.
+// or less for a row whose work there is not its products; rows of a sorted B beyond
+// team_max leave the team tier.
 struct BinTable {
   int32_t nb;
   long long hi[kMaxBins];
   int32_t mode[kMaxBins];  // 0 vector, 1 flattened, 2 either, 3 thread tier (flop capped too)
   long long thread_flop;
-  long long team_max;  // sorted B: rows beyond it leave the team tier
+  long long team_max;  // sorted B: spread rows of more products leave the team tier
   int32_t cols;        // columns of B
   long long pair_flop; // symbolic rows of more products: the window bins go by wq (see k_analyze_a)
   int32_t nwin;
@@ -155,7 +156,8 @@ struct BinTable {
 };
 
 __device__ __forceinline__ uint8_t classify(const BinTable& t, long long q, int flat, int span,
-                                            long long flop, int sorted, bool kept, long long wq) {
+                                            long long flop, int sorted, bool kept, long long wq,
+                                            long long team_max) {
   if (q <= 0) return kSkipBin;
   for (int b = 0; t.mode[b] == 3; ++b)
     if (q <= t.hi[b] && flop <= t.thread_flop) return (uint8_t)b;
@@ -167,7 +169,7 @@ __device__ __forceinline__ uint8_t classify(const BinTable& t, long long q, int 
         return (uint8_t)t.win_bin[w];
   }
   for (int b = 0; b < t.nb; ++b) {
-    if (t.mode[b] == 3 || (t.mode[b] < 2 && sorted && q > t.team_max)) continue;
+    if (t.mode[b] == 3 || (t.mode[b] < 2 && sorted && q > team_max)) continue;
     if (q <= t.hi[b] && (t.mode[b] == 2 || t.mode[b] == flat)) return (uint8_t)b;
   }
   return (uint8_t)(t.nb - 1);
@@ -186,7 +188,9 @@ __device__ __forceinline__ uint8_t classify(const BinTable& t, long long q, int 
 // Rows of more than tab.pair_flop products of a sorted B are binned for the window
 // by the compressed pairs of their B rows (blen, null: not known) where these hold
 // kWindowDense columns or more each; a second walk over the row's entries of A adds
-// the pairs up.  The others are binned by their products.
+// the pairs up.  The others are binned by their products.  The same walk tells which
+// rows of too wide a span for a window and more than tab.team_max products are
+// spread.
 template <int T, int U, bool STATS, bool LISTED>
 __global__ void __launch_bounds__(256, 6)
 k_analyze_a(CsrView A, const int32_t* __restrict__ brp,
@@ -284,9 +288,11 @@ k_analyze_a(CsrView A, const int32_t* __restrict__ brp,
     }
     if (bad) set_status(status, KK_ERR_BAD_INDEX);
     const long long span = hi >= lo ? (long long)hi - lo + 1 : 0;
-    long long wq = f;
-    if (on && sorted && f > tab.pair_flop) {  // (the same for all lanes of a team)
-      if (span <= kWindowFreeSpan) {
+    long long wq = f, team_max = (long long)9e18;
+    const bool heavy = f > tab.pair_flop;
+    const bool early = f > tab.team_max && f <= kSymTeamMaxFlop && span > window_bits(kNumWindowClasses - 1);
+    if (on && sorted && (heavy || early)) {  // (the same for all lanes of a team)
+      if (heavy && span <= kWindowFreeSpan) {
         wq = 1;
       } else if (blen) {
         long long pairs = 0;
@@ -299,7 +305,8 @@ k_analyze_a(CsrView A, const int32_t* __restrict__ brp,
         }
 #pragma unroll
         for (int o = T / 2; o > 0; o >>= 1) pairs += __shfl_xor_sync(mask, pairs, o, T);
-        if (pairs * kWindowDense <= f) wq = pairs;
+        if (heavy && pairs * kWindowDense <= f) wq = pairs;
+        if (early && wide_spread_row(f, pairs)) team_max = tab.team_max;
       }
     }
     if (on && tl == 0) {
@@ -308,7 +315,7 @@ k_analyze_a(CsrView A, const int32_t* __restrict__ brp,
       row_lo[r] = hi >= lo ? lo : 0;
       row_span[r] = sp;
       const int flat = (f < (long long)vec_min_len * (pe - pa)) ? 1 : 0;
-      bin[r] = classify(tab, f, flat, sp, f, sorted, false, wq);
+      bin[r] = classify(tab, f, flat, sp, f, sorted, false, wq, team_max);
       if (STATS) stat[r] = make_int2(mx, pe > pa ? mn : 0);
       acc += (unsigned long long)f;
     }
@@ -552,7 +559,7 @@ k_scan_final(int32_t m, const int32_t* __restrict__ cnt, const long long* __rest
         nbin[r] = wide_slot != nullptr && wide_slot[r] >= 0
                       ? (uint8_t)(ntab.nb - 1)  // kept bits: chunk tasks
                       : classify(ntab, v[t], flat, row_span[r], flop[r], sorted, kept_n != nullptr && kept_n[r] >= 0,
-                                 v[t]);
+                                 v[t], ntab.team_max);
       }
       if (r == m - 1) rowptr[m] = run + v[t];
     }
@@ -1464,8 +1471,10 @@ static cudaError_t launch_jacobi_rows(kk_spgemm_handle h, const CsrView& av, con
 static BinTable symbolic_table(kk_spgemm_handle h, int32_t cols) {
   const bool automatic = h->opt.force_tier == -1;
   BinTable t = to_table(h->sym_bins, false, cols, automatic);
-  if (automatic && h->opt.sym_team_max_flop == kSymTeamMaxFlop && cols <= kChunkMaxCols && h->opt.structure_cache &&
-      h->opt.wide_cache_mb >= 0 && wide_symbolic_fits(ctx_of(h), cols) && wide_numeric_fits(ctx_of(h), cols)) {
+  // (which rows are spread is known from the compressed B, that is with use_window)
+  const bool lines = automatic && h->opt.use_window && h->opt.sym_team_max_flop == kSymTeamMaxFlop;
+  if (lines && cols <= kChunkMaxCols && h->opt.structure_cache && h->opt.wide_cache_mb >= 0 &&
+      wide_symbolic_fits(ctx_of(h), cols) && wide_numeric_fits(ctx_of(h), cols)) {
     const long long least = wide_keep_min_flop(wide_word_count(cols)) - 1;
     t.team_max = least > kKeepEarlyFlop ? least : kKeepEarlyFlop;
   }

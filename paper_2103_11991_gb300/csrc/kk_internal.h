@@ -262,6 +262,18 @@ constexpr long long kKeepEarlyFlop = 512;
 // 45.3 and 48.7, 1,764 products 57.1 and 51.2; k = 300,000, 900 products 39.5 and
 // 25.4), so the line is words / 8 there.
 __host__ __device__ inline int wide_keep_min_flop(int words) { return words <= 10240 ? words / 16 : words / 8; }
+// Rows whose products outnumber the pairs of their B rows (by 9 to 4, of few pairs
+// by 7 to 4) stay in the team tier up to kSymTeamMaxFlop products: runs of
+// neighbouring columns mostly meet in few columns of C, too few for chunks (27-point
+// rows of a 200 x 200 x 3 grid, 567 products in 75 columns, 2.45 to 2.8 products to
+// a pair: symbolic phase 0.43 ms by hash, 0.52 in the wide tier; 250 x 250 x 4 0.60
+// and 1.13; 1.8 products to a pair in at most 405 pairs where a grid's lines put the
+// runs across words). Power-law rows of 513 to 3,072 products have 1.2 to 2.1 to a
+// pair, those of at most 384 pairs under 1.7.
+constexpr int kKeepFewPairs = 416;
+__host__ __device__ inline bool wide_spread_row(long long flop, long long pairs) {
+  return flop * 4 < pairs * (pairs <= kKeepFewPairs ? 7 : 9);
+}
 
 // Symbolic launch: rows[0..nrows) of A (a device array) get cnt[i] = nnz(C(i,:)).
 cudaError_t launch_symbolic_bin(const LaunchCtx& ctx, const BinSpec& bin, const CsrView& A,

@@ -58,3 +58,24 @@ def test_line_by_pairs(k, pairs):
             window = k > 65536 or (pairs <= 4096 and (dense == 1 or dense >= 6))
             assert st["sym_window_rows"] == (30 if window else 0), (dense, empty, st)
             check_against_oracle(A, B, rp, ci, va)
+
+
+# 27-point rows of a flat grid (567 products in 75 columns, a span beyond the widest
+# window) and with 2 x 2 blocks (2,268 products in 150 columns)
+@pytest.mark.parametrize("use_window", [1, 0])
+@pytest.mark.parametrize("blocks", [1, 2])
+def test_rows_of_few_columns_stay_in_the_team_tier(blocks, use_window):
+    d = blocks
+    S = I.stencil_3d(200, 190, 3, 27, 26.0, -1.0) if d == 1 else I.stencil_3d(150, 110, 3, 27, 26.0, -1.0)
+    rows = np.repeat(np.arange(S.m, dtype=np.int64), np.diff(S.rowptr))
+    pick = np.arange(S.m)[:: 37] if d == 2 else np.arange(S.m)
+    r = (rows[:, None, None] * d + np.arange(d)[None, :, None]).repeat(d, 2).reshape(-1)
+    c = (S.colind[:, None, None].astype(np.int64) * d + np.arange(d)[None, None, :]).repeat(d, 1).reshape(-1)
+    order = np.lexsort((c, r))
+    A = I._from_sorted_coo(S.m * d, S.n * d, r[order], c[order], I.uniform01(d, "db.f", r.size) - 0.5)
+    A2 = A if d == 1 else I.ensure_csr(len(pick), A.n, np.concatenate([[0], np.cumsum(np.diff(A.rowptr)[pick])]),
+                                       np.concatenate([A.colind[A.rowptr[i]:A.rowptr[i + 1]] for i in pick]),
+                                       np.concatenate([A.vals[A.rowptr[i]:A.rowptr[i + 1]] for i in pick]))
+    rp, ci, va, _, st = run_gpu(A2, A, arith=1, use_window=use_window, small_max_rows=0)
+    assert st["sym_team_rows"] == A2.m
+    check_against_oracle(A2, A, rp, ci, va)
