@@ -680,8 +680,12 @@ __device__ __forceinline__ void wide_write_columns(const uint32_t* bits, const u
 }
 
 // Rows without chunk tasks.  BLOCK threads per row; vcap value slots.
+// (The least number of CTAs per SM in its launch bounds is not idle: without it the
+// same 64 registers are scheduled otherwise, 500,000 random rows of 1,225 products in
+// 500,000 columns 49.9 ms, 43.8 with it.  k_sym_wide is the other way round: R-MAT
+// scale 18 4.0 ms without, 5.3 with.)
 template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK)
+__global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)
 k_num_wide(CsrView A, CsrView B, int32_t words, int32_t vcap, uint32_t sum_off, uint32_t reg_off,
            uint32_t val_off, const int64_t* __restrict__ c_rowptr, const long long* __restrict__ flop,
            const int32_t* __restrict__ rows, int32_t nrows, int32_t* __restrict__ c_colind,
