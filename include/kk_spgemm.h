@@ -103,10 +103,13 @@ typedef struct {
                                  (its non-empty 32-column words, at most 64 per row, 6 bytes
                                  each) so that the numeric phase of the same A and B arrays
                                  writes C's columns without re-deriving them (default 1) */
-  int32_t wide_cache_mb;      /* budget for the wide tier's kept bit vectors (rows whose values
-                                 go to C by atomics keep their k-bit column vector from the
-                                 symbolic phase): MiB, 0 = one eighth of the device memory,
-                                 -1 = none; only with structure_cache = 1 */
+  int32_t wide_cache_mb;      /* budget for what the wide tier keeps of its rows from the symbolic
+                                 phase: their k-bit column vectors and, for a sorted B of at most
+                                 2^19 columns, tables of column chunks, the chunks' tasks and an
+                                 index of B's long rows.  MiB, 0 = one eighth of the device memory
+                                 (and at most half of what is free when it has to be allocated),
+                                 -1 = none; only with structure_cache = 1.  Rows beyond the budget,
+                                 or all where memory is short, are computed without */
   int32_t batched_mode;       /* batched form (kk_batched.h): 1 = persistent work-queue kernels
                                  (graph-capturable), 2 = the batch as one block-diagonal product
                                  through the plain two-phase kernels, 0 = automatic (2) */

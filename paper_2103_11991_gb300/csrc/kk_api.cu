@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "kk_internal.h"
+#include "kk_keep.h"
 #include "kk_device.cuh"
 #include "kk_batched.h"
 #include "kk_learned.h"
@@ -102,11 +103,14 @@ struct DevBuf {
   size_t bytes = 0;
   cudaError_t ensure(size_t need) {
     if (need <= bytes) return cudaSuccess;
+    const size_t b = need < 256 ? 256 : need;
+    return fit(b + b / 4);  // slack for growth
+  }
+  cudaError_t fit(size_t b) {  // no slack (buffers held to a budget)
+    if (b <= bytes) return cudaSuccess;
     if (p) cudaFree(p);
     p = nullptr;
     bytes = 0;
-    size_t b = need < 256 ? 256 : need;
-    b += b / 4;  // slack for growth
     cudaError_t e = cudaMalloc(&p, b);
     if (e != cudaSuccess) {
       p = nullptr;
@@ -1250,8 +1254,30 @@ kk_status cache_for_symbolic(kk_spgemm_handle h, int32_t m, bool any_window, con
   return KK_OK;
 }
 
+// The buffers of a keep plan (with the usual slack where the budget has room for it),
+// and whether all of them could be had.
+bool keep_alloc(kk_spgemm_handle h, const KeepSizes& s, const KeepPlan& p, long long budget) {
+  const long long bytes = keep_bytes(s, p);
+  const bool slack = bytes + bytes / 4 <= budget, chunks = s.slot_tasks > 0;
+  auto get = [&](DevBuf& b, long long need) {
+    return (slack ? b.ensure((size_t)need) : b.fit((size_t)need)) == cudaSuccess;
+  };
+  bool ok = get(h->d_wbits, p.slots * s.slot_bytes) && get(h->d_wslot, s.rows * kMapBytes) &&
+            h->d_wnext.ensure(sizeof(int32_t) * 4) == cudaSuccess;
+  if (ok && chunks)
+    ok = get(h->d_wtasks, p.tasks * kTaskBytes) && get(h->d_widx, (s.b_rows + p.index_rows) * kMapBytes) &&
+         get(h->d_wtab, p.index_rows * s.index_bytes);
+  if (!ok) {
+    (void)cudaGetLastError();
+    for (DevBuf* b : {&h->d_wbits, &h->d_wslot, &h->d_wtasks, &h->d_widx, &h->d_wtab}) b->release();
+  }
+  return ok;
+}
+
 // Slots for the wide tier's kept bit vectors of this symbolic call (none when
-// the option is off, no row takes the wide tier or the budget is zero).
+// the option is off, no row takes the wide tier or the budget is zero).  Keeping is
+// optional: it stays within the budget with all that belongs to it, takes at most half
+// of the memory that is free, and a call that cannot have it runs without.
 kk_status keep_for_symbolic(kk_spgemm_handle h, int32_t m, int64_t wide_rows, const CsrView& av,
                             const CsrView& bv) {
   h->keep = WideKeep{};
@@ -1266,17 +1292,28 @@ kk_status keep_for_symbolic(kk_spgemm_handle h, int32_t m, int64_t wide_rows, co
   const bool tasks = h->b_sorted != 0 && bv.n <= kChunkMaxCols && h->opt.force_tier != 0;
   const int32_t chunks = tasks ? wide_max_chunks(bv.n) : 0;
   const size_t stride = words + ((size_t)chunks * 2 + 3) / 4 * 4;
-  const size_t budget = h->opt.wide_cache_mb > 0 ? ((size_t)h->opt.wide_cache_mb << 20) : h->dev_total / 8;
-  long long slots = (long long)(budget / (stride * 4));
-  if (slots > wide_rows) slots = wide_rows;
-  if (slots > 0x7fffffff) slots = 0x7fffffff;
-  if (slots <= 0) return KK_OK;
-  long long ntasks = tasks ? wide_max_tasks(bv.n, h->stats[6], slots) : 0;
-  if (ntasks > (1 << 28)) ntasks = 1 << 28;
-  KK_CUDA(h, h->d_wbits.ensure(stride * 4 * (size_t)slots), "alloc wide cache");
-  KK_CUDA(h, h->d_wslot.ensure(sizeof(int32_t) * (size_t)m), "alloc wide cache");
-  KK_CUDA(h, h->d_wnext.ensure(sizeof(int32_t) * 4), "alloc wide cache");
-  if (tasks) KK_CUDA(h, h->d_wtasks.ensure(sizeof(int2) * (size_t)ntasks), "alloc wide cache");
+  KeepSizes sizes{};
+  sizes.rows = m;
+  sizes.b_rows = bv.m;
+  sizes.wide_rows = wide_rows;
+  sizes.slot_bytes = (long long)stride * 4;
+  if (tasks) {
+    sizes.slot_tasks = wide_slot_tasks(bv.n);
+    sizes.column_tasks = wide_column_tasks(bv.n, h->stats[6]);
+    sizes.long_rows = wide_index_rows(bv);
+    sizes.index_bytes = (long long)wide_index_stride(bv.n) * 4;
+  }
+  long long budget = h->opt.wide_cache_mb > 0 ? (long long)h->opt.wide_cache_mb << 20 : (long long)(h->dev_total / 8);
+  KeepPlan plan = keep_plan(budget, sizes);
+  const long long held = (long long)(h->d_wbits.bytes + h->d_wslot.bytes + h->d_wtasks.bytes + h->d_widx.bytes +
+                                     h->d_wtab.bytes);
+  if (keep_bytes(sizes, plan) > held) {
+    size_t free_bytes = 0, total = 0;
+    KK_CUDA(h, cudaMemGetInfo(&free_bytes, &total), "memory info");
+    const long long most = held + (long long)(free_bytes / 2);
+    if (most < budget) plan = keep_plan(budget = most, sizes);
+  }
+  if (plan.slots <= 0 || !keep_alloc(h, sizes, plan, budget)) return KK_OK;
   KK_CUDA(h, cudaMemsetAsync(h->d_wslot.p, 0xFF, sizeof(int32_t) * (size_t)m, h->stream), "memset");
   KK_CUDA(h, cudaMemsetAsync(h->d_wnext.p, 0, sizeof(int32_t) * 4, h->stream), "memset");
   h->keep.bits = h->d_wbits.as<uint32_t>();
@@ -1284,7 +1321,7 @@ kk_status keep_for_symbolic(kk_spgemm_handle h, int32_t m, int64_t wide_rows, co
   h->keep.next = h->d_wnext.as<int32_t>();
   h->keep.tasks = tasks ? h->d_wtasks.as<int2>() : nullptr;
   h->keep.kept = &h->d_misc.as<Misc>()->wide_kept;
-  h->keep.max_slots = (int32_t)slots;
+  h->keep.max_slots = (int32_t)plan.slots;
   h->keep.min_cnt = !tasks                                ? wide_keep_min_cnt(probe, bv.n)
                     : bv.n <= kRankBits[kNumRankBits - 1] ? kRankNnz[kNumRankNnz - 1]
                                                           : kRankNnz[0];
@@ -1293,17 +1330,14 @@ kk_status keep_for_symbolic(kk_spgemm_handle h, int32_t m, int64_t wide_rows, co
     h->keep.min_cnt = h->opt.num_team_max_nnz;
   h->keep.stride = (int32_t)stride;
   h->keep.max_chunks = chunks;
-  h->keep.max_tasks = (int32_t)ntasks;
+  h->keep.max_tasks = (int32_t)plan.tasks;
   if (tasks) {
-    const size_t rows = (size_t)wide_index_slots(bv), tab = (size_t)wide_index_stride(bv.n);
-    KK_CUDA(h, h->d_widx.ensure(sizeof(int32_t) * ((size_t)bv.m + rows)), "alloc wide cache");
-    KK_CUDA(h, h->d_wtab.ensure(sizeof(int32_t) * rows * tab), "alloc wide cache");
     h->keep.bidx = h->d_widx.as<int32_t>();
     h->keep.btab = h->d_wtab.as<int32_t>();
-    h->keep.tab_stride = (int32_t)tab;
+    h->keep.tab_stride = wide_index_stride(bv.n);
     h->keep.shift = wide_chunk_shift(bv.n);
-    KK_CUDA(h, launch_chunk_index(ctx_of(h), bv, h->d_widx.as<int32_t>(), h->d_widx.as<int32_t>() + bv.m,
-                                  h->d_wtab.as<int32_t>()),
+    KK_CUDA(h, launch_chunk_index(ctx_of(h), bv, (int32_t)plan.index_rows, h->d_widx.as<int32_t>(),
+                                  h->d_widx.as<int32_t>() + bv.m, h->d_wtab.as<int32_t>()),
             "index launch");
     KK_TRY(symbolic_fingerprint(h, av, bv));
   }

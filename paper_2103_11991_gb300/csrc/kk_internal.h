@@ -304,10 +304,12 @@ cudaError_t launch_numeric_wide(const LaunchCtx& ctx, const CsrView& A, const Cs
 // longer rows that their numeric phase uses.
 int32_t wide_chunk_shift(int32_t k);
 int32_t wide_max_chunks(int32_t k);                                       // of a row of k columns
-long long wide_max_tasks(int32_t k, long long flops, long long slots);  // of `slots` rows with `flops` products
+long long wide_slot_tasks(int32_t k);                    // tasks that a row needs whatever its columns
+long long wide_column_tasks(int32_t k, long long flops);  // further tasks of rows with `flops` products together
 int32_t wide_index_stride(int32_t k);
-int32_t wide_index_slots(const CsrView& B);
-cudaError_t launch_chunk_index(const LaunchCtx& ctx, const CsrView& B, int32_t* slot, int32_t* row, int32_t* tab);
+int32_t wide_index_rows(const CsrView& B);  // rows of B worth an index, at most
+cudaError_t launch_chunk_index(const LaunchCtx& ctx, const CsrView& B, int32_t max_rows, int32_t* slot, int32_t* row,
+                               int32_t* tab);
 // (fp: structure fingerprints of the symbolic call and of this one).
 cudaError_t launch_num_chunk(const LaunchCtx& ctx, const CsrView& A, const CsrView& B, const unsigned long long* fp,
                              const int64_t* c_rowptr, int32_t* c_colind, double* c_vals);

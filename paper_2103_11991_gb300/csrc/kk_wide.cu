@@ -1200,20 +1200,19 @@ bool wide_numeric_fits(const LaunchCtx& ctx, int32_t k) {
 
 int32_t wide_chunk_shift(int32_t k) { return chunk_shift(k); }
 int32_t wide_max_chunks(int32_t k) { return k / chunk_cols(k) + wide_words(k) / kChunkWords + 2; }
-long long wide_max_tasks(int32_t k, long long flops, long long slots) {
-  // a chunk ends with every chunk_cols columns (a column has a product) and at
-  // fixed words
-  return flops / chunk_cols(k) + slots * (wide_words(k) / kChunkWords + 2);
-}
+// a chunk ends at fixed words, and with every chunk_cols columns (a column has a product)
+long long wide_slot_tasks(int32_t k) { return wide_words(k) / kChunkWords + 2; }
+long long wide_column_tasks(int32_t k, long long flops) { return flops / chunk_cols(k); }
 int32_t wide_index_stride(int32_t k) { return (wide_words(k) * 32 >> chunk_shift(k)) + 1; }
-int32_t wide_index_slots(const CsrView& B) { return B.nnz / kIndexMinLen + 1; }
+int32_t wide_index_rows(const CsrView& B) { return min(B.m, B.nnz / kIndexMinLen); }
 
-cudaError_t launch_chunk_index(const LaunchCtx& ctx, const CsrView& B, int32_t* slot, int32_t* row, int32_t* tab) {
-  const int slots = wide_index_slots(B), stride = wide_index_stride(B.n);
+cudaError_t launch_chunk_index(const LaunchCtx& ctx, const CsrView& B, int32_t max_rows, int32_t* slot, int32_t* row,
+                               int32_t* tab) {
+  const int stride = wide_index_stride(B.n);
   timer_begin(ctx.timer, ctx.stream, "chunk_index");
-  k_index_rows<<<min(ctx.num_sms * 8, (B.m + 255) / 256), 256, 0, ctx.stream>>>(B.m, B.rowptr, slots, slot, row,
+  k_index_rows<<<min(ctx.num_sms * 8, (B.m + 255) / 256), 256, 0, ctx.stream>>>(B.m, B.rowptr, max_rows, slot, row,
                                                                             ctx.keep.next + 3);
-  k_index_fill<<<ctx.num_sms * 8, 256, 0, ctx.stream>>>(B, chunk_shift(B.n), stride, slots, row, ctx.keep.next + 3,
+  k_index_fill<<<ctx.num_sms * 8, 256, 0, ctx.stream>>>(B, chunk_shift(B.n), stride, max_rows, row, ctx.keep.next + 3,
                                                        tab);
   timer_end(ctx.timer, ctx.stream);
   return cudaGetLastError();
