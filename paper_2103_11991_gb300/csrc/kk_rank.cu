@@ -53,8 +53,8 @@ struct RankGeom {
   int words, vmax;
   uint32_t pre_off, val_off, info_off, col_off, tag_off, bytes;
 };
-RankGeom rank_geom(int bits, int vmax, int nw) {
-  RankGeom g;
+constexpr RankGeom rank_geom(int bits, int vmax, int nw) {
+  RankGeom g{};
   // the window may start anywhere inside its first word
   const int unit = 128 * nw;
   g.words = (int)((((long long)bits + 31) / 32 + 1 + unit - 1) / unit * unit);
@@ -67,6 +67,13 @@ RankGeom rank_geom(int bits, int vmax, int nw) {
   g.bytes = g.tag_off + (uint32_t)al16((size_t)vmax + 16);
   return g;
 }
+
+// Every launch fits the 48 KB that need no function attribute: one set to each
+// launch's own size could be lowered by another thread's launch in between.
+constexpr size_t kRankPlainSmem = 48 * 1024 - 1024;
+static_assert(rank_geom(kRankBits[kNumRankBits - 1], kRankNnz[kNumRankNnz - 1], 2).bytes <= kRankPlainSmem &&
+                  kRankPairBytes * 2 <= kRankPlainSmem,
+              "k_num_rank's shared memory");
 
 struct RankArgs {
   CsrView A, B;
@@ -136,6 +143,8 @@ __device__ __forceinline__ u64 rank_add(u64 v, bool df, int2 a, float2 b) {
 // are loaded together and each costs one OR (90,666 rows of 510 products in 60,013
 // columns: 657 us by hash, 123 so; bound by the ORs and the load latency).
 constexpr int kSymRankWarps = 4;
+static_assert((size_t)kSymRankWarps * rank_geom(kRankBits[kNumRankBits - 1], 0, 1).words * 4 <= kRankPlainSmem,
+              "k_sym_rank's shared memory");
 __global__ void __launch_bounds__(kSymRankWarps * 32)
 k_sym_rank(CsrView A, CsrView B, const int32_t* __restrict__ rows, int32_t nrows, int32_t nwords,
            int32_t* __restrict__ cnt, int* status) {
@@ -491,8 +500,6 @@ cudaError_t launch_sym_rank(const LaunchCtx& ctx, const BinSpec& bin, const CsrV
   if (nrows <= 0) return cudaSuccess;
   const int nwords = rank_geom(B.n < bin.slots ? B.n : bin.slots, 0, 1).words;
   const size_t smem = (size_t)kSymRankWarps * nwords * 4;
-  cudaError_t e = cudaFuncSetAttribute(k_sym_rank, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sym_rank, kSymRankWarps * 32, smem) != cudaSuccess ||
       per_sm < 1) {
@@ -522,8 +529,6 @@ cudaError_t launch_num_rank(const LaunchCtx& ctx, const BinSpec& bin, const CsrV
                                   : (df ? k_num_rank<1, false, true> : k_num_rank<1, false, false>));
   const int rpc = kRankThreads / 32 / nw;  // rows per CTA
   const size_t smem = (size_t)rpc * geo.bytes;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   // one resident wave: neighbouring rows are in flight together and share B rows in L2
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kRankThreads, smem) != cudaSuccess ||

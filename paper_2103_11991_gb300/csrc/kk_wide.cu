@@ -1127,7 +1127,7 @@ k_num_chunk(CsrView A, CsrView B, int32_t words, const unsigned long long* __res
 // static arrays take the rest of the opt-in limit).
 template <int BLOCK>
 size_t wide_static() {
-  return sizeof(WideWalkSmem<BLOCK>) + 33 * sizeof(int) + 512;
+  return sizeof(WideWalkSmem<BLOCK>) + 33 * sizeof(int) + 512 + 64;
 }
 size_t wide_budget(const LaunchCtx& ctx) {
   return (size_t)ctx.max_smem_optin > wide_static<kWideBlock>() ? (size_t)ctx.max_smem_optin - wide_static<kWideBlock>()
@@ -1149,12 +1149,20 @@ int wide_block(const LaunchCtx& ctx, size_t dyn, bool light) {
   return kWideBlock;
 }
 
+// A kernel's limit of dynamic shared memory, the same for every launch: another
+// thread's launch of a smaller size must not lower it in between.
+template <int BLOCK, class Kernel>
+cudaError_t wide_smem_limit(const LaunchCtx& ctx, Kernel kern) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)((size_t)ctx.max_smem_optin - wide_static<BLOCK>()));
+}
+
 template <int BLOCK, bool PAIRS>
 cudaError_t sym_wide(const LaunchCtx& ctx, const CsrView& A, const CsrView& B, const BComp& bc, int words,
                      const WideGeom& g, uint32_t stage_off, size_t bytes, const long long* flop,
                      const int32_t* rows, int32_t nrows, int32_t* cnt) {
   auto kern = k_sym_wide<BLOCK, PAIRS>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  cudaError_t e = wide_smem_limit<BLOCK>(ctx, kern);
   if (e != cudaSuccess) return e;
   long long grid = (long long)ctx.num_sms * wide_per_sm(ctx, bytes + wide_static<BLOCK>(), BLOCK);
   if (grid > nrows) grid = nrows;
@@ -1168,7 +1176,7 @@ cudaError_t num_wide(const LaunchCtx& ctx, const CsrView& A, const CsrView& B, i
                      const int64_t* c_rowptr, const int32_t* rows, int32_t nrows, int32_t* c_colind,
                      double* c_vals) {
   auto kern = k_num_wide<BLOCK>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.bytes);
+  cudaError_t e = wide_smem_limit<BLOCK>(ctx, kern);
   if (e != cudaSuccess) return e;
   long long grid = (long long)ctx.num_sms * wide_per_sm(ctx, g.bytes + wide_static<BLOCK>(), BLOCK);
   if (grid > nrows) grid = nrows;
