@@ -10,9 +10,11 @@
  * Input rows may be unsorted and may repeat columns.
  *
  * Two phases, as in the paper: the symbolic phase counts the entries of every
- * row of C and keeps, in the handle, the slot in C's row of every entry of A
- * and of B; the numeric phase scatters alpha a and beta b to those slots, for
- * any values of A and B on the same index arrays (symbolic reuse).
+ * row of C and keeps, in the handle, how the numeric phase puts the row together;
+ * the numeric phase does so for any values of A and B on the same index arrays
+ * (symbolic reuse).  Rows that are strictly ascending in both matrices are merged
+ * (short ones by searching again, up to 256 combined entries by one bit per entry of
+ * C's row and of A's); of the others the slot in C's row of every entry is kept.
  *
  * kk_spadd_symbolic: A, B (values not read), c_rowptr device int64[m + 1]
  *   caller-allocated; *nnz_c (host) receives nnz(C).  Blocks until nnz(C) is on
@@ -27,7 +29,7 @@
  *   alpha a + beta b (each product rounded once, one rounded sum); repeated
  *   columns within A or B are added in no fixed order, within
  *   1e-12 * (sum |alpha a| + sum |beta b|).
- * The handle keeps int32 slots for nnz(A) + nnz(B) entries and int32 per row.
+ * The handle keeps room for nnz(A) + nnz(B) int32 slots and 9 bytes per row.
  */
 #ifndef KK_SPADD_H_
 #define KK_SPADD_H_

@@ -853,7 +853,7 @@ struct kk_spgemm_handle_s {
   DevBuf d_jpos;       // int32[m]: position of each row's first diagonal entry (Jacobi)
   DevBuf d_apos, d_bpos;  // SpAdd: slot in C's row of every entry of A and of B (int32)
   DevBuf d_acnt;          // SpAdd: nnz(C(i,:)) (int32[m])
-  DevBuf d_akind;         // SpAdd: 1 for a row merged by the numeric phase (uint8[m])
+  DevBuf d_akind;         // SpAdd: how the numeric phase takes every row (uint8[m])
   DevBuf d_along;         // SpAdd: long rows, their count first (int32[m + 1])
   // learned form
   DevBuf d_params;     // float[KK_MLP_NUM_PARAMS]
@@ -878,6 +878,7 @@ struct kk_spgemm_handle_s {
   const void* add_key[4] = {nullptr, nullptr, nullptr, nullptr};
   int32_t add_m = 0, add_n = 0, add_nnza = 0, add_nnzb = 0;
   int64_t add_nnzc = 0;
+  int32_t add_kinds[3] = {0, 0, 0};
   std::vector<int32_t> lnum_start;
   // batched form
   DevBuf d_bdesc, d_rowpair, d_bflop, d_bsbin, d_bnbin, d_bsrows, d_bnrows, d_bcnt, d_btiles, d_bstart,
@@ -938,6 +939,7 @@ namespace {
 
 struct Misc {
   int status;
+  int32_t add_kinds[3];  // SpAdd: 1 when there are rows for teams, warps, CTAs (right after status)
   int32_t sorted;
   int32_t range_bad;
   int32_t pad;
@@ -2025,9 +2027,10 @@ kk_status kk_spadd_symbolic(kk_spgemm_handle h, const kk_csr* A, const kk_csr* B
   KK_CUDA(h, h->d_bpos.ensure(sizeof(int32_t) * (size_t)(B->nnz > 0 ? B->nnz : 1)), "alloc SpAdd");
   KK_CUDA(h, h->d_acnt.ensure(sizeof(int32_t) * (size_t)(m > 0 ? m : 1)), "alloc SpAdd");
   KK_CUDA(h, h->d_along.ensure(sizeof(int32_t) * ((size_t)m + 1)), "alloc SpAdd");
-  // only the status word is reset: the rest of the device record belongs to
-  // the SpGEMM state of this handle (fingerprints, flags), which SpAdd leaves alone
-  KK_CUDA(h, cudaMemsetAsync(&dm->status, 0, sizeof(int), s), "memset");
+  // only the status word and SpAdd's own flags behind it are reset: the rest of the
+  // device record belongs to the SpGEMM state of this handle (fingerprints, flags),
+  // which SpAdd leaves alone
+  KK_CUDA(h, cudaMemsetAsync(&dm->status, 0, sizeof(int) + sizeof(dm->add_kinds), s), "memset");
   KK_CUDA(h, h->d_akind.ensure((size_t)(m > 0 ? m : 1)), "alloc SpAdd");
   int32_t* long_rows = h->d_along.as<int32_t>();
   KK_CUDA(h, cudaMemsetAsync(long_rows, 0, sizeof(int32_t), s), "memset");
@@ -2037,7 +2040,7 @@ kk_status kk_spadd_symbolic(kk_spgemm_handle h, const kk_csr* A, const kk_csr* B
     timer_begin(h->timer, s, "spadd_symbolic");
     cudaError_t e = launch_spadd_symbolic(ctx, view(A), view(B), h->d_acnt.as<int32_t>(),
                                           h->d_apos.as<int32_t>(), h->d_bpos.as<int32_t>(),
-                                          h->d_akind.as<uint8_t>(), long_rows);
+                                          h->d_akind.as<uint8_t>(), long_rows, dm->add_kinds);
     timer_end(h->timer, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "SpAdd symbolic launch");
     timer_begin(h->timer, s, "scan");
@@ -2061,6 +2064,7 @@ kk_status kk_spadd_symbolic(kk_spgemm_handle h, const kk_csr* A, const kk_csr* B
   h->add_nnza = A->nnz;
   h->add_nnzb = B->nnz;
   h->add_nnzc = nnz;
+  for (int t = 0; t < 3; ++t) h->add_kinds[t] = m > 0 ? hm->add_kinds[t] : 0;
   *nnz_c = nnz;
   return KK_OK;
 }
@@ -2084,7 +2088,7 @@ kk_status kk_spadd_numeric(kk_spgemm_handle h, double alpha, const kk_csr* A, do
   timer_begin(h->timer, s, "spadd_numeric");
   cudaError_t e = launch_spadd_numeric(ctx_of(h), view(A), view(B), alpha, beta, c_rowptr,
                                        h->d_apos.as<int32_t>(), h->d_bpos.as<int32_t>(), h->d_akind.as<uint8_t>(),
-                                       c_colind, c_vals);
+                                       h->d_along.as<int32_t>(), h->add_kinds, c_colind, c_vals);
   timer_end(h->timer, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "SpAdd numeric launch");
   return KK_OK;

@@ -196,15 +196,18 @@ struct BinSpec {
 // Analysis of B (kk_window.cu): clears *sorted_flag unless every row is
 // strictly ascending, sets KK_ERR_BAD_INDEX on out-of-range structure, and,
 // when bc is non-null, writes the compressed rows (pairs counted into *pairs).
-// Sparse matrix addition (kk_spadd.cu): symbolic counts and, for rows that are
-// not merged, the slots of A's and B's entries in C (long_rows: a list of up to
-// m rows, its count in the first element, zeroed by the caller; kind: per row, 1
-// when it is merged); numeric writes C's columns and values.
+// Sparse matrix addition (kk_spadd.cu): symbolic counts, and what the numeric phase
+// goes by: per row its kind, and (in apos and bpos) its bits or its entries' slots in C
+// (long_rows: a list of up to m rows, its count in the first element, zeroed by the
+// caller; kinds: whether there are rows for teams, warps and CTAs, on the device, zeroed
+// by the caller); numeric writes C's columns and values (kinds: on the
+// host).
 cudaError_t launch_spadd_symbolic(const LaunchCtx& ctx, const CsrView& A, const CsrView& B, int32_t* cnt,
-                                  int32_t* apos, int32_t* bpos, uint8_t* kind, int32_t* long_rows);
+                                  int32_t* apos, int32_t* bpos, uint8_t* kind, int32_t* long_rows, int32_t* kinds);
 cudaError_t launch_spadd_numeric(const LaunchCtx& ctx, const CsrView& A, const CsrView& B, double alpha,
                                  double beta, const int64_t* c_rowptr, const int32_t* apos,
-                                 const int32_t* bpos, const uint8_t* kind, int32_t* c_colind, double* c_vals);
+                                 const int32_t* bpos, const uint8_t* kind, const int32_t* long_rows, const int32_t* kinds,
+                                 int32_t* c_colind, double* c_vals);
 
 // Numeric phase of window rows with kept structure (kk_kept.cu).
 cudaError_t launch_num_kept(const LaunchCtx& ctx, const CsrView& A, const CsrView& B,
