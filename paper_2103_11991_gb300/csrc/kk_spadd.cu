@@ -306,6 +306,9 @@ k_spadd_count(CsrView A, CsrView B, int32_t* __restrict__ cnt, int32_t* __restri
               int32_t* __restrict__ bpos, uint8_t* __restrict__ kind, int32_t* __restrict__ long_rows,
               int32_t* __restrict__ kinds, int* status) {
   __shared__ u64 keys[kAddRowWarps][kAddWarpMax];
+  __shared__ unsigned cta_kinds;
+  if (threadIdx.x == 0) cta_kinds = 0u;
+  __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tl = lane % T, tm = lane / T;
   const unsigned team = team_mask<T>();
   const long long stride = (long long)gridDim.x * kAddRowWarps * (32 / T);
@@ -372,11 +375,16 @@ k_spadd_count(CsrView A, CsrView B, int32_t* __restrict__ cnt, int32_t* __restri
     }
   }
   if (bad) set_status(status, KK_ERR_BAD_INDEX);
-  // (looked at first: a store of every warp to one address takes its turn)
-  volatile int32_t* seen = kinds;
-  if (by_team && seen[0] == 0) seen[0] = 1;
-  if (by_warp && seen[1] == 0) seen[1] = 1;
-  if (by_cta && seen[2] == 0) seen[2] = 1;
+  // (one store per CTA, and only until it is seen: stores of every warp to one address
+  // take turns, 70 us for 26,738 rows)
+  const unsigned seen = (by_team ? 1u : 0u) | (by_warp ? 2u : 0u) | (by_cta ? 4u : 0u);
+  const unsigned mine = __reduce_or_sync(kFull, seen);
+  if (lane == 0 && mine) atomicOr(&cta_kinds, mine);
+  __syncthreads();
+  if (threadIdx.x < 3 && (cta_kinds >> threadIdx.x & 1u)) {
+    volatile int32_t* flag = kinds + threadIdx.x;
+    if (*flag == 0) *flag = 1;
+  }
 }
 
 // One CTA of kAddCtaThreads per long row (dynamic shared memory kAddCtaMax keys).
