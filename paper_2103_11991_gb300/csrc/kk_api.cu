@@ -156,6 +156,7 @@ struct BinTable {
   int32_t win_kept[kMaxWindowBins];     // 1: rows with kept structure only
   int32_t win_order[kMaxWindowBins];    // 0: sorted B only, 1: any, 2: unsorted only
   long long win_q[kMaxWindowBins];      // largest binning quantity of each window bin
+  int32_t win_qlo[kMaxWindowBins];      // the binning quantity must exceed this
   long long win_ratio[kMaxWindowBins];  // window W only when W <= ratio * flop
 };
 
@@ -168,7 +169,7 @@ __device__ __forceinline__ uint8_t classify(const BinTable& t, long long q, int 
   const int sp = sorted ? span : t.cols;
   if (sp > 0) {
     for (int w = 0; w < t.nwin; ++w)
-      if (wq <= t.win_q[w] && sp <= t.win_bits[w] && t.win_order[w] != (sorted ? 2 : 0) && (!t.win_kept[w] || kept) &&
+      if (wq <= t.win_q[w] && q > t.win_qlo[w] && sp <= t.win_bits[w] && t.win_order[w] != (sorted ? 2 : 0) && (!t.win_kept[w] || kept) &&
           (long long)t.win_bits[w] <= (q > kRankMinNnz ? t.win_ratio[w] : (long long)kWindowFlopRatio) * flop)
         return (uint8_t)t.win_bin[w];
   }
@@ -1106,6 +1107,12 @@ BinTable to_table(const std::vector<BinSpec>& bins, bool numeric, int32_t cols, 
       t.win_kept[t.nwin] = numeric && !rank ? 1 : 0;
       t.win_order[t.nwin] = !rank ? 0 : numeric ? 1 : 2;
       t.win_ratio[t.nwin] = rank ? kRankFlopRatio : kWindowFlopRatio;
+      const int32_t bits = bins[b].slots;
+      t.win_qlo[t.nwin] = !rank || !automatic        ? 0
+                          : bits > kRankShortBits    ? kRankWideMinNnz
+                          : !numeric                 ? kRankMinFlop
+                          : bits > kRankBits[0]      ? kRankMinNnz
+                                                     : 0;
       ++t.nwin;
     } else {
       t.nb = (int32_t)b + 1;

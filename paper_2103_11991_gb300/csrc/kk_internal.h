@@ -162,6 +162,14 @@ constexpr int32_t kRankNnz[kNumRankNnz] = {256, 512, 1024};
 // the team tier, 400 in the rank tier).
 constexpr int32_t kRankFlopRatio = 512;
 constexpr int32_t kRankMinNnz = 32;
+// ... and (automatic tiers) only for rows of more columns (numeric) or products
+// (symbolic) than these, where the window is wider than the first class and than
+// kRankShortBits: fewer are done sooner by hash.  300,000 rows, hash and rank: 36
+// columns in 8,192 580 and 465 us, in 16,384 595 and 501; 63 columns in 32,768 650 and
+// 798; 9-point rows of a 1,080 x 614 grid, 25 columns of 81 products in 4,325, 837 and
+// 1,054; symbolic 36 products of an unsorted B 225 and 305, 49 products 275 and 280,
+// 100 products 357 and 265.
+constexpr int32_t kRankShortBits = 16384, kRankWideMinNnz = 64, kRankMinFlop = 56;
 // Symbolic rank rows: flop bound <= this, the line of the window tier for a B as
 // narrow; heavier rows are too many products for one warp and stay where they were.
 constexpr long long kRankMaxFlop = 4096;
