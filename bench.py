@@ -860,12 +860,12 @@ def run_ours(args, rank, world, local_rank):
     # (structure + values) and C rows (row pointers read, columns + values
     # written), plus all of B (structure + values), which those rows reference.
     # The window tier runs as two kernels: num_kept (rows whose structure the
-    # symbolic phase kept) and num_window (the rest); the tier's bytes go with
+    # symbolic phase kept) and num_rank (the rest); the tier's bytes go with
     # their summed time.
-    tier_of = {"num_kept": "window", "num_window": "window", "num_warp_vec": "team",
+    tier_of = {"num_kept": "window", "num_rank": "window", "num_warp_vec": "team",
                "num_team_vec": "team", "num_team_flat": "team", "num_cta": "cta", "num_dense": "dense"}
     if tier_of.get(dom_name) == "window":
-        dom_ms = sum(kt[k][0] for k in ("num_kept", "num_window") if k in kt)
+        dom_ms = sum(kt[k][0] for k in ("num_kept", "num_rank") if k in kt)
     dom_madds = None
     if dom_name in tier_of:
         t = tier_of[dom_name]

@@ -66,11 +66,15 @@ typedef struct {
 
 /* Arithmetic of the numeric phase's accumulator. */
 typedef enum {
-  KK_ARITH_AUTO = 0,  /* DF32 where every value's exponent fits its safe range and the row's
-                         error bound holds, FP64 otherwise; the window tier's rows of at most 256
-                         columns run in FP64 (measured faster there on GB300) */
-  KK_ARITH_FP64 = 1,  /* native float64 fused multiply-add in storage order */
-  KK_ARITH_DF32 = 2   /* float64 emulated as an unevaluated pair of float32 on the FP32 pipe */
+  KK_ARITH_AUTO = 0,  /* DF32 in the hash tiers, where every value's exponent fits its safe range
+                         and the row's error bound holds; FP64 otherwise and in all other tiers
+                         (measured faster there on GB300) */
+  KK_ARITH_FP64 = 1,  /* native float64: fused multiply-adds in storage order, but for rows of the
+                         wide tier and its column chunks (from 257 columns on, where B has more than
+                         65,536 columns; from 1,025 otherwise) and flattened hash rows, whose
+                         products are added in no fixed order */
+  KK_ARITH_DF32 = 2   /* float64 emulated as an unevaluated pair of float32 on the FP32 pipe, in the
+                         hash, window and rank tiers; the other tiers run in float64 */
 } kk_arith;
 
 /* Options; kk_spgemm_options_default fills the defaults.  A NULL options
@@ -91,8 +95,9 @@ typedef struct {
                                  (default 1024; with the default, not those whose bits the wide tier
                                  kept) */
   int32_t num_cta_max_nnz;    /* rows up to this nnz use a CTA hash; above it dense chunks */
-  int32_t use_window;         /* 1: rows whose column span fits a shared-memory window use the
-                                 dense window accumulator (needs B rows sorted) */
+  int32_t use_window;         /* 1: rows whose column span fits a shared-memory window use a dense
+                                 accumulator over it: B rows sorted, the window and rank tiers; B
+                                 unsorted and of at most 65,536 columns, the rank tier */
   int32_t batched_graph;      /* 1: batched phases are captured into CUDA graphs and replayed
                                  (needs a non-default stream) */
   int32_t sym_load_pct;       /* hash tables of the symbolic phase are sized so the flop bound
@@ -193,6 +198,7 @@ kk_status kk_spgemm_kernel_times(kk_spgemm_handle h, int32_t max_kernels, const 
 
 /* Statistics: rows per tier in each phase of the last symbolic call
  * (stats[0..2] symbolic team/CTA/dense, stats[3..5] numeric team/CTA/dense),
+ * rows of the thread tier count as team, those of the rank tier as window rows;
  * stats[6] = total flops (multiply-adds), stats[7] = 1 if B's rows were
  * strictly ascending, stats[8] / stats[9] = kernels launched by the last
  * symbolic / numeric call, stats[10] / stats[11] = rows in the window tier of

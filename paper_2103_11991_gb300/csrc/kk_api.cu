@@ -138,8 +138,8 @@ constexpr uint8_t kSkipBin = 0xFF;
 // The thread bin (first) comes before everything, then the window bins: a row
 // qualifies for one when its span fits win_bits, the window is not too wide for
 // its flop count and q lies in the bin's range.  Kept bins (numeric) also need
-// the structure kept by the symbolic phase; the others take unsorted B too
-// (any_order), over all of its columns.  wq is the quantity of the window bins: q,
+// the structure kept by the symbolic phase; those whose win_order admits it take
+// unsorted B too, over all of its columns.  wq is the quantity of the window bins: q,
 // or less for a row whose work there is not its products; rows of a sorted B beyond
 // team_max leave the team tier.
 struct BinTable {
@@ -169,7 +169,8 @@ __device__ __forceinline__ uint8_t classify(const BinTable& t, long long q, int 
   const int sp = sorted ? span : t.cols;
   if (sp > 0) {
     for (int w = 0; w < t.nwin; ++w)
-      if (wq <= t.win_q[w] && q > t.win_qlo[w] && sp <= t.win_bits[w] && t.win_order[w] != (sorted ? 2 : 0) && (!t.win_kept[w] || kept) &&
+      if (wq <= t.win_q[w] && q > t.win_qlo[w] && sp <= t.win_bits[w] && t.win_order[w] != (sorted ? 2 : 0) &&
+          (!t.win_kept[w] || kept) &&
           (long long)t.win_bits[w] <= (q > kRankMinNnz ? t.win_ratio[w] : (long long)kWindowFlopRatio) * flop)
         return (uint8_t)t.win_bin[w];
   }
@@ -1373,9 +1374,9 @@ const int32_t* kept_counts(kk_spgemm_handle h) { return h->cache_valid ? h->d_cn
 // Slots of the rows of this symbolic call kept with chunk tasks (-1: none).
 const int32_t* kept_slots(kk_spgemm_handle h) { return h->keep.tasks ? h->keep.slot : nullptr; }
 
-// The kept structure, if it belongs to these index arrays.  Unless options.debug_checks asks for a check of
-// every product, the arrays' fingerprint is taken again and ctx->fingerprint
-// points the numeric kernels at both fingerprints.
+// The kept structure, if it belongs to these index arrays.  Unless
+// options.debug_checks asks for a check of every product, the arrays' fingerprint
+// is taken again and ctx->fingerprint points the numeric kernels at both.
 kk_status cache_view(kk_spgemm_handle h, const CsrView& av, const CsrView& bv, WinCacheView* view, LaunchCtx* ctx) {
   *view = WinCacheView{nullptr, nullptr, nullptr};
   if (!h->cache_valid || h->cache_key[0] != av.rowptr || h->cache_key[1] != av.colind ||
@@ -1539,7 +1540,8 @@ static void launch_analyze_a_t(kk_spgemm_handle h, const CsrView& av, const CsrV
   }
   const int64_t m = LISTED ? lr.most : av.m;
   kern<<<grid_for(m * T, 256, h->num_sms * (per_sm > 0 ? per_sm : 1)), 256, 0, s>>>(
-      av, bv.rowptr, bv.colind, h->opt.use_window ? h->d_bclen.as<int32_t>() : nullptr, bv.m, &dm->sorted, symbolic_table(h, bv.n), h->opt.team_vec_min_len,
+      av, bv.rowptr, bv.colind, h->opt.use_window ? h->d_bclen.as<int32_t>() : nullptr, bv.m, &dm->sorted,
+      symbolic_table(h, bv.n), h->opt.team_vec_min_len,
       h->d_flop.as<long long>(), bin, h->d_rowlo.as<int32_t>(), h->d_span.as<int32_t>(), stat,
       &dm->total_flop, &dm->status, lr);
 }
@@ -1941,7 +1943,8 @@ static kk_status numeric_impl(kk_spgemm_handle h, const kk_csr* A, const kk_csr*
       if (e != cudaSuccess) return cuda_fail(h, e, "Jacobi launch");
     }
   }
-  if ((st = launch_kept_chunks(h, ctx, av, bv, h->num_start, c_rowptr, c_colind, c_vals, &skip_wide)) != KK_OK) return st;
+  if ((st = launch_kept_chunks(h, ctx, av, bv, h->num_start, c_rowptr, c_colind, c_vals, &skip_wide)) != KK_OK)
+    return st;
   for (int b = 0; b < nbn; ++b) {
     const int cnt = h->num_start[b + 1] - h->num_start[b];
     if (cnt <= 0) continue;
@@ -2615,7 +2618,8 @@ kk_status kk_spgemm_batched_symbolic(kk_spgemm_handle h, int32_t count, const kk
   KK_CUDA(h, h->d_bstart.ensure(sizeof(int32_t) * 2 * (kMaxBBins + 1)), "alloc batch");
   KK_CUDA(h, h->d_bqueue.ensure(sizeof(int) * 2), "alloc batch");
   KK_CUDA(h, h->d_boff.ensure(sizeof(int64_t) * ((size_t)count + 1)), "alloc batch");
-  KK_CUDA(h, h->d_blk.ensure(sizeof(int32_t) * ((size_t)nbmax * (size_t)(nblk > 0 ? nblk : 1) + kMaxBins)), "alloc bins");
+  KK_CUDA(h, h->d_blk.ensure(sizeof(int32_t) * ((size_t)nbmax * (size_t)(nblk > 0 ? nblk : 1) + kMaxBins)),
+          "alloc bins");
   KK_CUDA(h, h->d_scan.ensure(sizeof(long long) * (size_t)(nblk_scan > 0 ? nblk_scan : 1)), "alloc scan");
   if (h->d_span.bytes == 0) KK_CUDA(h, h->d_span.ensure(4), "alloc");
   if (h->d_flop.bytes == 0) KK_CUDA(h, h->d_flop.ensure(8), "alloc");
@@ -2823,8 +2827,8 @@ kk_status kk_spgemm_destroy(kk_spgemm_handle h) {
                     &h->d_bnrows, &h->d_bcnt, &h->d_btiles, &h->d_bstart, &h->d_bqueue, &h->d_bsplit2,
                     &h->d_boff, &h->d_bc, &h->d_bclen, &h->d_cw, &h->d_cm, &h->d_cn, &h->d_wbits,
                     &h->d_wslot, &h->d_wnext, &h->d_wtasks, &h->d_widx, &h->d_wtab, &h->d_along_rows, &h->d_blong,
-                    &h->d_pa_rp, &h->d_pa_ci, &h->d_pa_v, &h->d_pb_rp, &h->d_pb_ci, &h->d_pb_v, &h->d_pbase, &h->d_jvals,
-                    &h->d_jpos, &h->d_apos, &h->d_bpos, &h->d_acnt, &h->d_akind, &h->d_along})
+                    &h->d_pa_rp, &h->d_pa_ci, &h->d_pa_v, &h->d_pb_rp, &h->d_pb_ci, &h->d_pb_v, &h->d_pbase,
+                    &h->d_jvals, &h->d_jpos, &h->d_apos, &h->d_bpos, &h->d_acnt, &h->d_akind, &h->d_along})
     b->release();
   for (void* p : {h->h_bdesc, h->h_bdesc2, h->h_boff})
     if (p) cudaFreeHost(p);

@@ -201,9 +201,6 @@ struct BinSpec {
   int64_t lo, hi; // bin range of the binning quantity (flop or nnz), inclusive
 };
 
-// Analysis of B (kk_window.cu): clears *sorted_flag unless every row is
-// strictly ascending, sets KK_ERR_BAD_INDEX on out-of-range structure, and,
-// when bc is non-null, writes the compressed rows (pairs counted into *pairs).
 // Sparse matrix addition (kk_spadd.cu): symbolic counts, and what the numeric phase
 // goes by: per row its kind, and (in apos and bpos) its bits or its entries' slots in C
 // (long_rows: a list of up to m rows, its count in the first element, zeroed by the
@@ -214,8 +211,8 @@ cudaError_t launch_spadd_symbolic(const LaunchCtx& ctx, const CsrView& A, const 
                                   int32_t* apos, int32_t* bpos, uint8_t* kind, int32_t* long_rows, int32_t* kinds);
 cudaError_t launch_spadd_numeric(const LaunchCtx& ctx, const CsrView& A, const CsrView& B, double alpha,
                                  double beta, const int64_t* c_rowptr, const int32_t* apos,
-                                 const int32_t* bpos, const uint8_t* kind, const int32_t* long_rows, const int32_t* kinds,
-                                 int32_t* c_colind, double* c_vals);
+                                 const int32_t* bpos, const uint8_t* kind, const int32_t* long_rows,
+                                 const int32_t* kinds, int32_t* c_colind, double* c_vals);
 
 // Numeric phase of window rows with kept structure (kk_kept.cu).
 cudaError_t launch_num_kept(const LaunchCtx& ctx, const CsrView& A, const CsrView& B,
@@ -243,6 +240,9 @@ struct LongRows {
   int32_t most;
 };
 
+// Analysis of B (kk_analyze.cu): clears *sorted_flag unless every row is
+// strictly ascending, sets KK_ERR_BAD_INDEX on out-of-range structure, and,
+// when bc is non-null, writes the compressed rows (pairs counted into *pairs).
 cudaError_t launch_analyze_b(const LaunchCtx& ctx, const CsrView& B, int32_t* sorted_flag,
                              int2* bc, int32_t* len, unsigned long long* pairs, const LongRows& lr);
 

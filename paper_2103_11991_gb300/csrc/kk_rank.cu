@@ -17,9 +17,10 @@
 // window rows of a 256-pair batch took 8.9 ms and its hash rows 4.6, together 5.2
 // here).  90,666 rows of about 500 columns of an unsorted B take 592 us: 1,250 with
 // an entry of A at a time, 905 flattened, 800 without branches, then two warps per
-// row where a row's shared memory leaves few of them on an SM.  C's columns come from the products themselves (each writes its
-// column's offset beside its value), not from expanding the bits; a slot that no
-// product wrote means that B is not the one whose compressed rows gave the bits.
+// row where a row's shared memory leaves few of them on an SM.  C's columns come
+// from the products themselves (each writes its column's offset beside its value),
+// not from expanding the bits; a slot that no product wrote means that B is not the
+// one whose compressed rows gave the bits.
 //
 // The row's products are walked flattened, 32 per step whatever the lengths of
 // the B rows (an entry at a time left lanes idle and, for B rows of more than
@@ -538,7 +539,7 @@ cudaError_t launch_num_rank(const LaunchCtx& ctx, const BinSpec& bin, const CsrV
   }
   long long blocks = ((long long)nrows + rpc - 1) / rpc;
   if (blocks > (long long)ctx.num_sms * per_sm) blocks = (long long)ctx.num_sms * per_sm;
-  timer_begin(ctx.timer, ctx.stream, "num_window");
+  timer_begin(ctx.timer, ctx.stream, "num_rank");
   const RankArgs g{A, B, bcomp, ctx.row_lo, b_split, b_range_bad, c_rowptr, rows, nrows, c_colind, c_vals,
                    ctx.status, ctx.fingerprint};
   kern<<<(int)blocks, kRankThreads, smem, ctx.stream>>>(g, geo);

@@ -671,8 +671,8 @@ cudaError_t launch_spadd_symbolic(const LaunchCtx& ctx, const CsrView& A, const 
 
 cudaError_t launch_spadd_numeric(const LaunchCtx& ctx, const CsrView& A, const CsrView& B, double alpha,
                                  double beta, const int64_t* c_rowptr, const int32_t* apos,
-                                 const int32_t* bpos, const uint8_t* kind, const int32_t* long_rows, const int32_t* kinds,
-                                 int32_t* c_colind, double* c_vals) {
+                                 const int32_t* bpos, const uint8_t* kind, const int32_t* long_rows,
+                                 const int32_t* kinds, int32_t* c_colind, double* c_vals) {
   if (A.m <= 0) return cudaSuccess;
   if (kinds[0]) {
     const int T = add_team(A, B), grid = add_grid(ctx, A.m, kAddRowWarps * 32 / T);

@@ -1261,7 +1261,8 @@ cudaError_t launch_numeric_wide(const LaunchCtx& ctx, const CsrView& A, const Cs
   const size_t budget = wide_budget(ctx);
   WideGeom g = wide_geom(words, budget, true);
   const bool light = max_nnz <= g.vcap;  // every row of the bin fits: no more slots than it needs
-  if (light) g = wide_geom(words, g.val_off + (size_t)max_nnz * 8 < budget ? g.val_off + (size_t)max_nnz * 8 : budget, true);
+  const size_t need = light ? g.val_off + (size_t)max_nnz * 8 : budget;
+  if (light) g = wide_geom(words, need < budget ? need : budget, true);
   const int block = wide_block(ctx, g.bytes, light);
   if (block == 256) return num_wide<256>(ctx, A, B, words, g, c_rowptr, rows, nrows, c_colind, c_vals);
   if (block == 512) return num_wide<512>(ctx, A, B, words, g, c_rowptr, rows, nrows, c_colind, c_vals);
@@ -1270,18 +1271,19 @@ cudaError_t launch_numeric_wide(const LaunchCtx& ctx, const CsrView& A, const Cs
 
 cudaError_t launch_num_chunk(const LaunchCtx& ctx, const CsrView& A, const CsrView& B, const unsigned long long* fp,
                              const int64_t* c_rowptr, int32_t* c_colind, double* c_vals) {
-  cudaError_t e = cudaFuncSetAttribute(k_num_chunk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ChunkSmem));
+  const size_t smem = sizeof(ChunkSmem);
+  cudaError_t e = cudaFuncSetAttribute(k_num_chunk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(ctx.keep.next + 2, 0, sizeof(int32_t), ctx.stream);
   if (e != cudaSuccess) return e;
   timer_begin(ctx.timer, ctx.stream, "num_chunk");
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_num_chunk, kChunkThreads, sizeof(ChunkSmem)) != cudaSuccess ||
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_num_chunk, kChunkThreads, smem) != cudaSuccess ||
       per_sm < 1) {
     (void)cudaGetLastError();
     per_sm = 1;
   }
-  k_num_chunk<<<ctx.num_sms * per_sm, kChunkThreads, sizeof(ChunkSmem), ctx.stream>>>(
+  k_num_chunk<<<ctx.num_sms * per_sm, kChunkThreads, smem, ctx.stream>>>(
       A, B, wide_words(B.n), fp, c_rowptr, c_colind, c_vals, ctx.keep, ctx.status);
   timer_end(ctx.timer, ctx.stream);
   return cudaGetLastError();
