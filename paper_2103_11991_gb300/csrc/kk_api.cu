@@ -191,13 +191,13 @@ __device__ __forceinline__ uint8_t classify(const BinTable& t, long long q, int 
 // is processed; T and U follow A's mean row length.  STATS (the learned
 // form): also the longest and shortest referenced B row of each row, to stat.
 // Long rows are listed for a second launch (LISTED), as in k_analyze_b.
-// Rows of more than tab.pair_flop products of a sorted B are binned for the window
-// by the compressed pairs of their B rows (blen, null: not known) where these hold
-// kWindowDense columns or more each; a second walk over the row's entries of A adds
-// the pairs up.  The others are binned by their products.  The same walk tells which
-// rows of too wide a span for a window and more than tab.team_max products are
-// spread.
-template <int T, int U, bool STATS, bool LISTED>
+// PAIRS (the compressed B's lengths blen are known and the table has lines for them):
+// rows of more than tab.pair_flop products of a sorted B are binned for the window by
+// the compressed pairs of their B rows where these hold kWindowDense columns or more
+// each; a second walk over the row's entries of A, by the whole warp, adds the pairs
+// up.  The others are binned by their products.  The same walk tells which rows of too
+// wide a span for a window and more than tab.team_max products are spread.
+template <int T, int U, bool STATS, bool LISTED, bool PAIRS>
 __global__ void __launch_bounds__(256, 6)
 k_analyze_a(CsrView A, const int32_t* __restrict__ brp,
                             const int32_t* __restrict__ bcol, const int32_t* __restrict__ blen, int32_t nb_rows,
@@ -295,24 +295,29 @@ k_analyze_a(CsrView A, const int32_t* __restrict__ brp,
     if (bad) set_status(status, KK_ERR_BAD_INDEX);
     const long long span = hi >= lo ? (long long)hi - lo + 1 : 0;
     long long wq = f, team_max = (long long)9e18;
-    const bool heavy = f > tab.pair_flop;
-    const bool early = f > tab.team_max && f <= kSymTeamMaxFlop && span > window_bits(kNumWindowClasses - 1);
-    if (on && sorted && (heavy || early)) {  // (the same for all lanes of a team)
-      if (heavy && span <= kWindowFreeSpan) {
-        wq = 1;
-      } else if (blen) {
+    if constexpr (PAIRS) {
+      const bool heavy = on && sorted && f > tab.pair_flop;
+      const bool early = on && sorted && f > tab.team_max && f <= kSymTeamMaxFlop &&
+                         span > window_bits(kNumWindowClasses - 1);
+      const bool few = heavy && span <= kWindowFreeSpan;
+      if (few) wq = 1;
+      for (unsigned m = __ballot_sync(0xffffffffu, (early || (heavy && !few)) && tl == 0); m; m &= m - 1) {
+        const int src = __ffs(m) - 1, lane = threadIdx.x & 31;
+        const int a0 = __shfl_sync(0xffffffffu, pa, src), a1 = __shfl_sync(0xffffffffu, pe, src);
         long long pairs = 0;
-        for (int p0 = pa; p0 < pe; p0 += T * U) {
+        for (int p0 = a0; p0 < a1; p0 += 32 * U) {
           int j[U];
 #pragma unroll
-          for (int u = 0; u < U; ++u) j[u] = p0 + u * T + tl < pe ? A.colind[p0 + u * T + tl] : -1;
+          for (int u = 0; u < U; ++u) j[u] = p0 + u * 32 + lane < a1 ? A.colind[p0 + u * 32 + lane] : -1;
 #pragma unroll
           for (int u = 0; u < U; ++u) pairs += (unsigned)j[u] < (unsigned)nb_rows ? blen[j[u]] : 0;
         }
 #pragma unroll
-        for (int o = T / 2; o > 0; o >>= 1) pairs += __shfl_xor_sync(mask, pairs, o, T);
-        if (heavy && pairs * kWindowDense <= f) wq = pairs;
-        if (early && wide_spread_row(f, pairs)) team_max = tab.team_max;
+        for (int o = 16; o > 0; o >>= 1) pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
+        if (lane / T == src / T) {
+          if (heavy && pairs * kWindowDense <= f) wq = pairs;
+          if (early && wide_spread_row(f, pairs)) team_max = tab.team_max;
+        }
       }
     }
     if (on && tl == 0) {
@@ -1529,10 +1534,10 @@ static BinTable symbolic_table(kk_spgemm_handle h, int32_t cols) {
 // strides over rows).
 // bin receives the symbolic bin ids; with STATS, stat the learned form's row
 // statistics.
-template <int T, int U, bool STATS, bool LISTED>
+template <int T, int U, bool STATS, bool LISTED, bool PAIRS>
 static void launch_analyze_a_t(kk_spgemm_handle h, const CsrView& av, const CsrView& bv, Misc* dm,
-                               cudaStream_t s, uint8_t* bin, int2* stat, const LongRows& lr) {
-  auto kern = k_analyze_a<T, U, STATS, LISTED>;
+                               cudaStream_t s, uint8_t* bin, int2* stat, const LongRows& lr, const BinTable& tab) {
+  auto kern = k_analyze_a<T, U, STATS, LISTED, PAIRS>;
   static int per_sm = 0;
   if (per_sm == 0 && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, 0) != cudaSuccess) {
     (void)cudaGetLastError();
@@ -1540,8 +1545,7 @@ static void launch_analyze_a_t(kk_spgemm_handle h, const CsrView& av, const CsrV
   }
   const int64_t m = LISTED ? lr.most : av.m;
   kern<<<grid_for(m * T, 256, h->num_sms * (per_sm > 0 ? per_sm : 1)), 256, 0, s>>>(
-      av, bv.rowptr, bv.colind, h->opt.use_window ? h->d_bclen.as<int32_t>() : nullptr, bv.m, &dm->sorted,
-      symbolic_table(h, bv.n), h->opt.team_vec_min_len,
+      av, bv.rowptr, bv.colind, h->d_bclen.as<int32_t>(), bv.m, &dm->sorted, tab, h->opt.team_vec_min_len,
       h->d_flop.as<long long>(), bin, h->d_rowlo.as<int32_t>(), h->d_span.as<int32_t>(), stat,
       &dm->total_flop, &dm->status, lr);
 }
@@ -1549,12 +1553,22 @@ static void launch_analyze_a_t(kk_spgemm_handle h, const CsrView& av, const CsrV
 // Teams by A's mean row length: the smallest whose U = 8 gathers per lane cover
 // a typical row in one round (more rows in flight per SM; measured against teams
 // of 4 and 8), then the listed long rows.
+template <bool STATS, bool PAIRS>
+static void launch_analyze_a_p(kk_spgemm_handle h, const CsrView& av, const CsrView& bv, Misc* dm, cudaStream_t s,
+                               uint8_t* bin, int2* stat, const LongRows& lr, const BinTable& tab) {
+  if ((long long)av.nnz / av.m <= 8)
+    launch_analyze_a_t<1, 8, STATS, false, PAIRS>(h, av, bv, dm, s, bin, stat, lr, tab);
+  else launch_analyze_a_t<4, 8, STATS, false, PAIRS>(h, av, bv, dm, s, bin, stat, lr, tab);
+  if (lr.rows) launch_analyze_a_t<32, 8, STATS, true, PAIRS>(h, av, bv, dm, s, bin, stat, lr, tab);
+}
 template <bool STATS = false>
 static void launch_analyze_a(kk_spgemm_handle h, const CsrView& av, const CsrView& bv, Misc* dm,
                              cudaStream_t s, uint8_t* bin, const LongRows& lr, int2* stat = nullptr) {
-  if ((long long)av.nnz / av.m <= 8) launch_analyze_a_t<1, 8, STATS, false>(h, av, bv, dm, s, bin, stat, lr);
-  else launch_analyze_a_t<4, 8, STATS, false>(h, av, bv, dm, s, bin, stat, lr);
-  if (lr.rows) launch_analyze_a_t<32, 8, STATS, true>(h, av, bv, dm, s, bin, stat, lr);
+  const BinTable tab = symbolic_table(h, bv.n);
+  const long long none = (long long)9e18;
+  if (h->opt.use_window && bv.m > 0 && (tab.pair_flop < none || tab.team_max < none))
+    launch_analyze_a_p<STATS, true>(h, av, bv, dm, s, bin, stat, lr, tab);
+  else launch_analyze_a_p<STATS, false>(h, av, bv, dm, s, bin, stat, lr, tab);
 }
 
 extern "C" {
