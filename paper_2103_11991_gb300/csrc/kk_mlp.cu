@@ -143,8 +143,8 @@ constexpr int kMlpBlock = 128;
 // 4,096 samples but was 1.8 times further from the float64 gradient than a warp sum
 // per weight (relative error at 4,096 and 20,001 samples, mean of 12 seeds: warp sums
 // 9.5e-8 and 2.0e-7, the chain 1.7e-7 and 3.4e-7, this 8.0e-8 and 1.4e-7).
-// What bounds it: issue and shared-memory reads; a tile is about 1,000
-// instructions a warp.  A thread per sample with a warp sum per weight (1,872 of
+// What bounds it: latency; the 8 warps of a CTA execute 1,640 instructions each for a
+// tile and its share of the sums, with a barrier after each layer.  A thread per sample with a warp sum per weight (1,872 of
 // five shuffles, then atomics) took 252 us for 4,096 samples; this takes 14.8.
 constexpr int kGradThreads = 256;
 constexpr int kGradLd = 36;

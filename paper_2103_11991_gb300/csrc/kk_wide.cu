@@ -904,9 +904,9 @@ k_num_wide(CsrView A, CsrView B, int32_t words, int32_t vcap, uint32_t sum_off, 
 // the piece's bounds without a search (k_index_fill).  The pieces' products are
 // walked flattened, a run of consecutive ones per warp, and added with a
 // compare-and-swap loop around one fma (in no fixed order).
-// What bounds it: the shared-memory data path (78% busy, 35 wavefronts per 32
-// products) and the float64 pipe, on which an instruction costs a warp the same
-// with one lane as with 32.  atomicAdd(double) needs a product and an addition
+// What bounds it: the shared-memory data path (79% busy on scale 15, 33 to 36
+// wavefronts per 32 products) and the float64 pipe, on which an instruction costs a
+// warp the same with one lane as with 32.  atomicAdd(double) needs a product and an addition
 // per try where this loop needs one fma: 22.6 -> 21.0 ms for the 2.85e9 products
 // of the scale-18 R-MAT square.  The kernel that this one replaces there (a CTA
 // of 1,024 threads per row and SM, atomics in shared memory or in C, the bits
