@@ -922,6 +922,8 @@ struct kk_spgemm_handle_s {
   DevBuf d_cw;         // uint16[m * kCacheWords]
   DevBuf d_cm;         // uint32[m * kCacheWords]
   DevBuf d_cn;         // int32[m]
+  bool cache_counts = false;  // d_cn is that of the last symbolic call
+  DevBuf d_rw, d_rm, d_rn;  // the same, derived again by a numeric call (d_rn: and the rows' counts)
   bool cache_valid = false;
   bool fp_taken = false;  // the symbolic call's fingerprint is in d_misc
   // wide-tier bit vectors kept by the symbolic phase
@@ -957,12 +959,13 @@ struct Misc {
   unsigned long long tier_a[4];  // numeric tiers: A entries of their rows
   unsigned long long tier_f[4];  // numeric tiers: multiply-adds of their rows
   unsigned long long kept;       // window rows whose structure was kept
+  unsigned long long not_kept;   // ... whose word counts alone were
   unsigned long long bc_pairs;   // pairs of the compressed B
   unsigned long long fp[2];      // structure fingerprints: symbolic call, numeric call
   int32_t small_flags[4];        // small-product path: row beyond it, bad index, CTA ticket
   int32_t wide_kept;             // rows kept with chunk tasks
   int32_t long_a, long_b;        // long rows listed by the analyses
-  int32_t pad2;
+  int32_t again_status;          // of structure derived again by a numeric call (not looked at)
 };
 static_assert(sizeof(Misc) <= 256, "the staging buffer's bin starts follow at byte 256");
 
@@ -1246,14 +1249,23 @@ kk_status symbolic_fingerprint(kk_spgemm_handle h, const CsrView& av, const CsrV
 }
 
 // Structure cache for the symbolic window kernel: every row starts without
-// kept structure (n = -1); null pointers when the option is off or no row of
-// the call takes the window tier.  The index arrays' fingerprint is recorded
-// with it.
+// kept structure (n = -1); null pointers when no row of the call takes the window
+// tier.  The index arrays' fingerprint is recorded with it.  With the option off
+// only the word counts are kept: they tell which rows a numeric call can derive the
+// structure of (rebuild_view).
 kk_status cache_for_symbolic(kk_spgemm_handle h, int32_t m, bool any_window, const CsrView& av,
                              const CsrView& bv, WinCache* out) {
   *out = WinCache{nullptr, nullptr, nullptr, nullptr};
   h->cache_valid = false;
-  if (!h->opt.structure_cache || !any_window || m <= 0) return KK_OK;
+  h->cache_counts = false;
+  if (!any_window || m <= 0) return KK_OK;
+  if (!h->opt.structure_cache) {
+    KK_CUDA(h, h->d_cn.ensure(sizeof(int32_t) * (size_t)m), "alloc structure cache");
+    KK_CUDA(h, cudaMemsetAsync(h->d_cn.p, 0xFF, sizeof(int32_t) * (size_t)m, h->stream), "memset cache");
+    *out = WinCache{nullptr, nullptr, h->d_cn.as<int32_t>(), &h->d_misc.as<Misc>()->not_kept};
+    h->cache_counts = true;
+    return KK_OK;
+  }
   KK_CUDA(h, h->d_cw.ensure(sizeof(uint16_t) * (size_t)m * kCacheWords), "alloc structure cache");
   KK_CUDA(h, h->d_cm.ensure(sizeof(uint32_t) * (size_t)m * kCacheWords), "alloc structure cache");
   KK_CUDA(h, h->d_cn.ensure(sizeof(int32_t) * (size_t)m), "alloc structure cache");
@@ -1262,6 +1274,7 @@ kk_status cache_for_symbolic(kk_spgemm_handle h, int32_t m, bool any_window, con
                   &h->d_misc.as<Misc>()->kept};
   KK_TRY(symbolic_fingerprint(h, av, bv));
   h->cache_valid = true;
+  h->cache_counts = true;
   h->cache_key[0] = av.rowptr;
   h->cache_key[1] = av.colind;
   h->cache_key[2] = bv.rowptr;
@@ -1374,7 +1387,7 @@ void keep_for_numeric(kk_spgemm_handle h, const CsrView& av, const CsrView& bv) 
 
 // Kept word counts of the rows of this symbolic call (-1: no kept structure),
 // null when it keeps none.
-const int32_t* kept_counts(kk_spgemm_handle h) { return h->cache_valid ? h->d_cn.as<int32_t>() : nullptr; }
+const int32_t* kept_counts(kk_spgemm_handle h) { return h->cache_counts ? h->d_cn.as<int32_t>() : nullptr; }
 
 // Slots of the rows of this symbolic call kept with chunk tasks (-1: none).
 const int32_t* kept_slots(kk_spgemm_handle h) { return h->keep.tasks ? h->keep.slot : nullptr; }
@@ -1394,6 +1407,52 @@ kk_status cache_view(kk_spgemm_handle h, const CsrView& av, const CsrView& bv, W
     if (st != KK_OK) return st;
     ctx->fingerprint = dm->fp;
   }
+  return KK_OK;
+}
+
+// The structure of the rows binned for it (start: the bins' row starts), derived again
+// by the symbolic window kernel, when none is kept for these arrays: other arrays than
+// the symbolic call's, or options.structure_cache = 0.  Their values then go by the kept
+// rows' kernel, which checks every product.  The rank kernel is slower on such rows,
+// whose products meet in few columns (structure_cache = 0, numeric phase: 125,000
+// 27-point rows 812 us by rank, 384 so, 24,300 rows of 81 x 81 blocks 1,412 and 540), and
+// takes them without the memory, or under a stream capture that would have to allocate
+// it.
+kk_status rebuild_view(kk_spgemm_handle h, const LaunchCtx& ctx, const CsrView& av, const CsrView& bv,
+                       const BComp& bcomp, const std::vector<int32_t>& start, const int32_t* rows, WinCacheView* view) {
+  if (view->n || !bcomp.bc) return KK_OK;
+  bool any = false;
+  for (size_t b = 0; b < h->num_bins.size(); ++b)
+    if (h->num_bins[b].tier == kTierWindow && start[b + 1] > start[b]) any = true;
+  if (!any) return KK_OK;
+  const size_t m = (size_t)av.m, words = m * kCacheWords;
+  const bool have = h->d_rw.bytes >= words * 2 && h->d_rm.bytes >= words * 4 && h->d_rn.bytes >= m * 8;
+  if (!have) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    KK_CUDA(h, cudaStreamIsCapturing(h->stream, &capture), "capture status");
+    if (capture != cudaStreamCaptureStatusNone) return KK_OK;
+    if (h->d_rw.ensure(words * 2) != cudaSuccess || h->d_rm.ensure(words * 4) != cudaSuccess ||
+        h->d_rn.ensure(m * 8) != cudaSuccess) {
+      (void)cudaGetLastError();
+      for (DevBuf* b : {&h->d_rw, &h->d_rm, &h->d_rn}) b->release();
+      return KK_OK;
+    }
+  }
+  // (a word outside a row's window belongs to another structure: its products are
+  // missing from the row's and reported by the kept rows' kernel)
+  LaunchCtx again = ctx;
+  again.status = &h->d_misc.as<Misc>()->again_status;
+  const WinCache out{h->d_rw.as<uint16_t>(), h->d_rm.as<uint32_t>(), h->d_rn.as<int32_t>(),
+                     &h->d_misc.as<Misc>()->not_kept};
+  for (size_t b = 0; b < h->num_bins.size(); ++b) {
+    const int32_t cnt = start[b + 1] - start[b];
+    if (h->num_bins[b].tier != kTierWindow || cnt <= 0) continue;
+    KK_CUDA(h, launch_symbolic_window(again, h->num_bins[b], av, bv, bcomp, rows + start[b], cnt,
+                                      h->d_rn.as<int32_t>() + m, out),
+            "window launch");
+    h->stats[9] += 1;
+  }
+  *view = WinCacheView{out.w, out.m, out.n};
   return KK_OK;
 }
 
@@ -1737,6 +1796,7 @@ kk_status kk_spgemm_symbolic(kk_spgemm_handle h, const kk_csr* A, const kk_csr* 
       h->stats[30] = m;
       h->small = true;
       h->cache_valid = false;
+      h->cache_counts = false;
       h->keep = WideKeep{};
       h->keep_valid = false;
       h->learned_valid = false;
@@ -1947,6 +2007,7 @@ static kk_status numeric_impl(kk_spgemm_handle h, const kk_csr* A, const kk_csr*
   }
   WinCacheView wview;
   if ((st = cache_view(h, av, bv, &wview, &ctx)) != KK_OK) return st;
+  KK_TRY(rebuild_view(h, ctx, av, bv, bcomp, h->num_start, h->d_nrows.as<int32_t>(), &wview));
   bool skip_wide = false;
   if (jac && ctx.keep.tasks && h->wide_kept > 0) {
     // the kept rows' scales come before their chunks
@@ -2251,6 +2312,7 @@ kk_status kk_spgemm_learned_symbolic(kk_spgemm_handle h, const kk_csr* A, const 
     if ((st = ensure_bcomp(h, bv, &bcomp, &bc_built)) != KK_OK) return st;
   }
   h->cache_valid = false;
+  h->cache_counts = false;
   if (m > 0) {
     KK_CUDA(h, cudaMemsetAsync(h->d_cnt.p, 0, sizeof(int32_t) * (size_t)m, s), "memset counts");
     for (int c = 0; c < kLearnedHeavy; ++c) {
@@ -2379,6 +2441,7 @@ kk_status kk_spgemm_learned_numeric(kk_spgemm_handle h, const kk_csr* A, const k
   }
   WinCacheView wview;
   if ((st = cache_view(h, av, bv, &wview, &ctx)) != KK_OK) return st;
+  KK_TRY(rebuild_view(h, ctx, av, bv, bcomp, h->lnum_start, h->d_lrows2.as<int32_t>(), &wview));
   bool skip_wide = false;
   if ((st = launch_kept_chunks(h, ctx, av, bv, h->lnum_start, c_rowptr, c_colind, c_vals, &skip_wide)) != KK_OK)
     return st;
@@ -2839,7 +2902,8 @@ kk_status kk_spgemm_destroy(kk_spgemm_handle h) {
                     &h->d_sval, &h->d_sball, &h->d_nbin2, &h->d_lrows, &h->d_lrows2, &h->d_mm,
                     &h->d_bdesc, &h->d_rowpair, &h->d_bflop, &h->d_bsbin, &h->d_bnbin, &h->d_bsrows,
                     &h->d_bnrows, &h->d_bcnt, &h->d_btiles, &h->d_bstart, &h->d_bqueue, &h->d_bsplit2,
-                    &h->d_boff, &h->d_bc, &h->d_bclen, &h->d_cw, &h->d_cm, &h->d_cn, &h->d_wbits,
+                    &h->d_boff, &h->d_bc, &h->d_bclen, &h->d_cw, &h->d_cm, &h->d_cn, &h->d_rw, &h->d_rm, &h->d_rn,
+                    &h->d_wbits,
                     &h->d_wslot, &h->d_wnext, &h->d_wtasks, &h->d_widx, &h->d_wtab, &h->d_along_rows, &h->d_blong,
                     &h->d_pa_rp, &h->d_pa_ci, &h->d_pa_v, &h->d_pb_rp, &h->d_pb_ci, &h->d_pb_v, &h->d_pbase,
                     &h->d_jvals, &h->d_jpos, &h->d_apos, &h->d_bpos, &h->d_acnt, &h->d_akind, &h->d_along})
