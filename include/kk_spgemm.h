@@ -107,7 +107,9 @@ typedef struct {
   int32_t structure_cache;    /* 1: the symbolic phase keeps the structure of every window row
                                  (its non-empty 32-column words, at most 64 per row, 6 bytes
                                  each) so that the numeric phase of the same A and B arrays
-                                 writes C's columns without re-deriving them (default 1) */
+                                 writes C's columns without re-deriving them (default 1).  With 0,
+                                 or for other arrays, the numeric phase derives it again, into as
+                                 much scratch, or does without where there is none */
   int32_t wide_cache_mb;      /* budget for what the wide tier keeps of its rows from the symbolic
                                  phase: their k-bit column vectors and, for a sorted B of at most
                                  2^19 columns, tables of column chunks, the chunks' tasks and an
